@@ -11,28 +11,14 @@
 #include <numeric>
 #include <vector>
 
-#include <atomic>
-
-#include "host.hpp"
-#include "march_bwd.cuh"
+#include "batch.hpp"
 #include "march_bwd_tile.cuh"
 
 using namespace dfs;
 
 namespace {
 
-constexpr uint32_t kPlanMagic = 0x44465350u;   // "DFSP"
-
-struct PlanPose {
-    int32_t n_rays, S;
-    double fov, depth;
-    float a2;
-    int32_t W;
-    int64_t img_off;
-    double a2d;
-    float l2_hi, l2_lo;      // log2(a^2) split (depth-gain reading)
-    int32_t pad;
-};
+constexpr uint32_t kPlanMagic = 0x44465351u;   // "DFSQ": plans with internal row offsets
 
 struct BlurTile {                 // one 32-row strip of one pose image
     int32_t pose, n_rays, k0, pad;
@@ -41,12 +27,12 @@ struct BlurTile {                 // one 32-row strip of one pose image
 struct PlanHeader {
     uint32_t magic;
     int32_t P;
-    int64_t total_rays, total_img, total_gz, total_ckpt, n_tiles, n_ftiles, total_bcar, n_spk;
+    int64_t total_rays, total_img, total_gz, total_ckpt, n_tiles, n_ftiles, total_bcar, n_spk, total_pad;
     double max_depth;
     int32_t max_S, blurW;
     int32_t warps, ctas_per_sm, gather_ctas, fwd_form;
     int64_t off_pose, off_depth, off_ray0, off_ray_pose, off_ray_j, off_order, off_row_off, off_gz_off, off_ck_off,
-        off_tiles, off_ftiles, off_spk;
+        off_tiles, off_ftiles, off_spk, off_pad_off;
     int64_t bytes;
     uint64_t params_fp;   // fingerprint of the parameters the plan was made for
     // backward chunks: chunk c covers poses chunk_pose[c] .. chunk_pose[c+1]-1,
@@ -78,7 +64,7 @@ uint64_t params_fingerprint(const diffus_params *p)
 }
 
 struct PlanSizes {
-    int64_t off[12];
+    int64_t off[13];
     int64_t bytes;
 };
 
@@ -102,6 +88,7 @@ PlanSizes plan_sizes(int P, int64_t total_rays, int64_t n_tiles, int64_t n_ftile
     put(9, sizeof(BlurTile) * n_tiles);
     put(10, sizeof(TileDesc) * n_ftiles);
     put(11, sizeof(SpkItem) * n_spk);
+    put(12, sizeof(int64_t) * total_rays);
     z.bytes = o;
     return z;
 }
@@ -144,7 +131,7 @@ struct BatchLayout {
     RefineSel sel;   // selective refinement (refine = 1)
     float *gy;       // blur transpose of grad_images (blur on)
     float *mbuf;     // speckle factors of every row, kept by the forward for the adjoint (speckle on)
-    float2 *kbuf;    // (impedance, r of the interface before) of every sample, kept by the forward for the adjoint
+    float2 *kbuf;    // impedance and r of the interface before of every sample, kept by the forward for the adjoint
     float *gz;
     double *part;
     float4 *ckpt;
@@ -161,10 +148,10 @@ BatchLayout batch_layout(void *ws, const PlanHeader &H, const diffus_volume_desc
     L.geo = c.take<RayGeo>((size_t)H.total_rays);
     L.frames = c.take<PoseFrame>((size_t)H.P);
     L.counter = c.take<unsigned>(kCounters);
-    L.y = blur ? c.take<float>((size_t)H.total_img) : nullptr;
+    L.y = blur ? c.take<float>((size_t)H.total_pad) : nullptr;
     // the one-warp-per-ray forward reads speckle factors drawn ahead of it
     const bool spk_ahead = speckle && H.fwd_form == 0;
-    L.mbuf = spk_ahead ? c.take<float>((size_t)H.total_img) : nullptr;
+    L.mbuf = spk_ahead ? c.take<float>((size_t)H.total_pad) : nullptr;
     L.sel = RefineSel{nullptr, nullptr, nullptr, nullptr};
     if (refine) {
         L.sel.rinfo = c.take<int2>((size_t)H.total_rays);
@@ -175,8 +162,8 @@ BatchLayout batch_layout(void *ws, const PlanHeader &H, const diffus_volume_desc
         }
     }
     L.fwd_bytes = c.used;
-    L.gy = (blur || atten) ? c.take<float>((size_t)H.total_img) : nullptr;
-    if (!spk_ahead) L.mbuf = speckle ? c.take<float>((size_t)H.total_img) : nullptr;
+    L.gy = (blur || atten) ? c.take<float>((size_t)H.total_pad) : nullptr;
+    if (!spk_ahead) L.mbuf = speckle ? c.take<float>((size_t)H.total_pad) : nullptr;
     L.kbuf = c.take<float2>((size_t)H.total_gz);
     L.gz = c.take<float>((size_t)H.total_gz);
     L.part = c.take<double>(6 * (size_t)H.total_rays);
@@ -188,21 +175,6 @@ BatchLayout batch_layout(void *ws, const PlanHeader &H, const diffus_volume_desc
 }
 
 // ------------------------------------------------------------------ kernels
-
-// What the forward keeps for the adjoint of the same call (each nullable).
-struct FwdKeep {
-    float4 *ckpt;
-    float *mbuf;
-    float2 *kbuf;
-    float4 *bcar;
-};
-
-struct BatchDev {
-    const PlanPose *pose;
-    const int32_t *ray_pose, *ray_j, *order;
-    const int64_t *row_off, *gz_off, *ck_off;
-    int64_t total_rays;
-};
 
 __global__ void k_batch_setup(const PoseFrame *__restrict__ frames, BatchDev B, VolPlace vp, RayGeo *__restrict__ geo)
 {
@@ -216,70 +188,6 @@ __global__ void k_batch_setup(const PoseFrame *__restrict__ frames, BatchDev B, 
     geo[r] = rg;
 }
 
-// Persistent forward: each warp takes rays from the queue (longest first).
-// With refinement on (sel.rinfo set) it is the FP32 pass, which lists the
-// rays that need the refined pass.
-template <typename T, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, kFwdThreadsPerSM / (WARPS * 32)) k_batch_fwd(const T *__restrict__ vol, MarchArgs A, BatchDev B,
-                                                          const RayGeo *__restrict__ geo, float *__restrict__ out,
-                                                          int *__restrict__ valid, uint32_t *__restrict__ status,
-                                                          unsigned *__restrict__ counter, float4 *__restrict__ ckpt,
-                                                          float *__restrict__ mbuf, float2 *__restrict__ kbuf,
-                                                          const float *__restrict__ spk_in, RefineSel sel, int64_t q0,
-                                                          int64_t qn)
-{
-    __shared__ float buf[WARPS][kSegPad];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned q = 0;
-        if (lane == 0) q = atomicAdd(counter, 1u);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if ((int64_t)q >= qn) break;   // entries q0 .. q0+qn-1 of the ray order
-        const int r = B.order[q0 + q];
-        RayGeo rg = geo[r];
-        MarchArgs Ap = A;
-        if (!A.atten) {   // the depth-gain reading keeps a2 = 1 (lossless systems)
-            Ap.a2 = B.pose[rg.pose].a2;
-            Ap.a2d = B.pose[rg.pose].a2d;
-        }
-        // with the speckle drawn ahead (spk_in) the march reads the factors
-        // instead of writing them
-        RayOut o{out + B.row_off[r], valid ? valid + r : nullptr, status, ckpt ? ckpt + B.ck_off[r] : nullptr,
-                 (mbuf && !spk_in) ? mbuf + B.row_off[r] : nullptr, kbuf ? kbuf + B.gz_off[r] : nullptr,
-                 spk_in ? spk_in + B.row_off[r] : nullptr, sel.rinfo ? sel.rinfo + r : nullptr, sel.rlist,
-                 sel.rcount, r};
-        march_fwd_ray<T, false, true>(vol, Ap, rg, o, buf[w]);
-        __syncwarp();
-    }
-}
-
-// Persistent forward with one lane per ray: each warp takes tiles of 32
-// consecutive rays of a pose from the queue (longest first).
-template <typename T>
-__global__ void __launch_bounds__(kTileWarps * 32, kFwdThreadsPerSM / (kTileWarps * 32)) k_batch_fwd_tiles(const T *__restrict__ vol, MarchArgs A, BatchDev B,
-                                                          const RayGeo *__restrict__ geo,
-                                                          const TileDesc *__restrict__ tiles, int64_t n_tiles,
-                                                          float *__restrict__ out, int *__restrict__ valid,
-                                                          uint32_t *__restrict__ status,
-                                                          unsigned *__restrict__ counter, float4 *__restrict__ ckpt,
-                                                          float *__restrict__ mbuf, float2 *__restrict__ kbuf,
-                                                          float4 *__restrict__ bcar, RefineSel sel)
-{
-    __shared__ TileSmem sm[kTileWarps];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned q = 0;
-        if (lane == 0) q = atomicAdd(counter, 1u);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if ((int64_t)q >= n_tiles) break;
-        const TileDesc tl = tiles[q];
-        MarchArgs Ap = A;
-        if (!A.atten) Ap.a2 = B.pose[tl.pose].a2;   // the depth-gain reading keeps a2 = 1
-        march_fwd_tile<T>(vol, Ap, tl, geo, out, valid, status, ckpt, mbuf, kbuf, bcar, sel, sm[w]);
-        __syncwarp();
-    }
-}
-
 // Persistent backward of the lane-per-ray forward (volume gradient asked):
 // tiles from the queue, longest first.
 __global__ void __launch_bounds__(kTileWarpsBwd * 32, kBwdValThreadsPerSM / (kTileWarpsBwd * 32)) k_batch_bwd_tiles(MarchArgs A, BatchDev B,
@@ -287,7 +195,7 @@ __global__ void __launch_bounds__(kTileWarpsBwd * 32, kBwdValThreadsPerSM / (kTi
                                                           const float *__restrict__ gy, const float *__restrict__ mbuf,
                                                           const float2 *__restrict__ kbuf,
                                                           const float4 *__restrict__ bcar, float *__restrict__ gz,
-                                                          unsigned *__restrict__ counter)
+                                                          unsigned *__restrict__ counter, bool gy_padded)
 {
     __shared__ BwdTileSmem sm[kTileWarpsBwd];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -299,7 +207,7 @@ __global__ void __launch_bounds__(kTileWarpsBwd * 32, kBwdValThreadsPerSM / (kTi
         const TileDesc tl = tiles[q];
         MarchArgs Ap = A;
         if (!A.atten) Ap.a2 = B.pose[tl.pose].a2;
-        march_bwd_tile(Ap, tl, gy, mbuf, kbuf, bcar, gz, sm[w]);
+        march_bwd_tile(Ap, tl, gy, mbuf, kbuf, bcar, gz, gy_padded, sm[w]);
         __syncwarp();
     }
 }
@@ -319,85 +227,19 @@ __global__ void __launch_bounds__(kTileWarps * 32) k_batch_speckle(Speckle sp, c
     }
 }
 
-// Refined pass of the batch over the rays the FP32 pass listed (in the order
-// it listed them, which follows its longest-first queue).
-template <typename T, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, kRefineWarpsPerSM / WARPS) k_batch_refine(const T *__restrict__ vol, MarchArgs A, BatchDev B,
-                                                                const RayGeo *__restrict__ geo,
-                                                                const PoseFrame *__restrict__ frames, VolPlace vp,
-                                                                float *__restrict__ out, int *__restrict__ valid,
-                                                                uint32_t *__restrict__ status,
-                                                                float4 *__restrict__ ckpt, RefineSel sel)
-{
-    __shared__ float buf[WARPS][kSegPad];
-    __shared__ float2 dbuf[WARPS][kSegPad];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned n = *sel.rcount;
-    for (;;) {
-        unsigned q = 0;
-        if (lane == 0) q = atomicAdd(sel.ticket, 1u);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if (q >= n) break;
-        const int r = sel.rlist[q];
-        const RayGeo rg = geo[r];
-        const PlanPose pp = B.pose[rg.pose];
-        MarchArgs Ap = A;
-        if (!A.atten) {
-            Ap.a2 = pp.a2;
-            Ap.a2d = pp.a2d;
-        }
-        const FanDev fd{pp.n_rays, pp.S, pp.fov, pp.depth};
-        RayOut o{out + B.row_off[r], valid ? valid + r : nullptr, status, ckpt ? ckpt + B.ck_off[r] : nullptr,
-                 nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, r};
-        refine_ray<T, true>(vol, Ap, rg, frames[rg.pose], fd, vp, o, sel.rinfo[r], buf[w], dbuf[w]);
-        __syncwarp();
-    }
-}
-
-template <typename T, int WARPS, bool POSE>
-__global__ void __launch_bounds__(WARPS * 32, (POSE ? kBwdThreadsPerSM : kBwdValThreadsPerSM) / (WARPS * 32)) k_batch_bwd(const T *__restrict__ vol, MarchArgs A, BatchDev B,
-                                                          const RayGeo *__restrict__ geo,
-                                                          const float *__restrict__ gy, float *__restrict__ gz,
-                                                          double *__restrict__ part, float4 *__restrict__ ckpt,
-                                                          unsigned *__restrict__ counter,
-                                                          const float *__restrict__ mbuf,
-                                                          const float2 *__restrict__ kbuf, int64_t q0, int64_t qn)
-{
-    // WARPS slots of BwdSmem, in dynamic shared memory (above the 48 KB of
-    // static arrays with 8 warps)
-    extern __shared__ __align__(16) unsigned char bwd_smem[];
-    BwdSmem<POSE> *sm = reinterpret_cast<BwdSmem<POSE> *>(bwd_smem);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned q = 0;
-        if (lane == 0) q = atomicAdd(counter, 1u);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if ((int64_t)q >= qn) break;   // entries q0 .. q0+qn-1 of the ray order
-        const int r = B.order[q0 + q];
-        RayGeo rg = geo[r];
-        MarchArgs Ap = A;
-        if (!A.atten) {   // the depth-gain reading keeps a2 = 1 (lossless systems)
-            Ap.a2 = B.pose[rg.pose].a2;
-            Ap.a2d = B.pose[rg.pose].a2d;
-        }
-        // the value-only march reads the samples the forward kept
-        march_bwd_ray<T, POSE, !POSE>(vol, Ap, rg, gy + B.row_off[r], gz + B.gz_off[r], part + 6 * (size_t)r,
-                                      ckpt + B.ck_off[r], sm[w], true, mbuf ? mbuf + B.row_off[r] : nullptr,
-                                      kbuf + B.gz_off[r]);
-        __syncwarp();
-    }
-}
-
 // Depth-gain row pass over all rays of the batch (one warp per ray):
-// out[row + k] = in[row + k] gain_p(k) (in and out may alias).
-__global__ void k_batch_row_gain(const float *in, float *out, BatchDev B)
+// out row k = in row k gain_p(k), rows at in_off and out_off (in and out may
+// alias).
+__global__ void k_batch_row_gain(const float *in, const int64_t *__restrict__ in_off, float *out,
+                                 const int64_t *__restrict__ out_off, BatchDev B)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < B.total_rays; r += nw) {
         const PlanPose pp = B.pose[B.ray_pose[r]];
-        const int64_t off = B.row_off[r];
-        for (int k = lane; k < pp.S; k += 32) out[off + k] = in[off + k] * depth_gain(pp.l2_hi, pp.l2_lo, k);
+        const float *src = in + in_off[r];
+        float *dst = out + out_off[r];
+        for (int k = lane; k < pp.S; k += 32) dst[k] = src[k] * depth_gain(pp.l2_hi, pp.l2_lo, k);
     }
 }
 
@@ -418,8 +260,10 @@ __global__ void __launch_bounds__(kBlurWarps * 32) k_batch_blur(const float *__r
         if ((int64_t)q >= n_tiles) break;
         const BlurTile tl = tiles[q];
         const PlanPose pp = poses[tl.pose];
-        blur_strip<TRANSPOSE, WT>(in + pp.img_off, out + pp.img_off, pp.n_rays, pp.S, b, tl.k0, 0, pp.n_rays,
-                                  pp.l2_hi, pp.l2_lo);
+        // the march's side of the blur is internal rows, the caller's packed
+        const int64_t io = TRANSPOSE ? pp.img_off : pp.pad_off, oo = TRANSPOSE ? pp.pad_off : pp.img_off;
+        blur_strip<TRANSPOSE, WT>(in + io, out + oo, pp.n_rays, pp.S, TRANSPOSE ? pp.S : pp.ld,
+                                  TRANSPOSE ? pp.ld : pp.S, b, tl.k0, 0, pp.n_rays, pp.l2_hi, pp.l2_lo);
     }
 }
 
@@ -440,108 +284,6 @@ void launch_batch_blur(const float *in, float *out, const PlanPose *poses, const
     }
 }
 
-
-int sm_count()
-{
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
-}
-
-// The forward's launch: fwd_form 0 one warp per ray, 1 tiles with one lane
-// per ray (grid = CTAs per SM x SMs of kTileWarps warps).
-struct FwdLaunch {
-    int grid, form;
-    const TileDesc *tiles;
-    int64_t n_tiles;
-    const float *spk_in;   // speckle factors drawn ahead (one warp per ray only), or null
-};
-
-template <typename T, int WARPS>
-void launch_fwd_t(const void *vol, const MarchArgs &A, const BatchDev &B, const RayGeo *geo, float *out, int *valid,
-                  uint32_t *status, unsigned *counter, const FwdKeep &kp, const FwdLaunch &fl, const RefineSel &sel,
-                  const PoseFrame *frames, const VolPlace &vp, int64_t q0, int64_t qn, cudaStream_t s)
-{
-    if (fl.form == 1)
-        k_batch_fwd_tiles<T><<<fl.grid, kTileWarps * 32, 0, s>>>((const T *)vol, A, B, geo, fl.tiles, fl.n_tiles,
-                                                                 out, valid, status, counter, kp.ckpt, kp.mbuf,
-                                                                 kp.kbuf, kp.bcar, sel);
-    else
-        k_batch_fwd<T, WARPS><<<fl.grid, WARPS * 32, 0, s>>>((const T *)vol, A, B, geo, out, valid, status, counter,
-                                                             kp.ckpt, kp.mbuf, kp.kbuf, fl.spk_in, sel, q0, qn);
-    if (sel.rinfo)
-        k_batch_refine<T, WARPS><<<kRefineWarpsPerSM / WARPS * sm_count(), WARPS * 32, 0, s>>>((const T *)vol, A, B, geo, frames, vp, out, valid,
-                                                                  status, kp.ckpt, sel);
-}
-
-// Opt the batched adjoint in to its dynamic shared memory, once per kernel
-// and device (the attribute is not a stream operation, so this is safe
-// inside a capture).  Returns nonzero on failure.
-template <typename T, int WARPS, bool POSE>
-int bwd_smem_optin(size_t bytes)
-{
-    static std::atomic<unsigned long long> done{0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (done.load(std::memory_order_acquire) & bit) return 0;
-    if (cudaFuncSetAttribute(k_batch_bwd<T, WARPS, POSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-        cudaSuccess)
-        return 1;
-    done.fetch_or(bit, std::memory_order_acq_rel);
-    return 0;
-}
-
-template <typename T, int WARPS>
-int launch_bwd_t(const void *vol, const MarchArgs &A, const BatchDev &B, const RayGeo *geo, const float *gy,
-                  float *gz, double *part, float4 *ckpt, unsigned *counter, const float *mbuf, const float2 *kbuf,
-                  int grid, bool pose, int64_t q0, int64_t qn, cudaStream_t s)
-{
-    if (pose) {
-        const size_t sb = WARPS * sizeof(BwdSmem<true>);
-        if (bwd_smem_optin<T, WARPS, true>(sb)) return DIFFUS_E_LAUNCH;
-        k_batch_bwd<T, WARPS, true><<<grid, WARPS * 32, sb, s>>>((const T *)vol, A, B, geo, gy, gz, part, ckpt,
-                                                                 counter, mbuf, kbuf, q0, qn);
-    } else {
-        const size_t sb = WARPS * sizeof(BwdSmem<false>);
-        if (bwd_smem_optin<T, WARPS, false>(sb)) return DIFFUS_E_LAUNCH;
-        k_batch_bwd<T, WARPS, false><<<grid, WARPS * 32, sb, s>>>((const T *)vol, A, B, geo, gy, gz, part, ckpt,
-                                                                  counter, mbuf, kbuf, q0, qn);
-    }
-    return DIFFUS_OK;
-}
-
-template <typename T>
-int launch_fwd_w(int warps, const void *vol, const MarchArgs &A, const BatchDev &B, const RayGeo *geo, float *out,
-                 int *valid, uint32_t *status, unsigned *counter, const FwdKeep &kp, const FwdLaunch &fl,
-                 const RefineSel &sel, const PoseFrame *frames, const VolPlace &vp, int64_t q0, int64_t qn,
-                 cudaStream_t s)
-{
-    switch (warps) {
-    case 2: launch_fwd_t<T, 2>(vol, A, B, geo, out, valid, status, counter, kp, fl, sel, frames, vp, q0, qn, s); break;
-    case 4: launch_fwd_t<T, 4>(vol, A, B, geo, out, valid, status, counter, kp, fl, sel, frames, vp, q0, qn, s); break;
-    case 8: launch_fwd_t<T, 8>(vol, A, B, geo, out, valid, status, counter, kp, fl, sel, frames, vp, q0, qn, s); break;
-    default: return DIFFUS_E_PLAN;
-    }
-    return DIFFUS_OK;
-}
-
-template <typename T>
-int launch_bwd_w(int warps, const void *vol, const MarchArgs &A, const BatchDev &B, const RayGeo *geo, const float *gy,
-                 float *gz, double *part, float4 *ckpt, unsigned *counter, const float *mbuf, const float2 *kbuf,
-                 int grid, bool pose, int64_t q0, int64_t qn, cudaStream_t s)
-{
-    switch (warps) {
-    case 2: return launch_bwd_t<T, 2>(vol, A, B, geo, gy, gz, part, ckpt, counter, mbuf, kbuf, grid, pose, q0, qn,
-                                       s);
-    case 4: return launch_bwd_t<T, 4>(vol, A, B, geo, gy, gz, part, ckpt, counter, mbuf, kbuf, grid, pose, q0, qn,
-                                       s);
-    case 8: return launch_bwd_t<T, 8>(vol, A, B, geo, gy, gz, part, ckpt, counter, mbuf, kbuf, grid, pose, q0, qn,
-                                       s);
-    default: return DIFFUS_E_PLAN;
-    }
-}
 
 }  // namespace
 
@@ -588,14 +330,15 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
     if ((rc = check_params(prm))) return rc;
     if (!fans || !plan_host || !img_offsets) return DIFFUS_E_NULL;
     if (P < 1) return DIFFUS_E_DIMS;
-    int64_t total_rays = 0, total_img = 0, total_gz = 0, total_ck = 0;
+    int64_t total_rays = 0, total_img = 0, total_pad = 0, total_gz = 0, total_ck = 0;
     int max_S = 0;
     double max_depth = 0.0;
     for (int p = 0; p < P; p++) {
         if ((rc = check_fan(&fans[p], vd))) return rc;
         total_rays += fans[p].n_rays;
         total_img += (int64_t)fans[p].n_rays * fans[p].n_samples;
-        total_gz += (int64_t)fans[p].n_rays * (fans[p].n_samples + 1);
+        total_pad += (int64_t)fans[p].n_rays * row_stride(fans[p].n_samples);
+        total_gz += (int64_t)fans[p].n_rays * gz_stride(fans[p].n_samples);
         total_ck += (int64_t)fans[p].n_rays * ((fans[p].n_samples + kSeg - 1) / kSeg);
         max_S = std::max(max_S, (int)fans[p].n_samples);
         max_depth = std::max(max_depth, fans[p].depth_mm);
@@ -622,6 +365,7 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
     H.P = P;
     H.total_rays = total_rays;
     H.total_img = total_img;
+    H.total_pad = total_pad;
     H.total_gz = total_gz;
     H.total_ckpt = total_ck;
     H.n_tiles = n_tiles;
@@ -643,6 +387,7 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
     H.off_pose = z.off[0]; H.off_depth = z.off[1]; H.off_ray0 = z.off[2]; H.off_ray_pose = z.off[3];
     H.off_ray_j = z.off[4]; H.off_order = z.off[5]; H.off_row_off = z.off[6]; H.off_gz_off = z.off[7];
     H.off_ck_off = z.off[8]; H.off_tiles = z.off[9]; H.off_ftiles = z.off[10]; H.off_spk = z.off[11];
+    H.off_pad_off = z.off[12];
     H.bytes = z.bytes;
     H.params_fp = params_fingerprint(prm);
     {
@@ -672,25 +417,29 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
     int64_t *row_off = at_mut<int64_t>(plan_host, H.off_row_off);
     int64_t *gz_off = at_mut<int64_t>(plan_host, H.off_gz_off);
     int64_t *ck_off = at_mut<int64_t>(plan_host, H.off_ck_off);
+    int64_t *pad_off = at_mut<int64_t>(plan_host, H.off_pad_off);
     BlurTile *tiles = at_mut<BlurTile>(plan_host, H.off_tiles);
     TileDesc *ftiles = at_mut<TileDesc>(plan_host, H.off_ftiles);
 
-    int64_t r = 0, img = 0, g = 0, ck = 0, t = 0, ft = 0, cb = 0;
+    int64_t r = 0, img = 0, pad = 0, g = 0, ck = 0, t = 0, ft = 0, cb = 0;
     for (int p = 0; p < P; p++) {
         const diffus_fan &f = fans[p];
+        const int ld = row_stride(f.n_samples), ldz = gz_stride(f.n_samples);
         {
             const int nseg_p = (f.n_samples + kSeg - 1) / kSeg;
             const int ncar_p = (f.n_samples + kCarryRows - 1) / kCarryRows;
             for (int j0 = 0; j0 < f.n_rays; j0 += kWarp)
                 ftiles[ft++] = TileDesc{p, j0, std::min(kWarp, f.n_rays - j0), f.n_samples,
-                                        img + (int64_t)j0 * f.n_samples, g + (int64_t)j0 * (f.n_samples + 1),
-                                        ck + (int64_t)j0 * nseg_p, cb + (int64_t)j0 * ncar_p, (int32_t)(r + j0), 0};
+                                        img + (int64_t)j0 * f.n_samples, pad + (int64_t)j0 * ld,
+                                        g + (int64_t)j0 * ldz + kGzLead, ck + (int64_t)j0 * nseg_p,
+                                        cb + (int64_t)j0 * ncar_p, (int32_t)(r + j0), 0};
             cb += (int64_t)f.n_rays * ncar_p;
         }
         double a = attenuation_a(&f);
         float hi, lo;
         gain_l2(a, hi, lo);
-        pp[p] = PlanPose{f.n_rays, f.n_samples, f.fov_rad, f.depth_mm, (float)(a * a), H.blurW, img, a * a, hi, lo, 0};
+        pp[p] = PlanPose{f.n_rays, f.n_samples, f.fov_rad, f.depth_mm, (float)(a * a), H.blurW, img, a * a, hi, lo, ld, 0,
+                         pad};
         depth[p] = f.depth_mm;
         ray0[p] = (int32_t)r;
         img_offsets[p] = img;
@@ -699,13 +448,15 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
             ray_pose[r] = p;
             ray_j[r] = j;
             row_off[r] = img + (int64_t)j * f.n_samples;
-            gz_off[r] = g;
+            pad_off[r] = pad + (int64_t)j * ld;
+            gz_off[r] = g + kGzLead;
             ck_off[r] = ck;
-            g += f.n_samples + 1;
+            g += ldz;
             ck += nseg;
         }
         for (int k0 = 0; k0 < f.n_samples; k0 += kBlurRows) tiles[t++] = BlurTile{p, f.n_rays, k0, 0};
         img += (int64_t)f.n_rays * f.n_samples;
+        pad += (int64_t)f.n_rays * ld;
     }
     ray0[P] = (int32_t)r;
     img_offsets[P] = img;
@@ -801,6 +552,7 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
     B.row_off = at<int64_t>(plan_dev, H.off_row_off);
     B.gz_off = at<int64_t>(plan_dev, H.off_gz_off);
     B.ck_off = at<int64_t>(plan_dev, H.off_ck_off);
+    B.pad_off = at<int64_t>(plan_dev, H.off_pad_off);
     B.total_rays = H.total_rays;
 
     if (status && cudaMemsetAsync(status, 0, 4 * sizeof(uint32_t), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
@@ -821,10 +573,17 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
     // (the adjoint samples dZ/dp itself only in a pose-only call)
     const bool march_pose = grad_poses && !grad_vol;
     const bool keep_samples = bwd && !march_pose;
-    const FwdKeep kp{bwd ? L.ckpt : nullptr, bwd ? L.mbuf : nullptr, keep_samples ? L.kbuf : nullptr,
-                     keep_samples ? L.bcar : nullptr};
+    // the lane-per-ray form keeps (impedance, r) pairs, the warp-per-ray form
+    // two rows of floats, so that a lane's chunk of either is whole 16-byte
+    // accesses
+    float *zbuf = (float *)L.kbuf, *rbuf = zbuf + H.total_gz;
+    const bool tiles = H.fwd_form == 1;
+    const FwdKeep kp{bwd ? L.ckpt : nullptr, bwd && tiles ? L.mbuf : nullptr, keep_samples && tiles ? L.kbuf : nullptr,
+                     keep_samples && tiles ? L.bcar : nullptr, keep_samples && !tiles ? zbuf : nullptr,
+                     keep_samples && !tiles ? rbuf : nullptr};
     const VolPlace vp = make_place(vd);
-    FwdLaunch fl{grid, H.fwd_form, at<TileDesc>(plan_dev, H.off_ftiles), H.n_ftiles, nullptr};
+    FwdLaunch fl{grid, H.fwd_form, at<TileDesc>(plan_dev, H.off_ftiles), H.n_ftiles, nullptr,
+                 prm->blur != 0};
     if (H.fwd_form == 0 && prm->speckle) {
         // the speckle field first; the march reads it, and so does the adjoint
         const int sgrid = (int)std::min<int64_t>((H.n_spk + kTileWarps - 1) / kTileWarps, (int64_t)sm_count() * 16);
@@ -834,11 +593,8 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
     }
     if (H.fwd_form == 1) fl.grid = sm_count() * std::max(1, H.ctas_per_sm * H.warps / kTileWarps);
     auto march = [&](int64_t q0, int64_t qn, unsigned *ctr) {
-        if (vd->dtype == DIFFUS_F32)
-            return launch_fwd_w<float>(H.warps, vol, A, B, L.geo, march_out, ray_valid, status, ctr, kp, fl, L.sel,
-                                       L.frames, vp, q0, qn, s);
-        return launch_fwd_w<unsigned short>(H.warps, vol, A, B, L.geo, march_out, ray_valid, status, ctr, kp, fl,
-                                            L.sel, L.frames, vp, q0, qn, s);
+        return launch_batch_fwd(vd->dtype, H.warps, vol, A, B, L.geo, march_out, ray_valid, status, ctr, kp, fl, L.sel,
+                                L.frames, vp, q0, qn, s);
     };
     const int rgrid = (int)std::min<int64_t>((H.total_rays + 7) / 8, (int64_t)sm_count() * 16);
     BlurArgs bl{(float)prm->sigma0, (float)prm->sigma1, H.blurW, prm->atten};
@@ -875,7 +631,7 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
     } else {
         if ((rc = march(0, H.total_rays, L.counter + 0))) return rc;
         // the depth gain rides on the blur's output; without blur it is a row pass
-        if (prm->atten && !prm->blur) k_batch_row_gain<<<rgrid, 256, 0, s>>>(march_out, march_out, B);
+        if (prm->atten && !prm->blur) k_batch_row_gain<<<rgrid, 256, 0, s>>>(march_out, B.row_off, march_out, B.row_off, B);
         mark(DIFFUS_TR_BLUR);
         if (prm->blur) launch_batch_blur<false>(L.y, images, dpose, dtiles, H.n_tiles, bl, tgrid, L.counter + 2, s);
         mark(DIFFUS_TR_FWD_END);
@@ -896,12 +652,11 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
             return DIFFUS_E_LAUNCH;
         return DIFFUS_OK;
     };
+    // dL/dy in internal rows: what the blur transpose or the gain pass wrote
+    const bool gy_padded = prm->blur || prm->atten;
     auto adjoint = [&](const float *gyc, int64_t q0, int64_t qn, unsigned *ctr) {
-        if (vd->dtype == DIFFUS_F32)
-            return launch_bwd_w<float>(H.warps, vol, A, B, L.geo, gyc, L.gz, L.part, L.ckpt, ctr, L.mbuf, L.kbuf, grid,
-                                       march_pose, q0, qn, s);
-        return launch_bwd_w<unsigned short>(H.warps, vol, A, B, L.geo, gyc, L.gz, L.part, L.ckpt, ctr, L.mbuf, L.kbuf,
-                                            grid, march_pose, q0, qn, s);
+        return launch_batch_bwd(vd->dtype, H.warps, vol, A, B, L.geo, gyc, gy_padded, L.gz, L.part, L.ckpt, ctr, L.mbuf,
+                                zbuf, rbuf, grid, march_pose, q0, qn, s);
     };
     const bool tile_bwd = H.fwd_form == 1 && !march_pose;
     // range by range: each chunk's blur transpose and adjoint march after its
@@ -934,7 +689,7 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
             gy = L.gy;
         }
         if (prm->atten && !prm->blur) {   // the depth gain is its own adjoint (with blur it rides on the blur)
-            k_batch_row_gain<<<rgrid, 256, 0, s>>>(gy, L.gy, B);
+            k_batch_row_gain<<<rgrid, 256, 0, s>>>(gy, B.row_off, L.gy, B.pad_off, B);
             gy = L.gy;
         }
         mark(DIFFUS_TR_MARCH_BWD);
@@ -945,7 +700,7 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
             const int bgrid = sm_count() * 6;
             k_batch_bwd_tiles<<<bgrid, kTileWarpsBwd * 32, 0, s>>>(A, B, at<TileDesc>(plan_dev, H.off_ftiles),
                                                                 H.n_ftiles, gy, L.mbuf, L.kbuf, L.bcar, L.gz,
-                                                                L.counter + 1);
+                                                                L.counter + 1, gy_padded);
             rc = DIFFUS_OK;
         } else {
             rc = adjoint(gy, 0, H.total_rays, L.counter + 1);

@@ -28,6 +28,15 @@ constexpr int kBwdValThreadsPerSM = 768;
 // 512-pose batch: forward phase 1.780 ms at 768 threads, 1.711 at 896, 1.789
 // at 1024 and 64 registers)
 constexpr int kFwdThreadsPerSM = 896;
+// Internal rows (pre-blur echoes, speckle factors, blurred gradients) of S
+// values are kept at a stride of whole 32-byte sectors, so that a lane's
+// chunk of kChunk rows is two aligned 16-byte accesses; a row of S + 1
+// gradient samples starts kChunk - 1 floats into its block, which puts the
+// kChunk samples that a lane finalises (its chunk's first sample belongs to
+// the lane before) on a sector too.
+__host__ __device__ inline int row_stride(int S) { return (S + kChunk - 1) / kChunk * kChunk; }
+__host__ __device__ inline int gz_stride(int S) { return row_stride(S) + kChunk; }
+constexpr int kGzLead = kChunk - 1;
 constexpr float kPoleEps = 1e-6f;            // det(A_k) threshold of a well-posed depth
 constexpr int kMaxW = 32;                    // largest lateral blur half-width
 
@@ -77,7 +86,8 @@ __device__ __forceinline__ float ldv(const unsigned short *__restrict__ p, unsig
 __device__ __forceinline__ void axis_split(long long X, int n, int &i0, float &f, bool &inside)
 {
     int hi = (int)(X >> 32);
-    float fr = __uint_as_float(0x3F800000u | ((unsigned)X >> 9)) - 1.0f;  // 23-bit fraction
+    // 1.f with the 23-bit fraction: (0x7F : low word) >> 9 is one funnel shift
+    float fr = __uint_as_float(__funnelshift_r((unsigned)X, 0x7Fu, 9)) - 1.0f;
     bool below = X < 0;
     bool above = hi >= n - 1;
     i0 = below ? 0 : (above ? n - 2 : hi);
@@ -227,11 +237,14 @@ struct Xfer {
     float m00, m01, m10, delta;
 };
 
-__device__ __forceinline__ Xfer xfer(float r, float a2, int mode)
+// The mode is a template argument of the hot marches: with a runtime mode
+// every use computes both readings' entries.
+template <int MODE>
+__device__ __forceinline__ Xfer xfer_t(float r, float a2)
 {
     Xfer t;
     float r2 = __fmul_rn(r, r);   // rounded on its own: 1 - r^2 is never fused (same bits in every kernel)
-    if (mode == DIFFUS_MODE_LITERAL) {
+    if (MODE == DIFFUS_MODE_LITERAL) {
         float R = fabsf(r);
         t.m00 = a2 * fmaf(-2.0f, r2, 1.0f);
         t.m01 = a2 * R;
@@ -243,6 +256,11 @@ __device__ __forceinline__ Xfer xfer(float r, float a2, int mode)
     }
     t.delta = a2 * (1.0f - r2);
     return t;
+}
+
+__device__ __forceinline__ Xfer xfer(float r, float a2, int mode)
+{
+    return mode == DIFFUS_MODE_LITERAL ? xfer_t<DIFFUS_MODE_LITERAL>(r, a2) : xfer_t<DIFFUS_MODE_SIGNED>(r, a2);
 }
 
 // Transfer entries of one interface in double-single precision (the

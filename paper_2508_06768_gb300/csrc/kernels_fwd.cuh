@@ -150,20 +150,20 @@ struct RefineSel {
     unsigned *ticket;
 };
 
-template <typename T>
+template <typename T, int MODE, bool TRACK>
 __global__ void __launch_bounds__(kWarpsFwd * 32) k_march_fwd(const T *__restrict__ vol, MarchArgs A,
                                                               const RayGeo *__restrict__ geo, int n_rays,
                                                               float *__restrict__ out, int *__restrict__ valid,
                                                               uint32_t *__restrict__ status, RefineSel sel)
 {
-    __shared__ float buf[kWarpsFwd][kSegPad];
+    __shared__ float2 buf[kWarpsFwd][kSegPad];
     const int w = threadIdx.x >> 5;
     const int j = blockIdx.x * kWarpsFwd + w;
     if (j >= n_rays) return;
     RayGeo rg = geo[j];
     RayOut o{out + (size_t)j * rg.S, valid ? valid + j : nullptr, status, nullptr, nullptr, nullptr, nullptr,
-             sel.rinfo ? sel.rinfo + j : nullptr, sel.rlist, sel.rcount, j};
-    march_fwd_ray<T>(vol, A, rg, o, buf[w]);
+             sel.rinfo ? sel.rinfo + j : nullptr, sel.rlist, sel.rcount, j, false};
+    march_fwd_ray<T, MODE, TRACK, true, false>(vol, A, rg, o, buf[w]);
 }
 
 // The refined pass of one ray that the FP32 pass listed: its FP64 line from
@@ -176,7 +176,7 @@ __device__ __forceinline__ void refine_ray(const T *__restrict__ vol, const Marc
     RayLine64 line;
     double st, ct;
     ray_line(f, rg.ray, fan, vp, line.x0, line.dx, st, ct);
-    march_fwd_ray<T, true, STREAM>(vol, A, rg, out, buf, dbuf, &line, info);
+    march_refine_ray<T, STREAM>(vol, A, rg, out, buf, dbuf, line, info);
 }
 
 // Refined pass of one pose: each warp takes listed rays from the ticket
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kWarpsFwd * 32, kRefineWarpsPerSM / kWarpsFwd)
         const int j = sel.rlist[q];
         const RayGeo rg = geo[j];
         RayOut o{out + (size_t)j * rg.S, valid ? valid + j : nullptr, status, nullptr, nullptr, nullptr, nullptr,
-                 nullptr, nullptr, nullptr, j};
+                 nullptr, nullptr, nullptr, j, false};
         refine_ray<T, false>(vol, A, rg, f, fan, vp, o, sel.rinfo[j], buf[w], dbuf[w]);
         __syncwarp();
     }
@@ -232,7 +232,7 @@ __device__ __forceinline__ float blur_w(const BlurArgs &b, int m, int k, float i
 // Lateral blur of one pose image (Section 2.4), or its transpose, on one
 // strip of 32 echo rows [k0, k0 + 32) (one row per lane), output rays
 // [j0, j1) of the n rays.
-// in/out: [n][S].
+// in/out: [n] rows of S at strides si and so.
 // Forward:   out[j] = sum_m w_m in[j+m] / N_j        (valid j+m)
 // Transpose: out[j] = sum_m w_m in[j+m] / N_{j+m}    (valid j+m)
 // with N_j = sum of w_m over the valid j+m.  The warp sweeps the rays once:
@@ -243,7 +243,7 @@ __device__ __forceinline__ float blur_w(const BlurArgs &b, int m, int k, float i
 // known at compile time; WT < 0 is the general path for wide kernels, which
 // reads the window through the cache instead.
 template <bool TRANSPOSE, int WT>
-__device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out, int n, int S,
+__device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out, int n, int S, int si, int so,
                            const BlurArgs &b, int k0, int j0, int j1, float l2_hi, float l2_lo)
 {
     const int lane = threadIdx.x & 31;
@@ -275,7 +275,7 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
         };
         auto ld = [&](int j) -> float {
             if (!kin || j < 0 || j >= n) return 0.0f;
-            float x = __ldg(src + (size_t)j * S);
+            float x = __ldg(src + (size_t)j * si);
             if (TRANSPOSE) x *= rnorm(j);
             return x;
         };
@@ -288,11 +288,11 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
             // the other lanes' rows of this block are read at row 0 (valid
             // memory) and not written
             if (jb >= WW && jb + B + 2 * WW <= n && jb + B <= j1) {
-                const float *p = src + (size_t)(jb + WW) * S;
-                float *q = dst + (size_t)jb * S;
+                const float *p = src + (size_t)(jb + WW) * si;
+                float *q = dst + (size_t)jb * so;
 #pragma unroll
                 for (int t = 0; t < B; t++) {
-                    const float x = __ldg(p + (size_t)t * S);
+                    const float x = __ldg(p + (size_t)t * si);
                     win[2 * WW + t] = TRANSPOSE ? x * rfull : x;
                 }
 #pragma unroll
@@ -301,7 +301,7 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
 #pragma unroll
                     for (int m = 1; m <= WW; m++) acc = fmaf(w[m], win[i + WW - m] + win[i + WW + m], acc);
                     if (!TRANSPOSE) acc *= rfull;
-                    if (kin) q[(size_t)i * S] = acc * gk;
+                    if (kin) q[(size_t)i * so] = acc * gk;
                 }
 #pragma unroll
                 for (int t = 0; t < 2 * WW; t++) win[t] = win[t + B];
@@ -309,7 +309,7 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
             }
             float nx[B];
 #pragma unroll
-            for (int t = 0; t < B; t++) nx[t] = (kin && jb + WW + t < n) ? __ldg(src + (size_t)(jb + WW + t) * S) : 0.0f;
+            for (int t = 0; t < B; t++) nx[t] = (kin && jb + WW + t < n) ? __ldg(src + (size_t)(jb + WW + t) * si) : 0.0f;
 #pragma unroll
             for (int t = 0; t < B; t++)
                 win[2 * WW + t] = (TRANSPOSE && jb + WW + t < n) ? nx[t] * rnorm(jb + WW + t) : nx[t];
@@ -321,7 +321,7 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
                 for (int m = 1; m <= WW; m++) acc = fmaf(w[m], win[i + WW - m] + win[i + WW + m], acc);
                 if (kin && j < j1) {
                     if (!TRANSPOSE) acc *= rnorm(j);
-                    dst[(size_t)j * S] = acc * gk;
+                    dst[(size_t)j * so] = acc * gk;
                 }
             }
 #pragma unroll
@@ -340,7 +340,7 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
     };
     auto ld = [&](int j) -> float {
         if (j < 0 || j >= n) return 0.0f;
-        float x = __ldg(src + (size_t)j * S);
+        float x = __ldg(src + (size_t)j * si);
         if (TRANSPOSE) x *= 1.0f / N_of(j);
         return x;
     };
@@ -348,7 +348,7 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
         float acc = wt(0) * ld(j);
         for (int m = 1; m <= W; m++) acc = fmaf(wt(m), ld(j - m) + ld(j + m), acc);
         if (!TRANSPOSE) acc *= 1.0f / N_of(j);
-        dst[(size_t)j * S] = acc * gk;
+        dst[(size_t)j * so] = acc * gk;
     }
 }
 
@@ -358,12 +358,12 @@ constexpr int kBlurSegRays = 64;
 
 template <bool TRANSPOSE, int WT>
 __global__ void __launch_bounds__(kBlurWarps * 32) k_blur(const float *__restrict__ in, float *__restrict__ out,
-                                                          int n, int S, BlurArgs b, float l2_hi, float l2_lo)
+                                                          int n, int S, int si, int so, BlurArgs b, float l2_hi, float l2_lo)
 {
     const int strip = blockIdx.x * kBlurWarps + (threadIdx.x >> 5);
     if (strip * kBlurRows >= S) return;
     const int j0 = blockIdx.y * kBlurSegRays;
-    blur_strip<TRANSPOSE, WT>(in, out, n, S, b, strip * kBlurRows, j0, min(n, j0 + kBlurSegRays), l2_hi, l2_lo);
+    blur_strip<TRANSPOSE, WT>(in, out, n, S, si, so, b, strip * kBlurRows, j0, min(n, j0 + kBlurSegRays), l2_hi, l2_lo);
 }
 
 }  // namespace dfs

@@ -78,15 +78,30 @@ struct RayOut {
     int *valid;       // nullable: leading pole-free rows
     uint32_t *status; // nullable
     float4 *ckpt;     // nullable: scan carry (b0, b1, D) at every segment start, for the adjoint
-    float *mrow;      // nullable: speckle factor of every row, for the adjoint
-    float2 *krow;     // nullable: per sample k = 0..S, (zref + dz, r_{k-1}) for the adjoint (r_{-1} = 0)
+    float *zrow;      // nullable: per sample k = 0..S, zref + dz for the adjoint (a row of a gz_stride block) ...
+    float *rrow;      // ... and r of the interface before it, r_{k-1}, at k = 1..S (set together with zrow)
     const float *min; // nullable: the row's speckle factors, drawn ahead of the march (then not drawn here)
     // selective refinement (FP32 pass; all null when refinement is off):
     int2 *rinfo;      // this ray's (segments for the refined pass, first ill-posed depth of the FP32 pass)
     int *rlist;       // rays that need the refined pass are appended here ...
     unsigned *rcount; // ... at this counter
     int rid;          // this ray's index in rinfo / rlist
+    bool padded;      // row is an internal row (row_stride, aligned): whole chunks are stored
 };
+
+// A lane's chunk of an internal row (aligned, row_stride long): two 16-byte
+// evict-first accesses, zeros for a lane past the row's end (!on).  In the
+// last chunk the entries past the row's end are whatever the buffer holds.
+__device__ __forceinline__ void load_chunk(const float *p, bool on, float (&v)[kChunk])
+{
+    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+    if (on) {
+        a = __ldcs(reinterpret_cast<const float4 *>(p));
+        b = __ldcs(reinterpret_cast<const float4 *>(p) + 1);
+    }
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
 
 __device__ __forceinline__ int smem_idx(int x) { return x + (x >> 3); }
 
@@ -97,24 +112,21 @@ __device__ __forceinline__ void sample_pos(const RayGeo &rg, int k, long long &X
     Z = rg.X0[2] + (long long)k * rg.DX[2];
 }
 
-// Phase A of a segment: samples base+1 .. base+256 lane-interleaved and
-// writes r_i (i = base..base+255, 0 past the ray) into buf[smem_idx(i-base)].
-// (czr, cdz) carries the sample at `base` in and the one at base+256 out.
-// krow (nullable) also receives, per sample k, (zref + dz, r_{k-1}).
-// REFINE (the refined pass) also writes r_i in double-single precision into
-// dbuf (h, l), from double-single samples (sample_z_ff) at the FP64-line
-// positions of `line`; czf carries that sample at `base` in and the one at
+// Phase A of a segment in the refined pass: samples base+1 .. base+256
+// lane-interleaved, r_i (i = base..base+255, 0 past the ray) into
+// buf[smem_idx(i-base)] and, in double-single precision, into dbuf (h, l),
+// from double-single samples (sample_z_ff) at the FP64-line positions of
+// `line`.  (czr, cdz) and czf carry the sample at `base` in and the one at
 // base+256 out.
-template <typename T, bool REFINE = false>
-__device__ __forceinline__ void seg_reflections(const T *__restrict__ vol, const VolGeo &g, const RayGeo &rg,
-                                                int base, float &czr, float &cdz, float *__restrict__ buf,
-                                                float2 *__restrict__ dbuf = nullptr, float2 *__restrict__ krow = nullptr,
-                                                const RayLineFF *line = nullptr, FF *czf = nullptr)
+template <typename T>
+__device__ __forceinline__ void seg_reflections_ff(const T *__restrict__ vol, const VolGeo &g, const RayGeo &rg,
+                                                   int base, float &czr, float &cdz, float *__restrict__ buf,
+                                                   float2 *__restrict__ dbuf, const RayLineFF &line, FF &czf)
 {
     const int lane = threadIdx.x & 31;
     const int S = rg.S;
     float pzr = czr, pdz = cdz;
-    FF pzf = REFINE ? *czf : FF{0.0f, 0.0f};
+    FF pzf = czf;
     long long X, Y, Z;
     sample_pos(rg, base + lane + 1, X, Y, Z);
     const long long sX = rg.DX[0] * kWarp, sY = rg.DX[1] * kWarp, sZ = rg.DX[2] * kWarp;
@@ -125,12 +137,10 @@ __device__ __forceinline__ void seg_reflections(const T *__restrict__ vol, const
         FF zf{0.0f, 0.0f};
         if (k <= S) {
             float cor[8];
-            sample_z<T, false>(vol, g, X, Y, Z, zr, dz, nullptr, REFINE ? cor : nullptr);
-            if (REFINE) {
-                const float kf = (float)k;
-                zf = sample_z_ff(cor, g, X, Y, Z, line_pos(line->x0[0], line->dx[0], kf),
-                                 line_pos(line->x0[1], line->dx[1], kf), line_pos(line->x0[2], line->dx[2], kf));
-            }
+            sample_z<T, false>(vol, g, X, Y, Z, zr, dz, nullptr, cor);
+            const float kf = (float)k;
+            zf = sample_z_ff(cor, g, X, Y, Z, line_pos(line.x0[0], line.dx[0], kf),
+                             line_pos(line.x0[1], line.dx[1], kf), line_pos(line.x0[2], line.dx[2], kf));
         }
         X += sX;
         Y += sY;
@@ -140,25 +150,112 @@ __device__ __forceinline__ void seg_reflections(const T *__restrict__ vol, const
         if (lane == 0) { lzr = pzr; ldz = pdz; }
         float r = (k - 1 < S) ? refl(lzr, ldz, zr, dz) : 0.0f;
         buf[smem_idx(t * kWarp + lane)] = r;
-        if (krow && k <= S) __stcs(krow + k, make_float2(zr + dz, r));
-        if (REFINE) {
-            FF lzf{__shfl_up_sync(0xffffffffu, zf.h, 1), __shfl_up_sync(0xffffffffu, zf.l, 1)};
-            if (lane == 0) lzf = pzf;
-            const FF rf = (k - 1 < S) ? refl_ff(lzf, zf) : FF{0.0f, 0.0f};
-            dbuf[smem_idx(t * kWarp + lane)] = make_float2(rf.h, rf.l);
-            pzf = FF{__shfl_sync(0xffffffffu, zf.h, 31), __shfl_sync(0xffffffffu, zf.l, 31)};
-        }
+        FF lzf{__shfl_up_sync(0xffffffffu, zf.h, 1), __shfl_up_sync(0xffffffffu, zf.l, 1)};
+        if (lane == 0) lzf = pzf;
+        const FF rf = (k - 1 < S) ? refl_ff(lzf, zf) : FF{0.0f, 0.0f};
+        dbuf[smem_idx(t * kWarp + lane)] = make_float2(rf.h, rf.l);
+        pzf = FF{__shfl_sync(0xffffffffu, zf.h, 31), __shfl_sync(0xffffffffu, zf.l, 31)};
         pzr = __shfl_sync(0xffffffffu, zr, 31);
         pdz = __shfl_sync(0xffffffffu, dz, 31);
     }
     czr = pzr;
     cdz = pdz;
-    if (REFINE) *czf = pzf;
+    czf = pzf;
 }
 
-// Chunk product Q = M_{i0} ... M_{i0+7} (identity past the ray) and its
-// determinant dq.
-__device__ __forceinline__ void chunk_product(const float *rr, int i0, int S, float a2, int mode, Mat2 &Q, float &dq)
+// Samples per lane and branch of the segment sampling: two samples' loads
+// are in flight together.
+constexpr int kSampleGroup = 2;
+
+// Reflection coefficients of a segment, rr[t] = r of interface i0 + t of this
+// lane's chunk (i0 = base + 8 lane; 0 past the ray).  The samples base+1 ..
+// base+256 are taken lane-interleaved (neighbouring lanes share cells and
+// lines), go through shared memory as (zref, dz) pairs, and every lane forms
+// its chunk's coefficients from its own eight samples and the one before, so
+// no neighbour exchange is needed per sample.  The branches are uniform over
+// the warp: past the ray's end a lane samples at a clamped position (valid
+// memory) and the coefficient is dropped.  (czr, cdz) carries the sample at
+// `base` in and the one at base+256 out.  zrow (nullable) receives
+// zref + dz of the samples.
+template <typename T, bool STREAM>
+__device__ __forceinline__ void seg_coefficients(const T *__restrict__ vol, const VolGeo &g, const RayGeo &rg,
+                                                 int base, float &czr, float &cdz, float2 *__restrict__ buf,
+                                                 float *__restrict__ zrow, float (&rr)[kChunk])
+{
+    const int lane = threadIdx.x & 31;
+    const int S = rg.S;
+    long long X, Y, Z;
+    sample_pos(rg, base + lane + 1, X, Y, Z);
+    const long long sX = rg.DX[0] * kWarp, sY = rg.DX[1] * kWarp, sZ = rg.DX[2] * kWarp;
+    float2 *dst = buf + smem_idx(lane);
+    float *zdst = zrow + base + lane + 1;
+    const int left = S - base - lane;   // samples base + lane + 1 + n exist for n < left
+#pragma unroll
+    for (int t0 = 0; t0 < kChunk; t0 += kSampleGroup) {
+        if (base + t0 * kWarp < S) {
+#pragma unroll
+            for (int t = t0; t < t0 + kSampleGroup; t++) {
+                float zr, dz;
+                sample_z<T, false>(vol, g, X, Y, Z, zr, dz);
+                X += sX;
+                Y += sY;
+                Z += sZ;
+                dst[smem_idx(t * kWarp)] = make_float2(zr, dz);
+                if (zrow && t * kWarp < left) {
+                    if (STREAM)
+                        __stcs(zdst + t * kWarp, zr + dz);
+                    else
+                        zdst[t * kWarp] = zr + dz;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    const float2 *src = buf + lane * (kChunk + 1);   // smem_idx(8 lane)
+    float2 s[kChunk];
+#pragma unroll
+    for (int t = 0; t < kChunk; t++) s[t] = src[t];
+    float pzr = __shfl_up_sync(0xffffffffu, s[kChunk - 1].x, 1);
+    float pdz = __shfl_up_sync(0xffffffffu, s[kChunk - 1].y, 1);
+    if (lane == 0) {
+        pzr = czr;
+        pdz = cdz;
+    }
+    czr = __shfl_sync(0xffffffffu, s[kChunk - 1].x, 31);
+    cdz = __shfl_sync(0xffffffffu, s[kChunk - 1].y, 31);
+#pragma unroll
+    for (int t = 0; t < kChunk; t++) {
+        rr[t] = refl(pzr, pdz, s[t].x, s[t].y);
+        pzr = s[t].x;
+        pdz = s[t].y;
+    }
+    if (base + kSeg > S) {
+        const int i0 = base + lane * kChunk;
+#pragma unroll
+        for (int t = 0; t < kChunk; t++)
+            if (i0 + t >= S) rr[t] = 0.0f;
+    }
+    __syncwarp();
+}
+
+// Chunk product Q = M_{i0} ... M_{i0+7} and its determinant dq.  Past the
+// ray r is 0; the product of such a chunk reaches no row of the ray.
+template <int MODE>
+__device__ __forceinline__ void chunk_product(const float (&rr)[kChunk], float a2, Mat2 &Q, float &dq)
+{
+    const Xfer x0 = xfer_t<MODE>(rr[0], a2);
+    Q = {x0.m00, x0.m01, x0.m10, 1.0f};
+    dq = x0.delta;
+#pragma unroll
+    for (int t = 1; t < kChunk; t++) {
+        const Xfer x = xfer_t<MODE>(rr[t], a2);
+        mat_mul_xfer(Q, x);
+        dq *= x.delta;
+    }
+}
+
+// The same with a runtime mode, the identity past the ray (refined pass).
+__device__ __forceinline__ void chunk_product_ref(const float *rr, int i0, int S, float a2, int mode, Mat2 &Q, float &dq)
 {
     Q = mat_ident();
     dq = 1.0f;
@@ -309,78 +406,78 @@ __device__ __forceinline__ void chunk_speckle(const Speckle &sp, int i0, int S, 
     }
 }
 
+// A lane's chunk of echo rows: whole 16-byte stores where the row allows it
+// (STREAM: evict-first; the batched kernel writes gigabytes of one-pass rows).
+template <bool STREAM>
+__device__ __forceinline__ void store_rows(const RayOut &out, int i0, int S, const float (&y)[kChunk])
+{
+    const int over = out.padded ? kChunk - 1 : 0;   // rows a chunk store may write past S
+    if (((((uintptr_t)out.row) & 15) == 0) && i0 + kChunk <= S + over) {
+        float4 *dst = reinterpret_cast<float4 *>(out.row + i0);
+        const float4 lo = make_float4(y[0], y[1], y[2], y[3]), hi = make_float4(y[4], y[5], y[6], y[7]);
+        if (STREAM) {
+            __stcs(dst, lo);
+            __stcs(dst + 1, hi);
+        } else {
+            dst[0] = lo;
+            dst[1] = hi;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < kChunk; t++)
+            if (i0 + t < S) {
+                if (STREAM)
+                    __stcs(out.row + i0 + t, y[t]);
+                else
+                    out.row[i0 + t] = y[t];
+            }
+    }
+}
+
 // Forward march of one ray by one warp.  buf: this warp's shared row of
-// kSegPad floats; dbuf: kSegPad float pairs when REFINE.  STREAM writes the
-// output row with evict-first stores (the batched kernel).
+// kSegPad float pairs.  SPK_INLINE draws the speckle here (when it is on and
+// no factors are passed in out.min); without it the factors come from out.min
+// or there are none.  STREAM writes one-pass rows with evict-first stores
+// (the batched kernel).
 //
-// Without REFINE (the FP32 pass) and with out.rinfo set, the march also
-// decides whether the ray needs the refined pass (rows whose md falls below
+// TRACK (the FP32 pass of a refined render, out.rinfo set) also decides
+// whether the ray needs the refined pass (rows whose md falls below
 // kNeedCoef sqrt(S), or a pole): such a ray is appended to out.rlist, and its
 // valid-row count and status are left to the refined pass.
 //
-// REFINE (the refined pass, line = the ray's FP64 line, rinfo = what the FP32
-// pass recorded) redoes the first segments of the ray with one
-// iterative-refinement pass of the depth recurrence b_{i+1} = b_i M_i,
-// D_{i+1} = D_i delta_i: the FP32 states are kept, their residuals
-// rho_{i+1} = b_i M*_i - b_{i+1} are computed in double-single precision
-// (about 47 bits, ff.cuh) with M*_i the coefficients of double-single samples
-// at the FP64 line's positions (sample_z_ff), the error recurrence
-// e_{i+1} = e_i M_i + rho_{i+1} (e_0 = 0) of e_i = b*_i - b_i (b* the states
-// of the exact coefficients) is solved in FP32 with the same scan (affine
-// maps), and the echoes use the corrected states b_i + e_i and the refined
-// coefficient x*_i.  It covers rinfo.x segments, and goes on while the FP32
-// pass saw a pole there that the refined states do not confirm; rows beyond
-// keep the FP32 pass's values.
-template <typename T, bool REFINE = false, bool STREAM = false>
-__device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg,
-                              const RayOut &out, float *__restrict__ buf, float2 *__restrict__ dbuf = nullptr,
-                              const RayLine64 *line64 = nullptr, int2 rinfo = make_int2(0, 0))
+// The rows carry no per-row tests: a chunk keeps the smallest determinant
+// and a sum that is NaN once any row is not finite, and only a chunk that
+// fails either is walked again for the first ill-posed row and the count.
+template <typename T, int MODE, bool TRACK, bool SPK_INLINE, bool STREAM>
+__device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg, const RayOut &out,
+                              float2 *__restrict__ buf)
 {
     const int lane = threadIdx.x & 31;
     const int S = rg.S;
-    const uint32_t pose = A.sp.pose_ctr + (uint32_t)rg.pose;
-    const int nseg = (S + kSeg - 1) / kSeg;
-
-    float czr, cdz, cor0[8];
-    sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz, nullptr, REFINE ? cor0 : nullptr);
-    RayLineFF line_f;
-    FF czf{0.0f, 0.0f};
-    FF a2f{0.0f, 0.0f};
-    if (REFINE) {
-        line_f = line_ff(*line64);
-        czf = sample_z_ff(cor0, A.g, rg.X0[0], rg.X0[1], rg.X0[2], line_f.x0[0], line_f.x0[1], line_f.x0[2]);
-        a2f = ff_from_double(A.a2d);
-    }
-    if (!REFINE && out.krow && lane == 0) out.krow[0] = make_float2(czr + cdz, 0.0f);
+    const float a2 = A.a2;
+    float czr, cdz;
+    sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz);
+    if (out.zrow && lane == 0) out.zrow[0] = czr + cdz;
     float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;   // bottom row and det at segment start
     int first_bad = 0x7fffffff;
     int nonfinite = 0;
-    int last_need = -1;                         // FP32 pass: last row with md below the threshold
-    const float need_md = fmaxf(kNeedFloor, kNeedCoef * sqrtf((float)S));
-    const bool vec4 = ((((uintptr_t)out.row) & 15) == 0);
+    int last_need = -1;                         // TRACK: last row with md below the threshold
+    const float need_md = TRACK ? fmaxf(kNeedFloor, kNeedCoef * sqrtf((float)S)) : 0.0f;
+    bool pole_seen = false;                     // in an earlier segment
 
-    float es0 = 0.0f, es1 = 0.0f, esD = 0.0f;  // refinement: correction at segment start
-    // REFINE: segments to redo; extended while the FP32 pass's pole lies
-    // before the end and the refined states have not found one
-    const bool fp32_pole = rinfo.y <= S;
-    int seg = 0;
-    for (; seg < nseg; seg++) {
-        if (REFINE && seg >= rinfo.x) {
-            const bool pole_seen = __shfl_sync(0xffffffffu, first_bad, 0) <= S;   // lane 0 holds the reduced value
-            if (!(fp32_pole && !pole_seen)) break;
-        }
-        const int base = seg * kSeg;
-        if (out.ckpt && lane == 0) out.ckpt[seg] = make_float4(bs0 + es0, bs1 + es1, Ds + esD, 0.0f);
-        seg_reflections<T, REFINE>(vol, A.g, rg, base, czr, cdz, buf, dbuf, REFINE ? nullptr : out.krow, &line_f,
-                                   &czf);
-        __syncwarp();
+    for (int base = 0; base < S; base += kSeg) {
+        if (out.ckpt && lane == 0) out.ckpt[base / kSeg] = make_float4(bs0, bs1, Ds, 0.0f);
         const int i0 = base + lane * kChunk;
         float rr[kChunk];
-#pragma unroll
-        for (int t = 0; t < kChunk; t++) rr[t] = buf[smem_idx(lane * kChunk + t)];
+        seg_coefficients<T, STREAM>(vol, A.g, rg, base, czr, cdz, buf, out.zrow, rr);
+        if (out.rrow && i0 < S) {
+            float4 *dst = reinterpret_cast<float4 *>(out.rrow + i0 + 1);   // r_{i0} belongs to sample i0 + 1
+            __stcs(dst, make_float4(rr[0], rr[1], rr[2], rr[3]));
+            __stcs(dst + 1, make_float4(rr[4], rr[5], rr[6], rr[7]));
+        }
         Mat2 Q, E, Qall;
         float dq, de, dall;
-        chunk_product(rr, i0, S, A.a2, A.mode, Q, dq);
+        chunk_product<MODE>(rr, a2, Q, dq);
         warp_scan_prefix(Q, dq, E, de, Qall, dall);
         float b0 = fmaf(bs0, E.a, bs1 * E.c);
         float b1 = fmaf(bs0, E.b, bs1 * E.d);
@@ -393,50 +490,154 @@ __device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
             Ds *= dall;
         }
         float m[kChunk];
-        if (!REFINE && out.min) {
+        if (out.min) {
+            load_chunk(out.min + i0, i0 < S, m);
+        } else if (SPK_INLINE && A.sp.on) {
+            chunk_speckle(A.sp, i0, S, rg.ray, A.sp.pose_ctr + (uint32_t)rg.pose, m);
+        } else {
 #pragma unroll
-            for (int t = 0; t < kChunk; t++) m[t] = (i0 + t < S) ? __ldcs(out.min + i0 + t) : 1.0f;
-        } else if (A.sp.on) {
+            for (int t = 0; t < kChunk; t++) m[t] = 1.0f;
+        }
+        float y[kChunk];
+        const float cb0 = b0, cb1 = b1;          // state at the chunk start
+        float minq = 3.402823466e38f, fin = 0.0f;
+#pragma unroll
+        for (int t = 0; t < kChunk; t++) {
+            const Xfer x = xfer_t<MODE>(rr[t], a2);
+            const float q = fmaf(b0, x.m01, b1);          // det(A_{i+1})
+            const float e = x.m01 * D * frcp(b1 * q);
+            if (TRACK && i0 + t < S && fminf(b1, q) < need_md) last_need = i0 + t;
+            minq = fminf(minq, q);
+            const float nb0 = fmaf(b0, x.m00, b1 * x.m10);
+            b1 = q;
+            b0 = nb0;
+            D *= x.delta;
+            y[t] = m[t] * e;
+            fin = fmaf(y[t], 0.0f, fin);
+        }
+        const bool odd = !(fin == 0.0f);          // a row that is not finite (NaN states among them)
+        if (odd || (!pole_seen && minq < kPoleEps)) {
+            float c0 = cb0, c1 = cb1;
+#pragma unroll
+            for (int t = 0; t < kChunk; t++) {
+                const Xfer x = xfer_t<MODE>(rr[t], a2);
+                const float q = fmaf(c0, x.m01, c1);
+                if (i0 + t < S) {
+                    if (!(q >= kPoleEps)) first_bad = min(first_bad, i0 + t + 1);
+                    nonfinite += !isfinite(y[t]);
+                }
+                c0 = fmaf(c0, x.m00, c1 * x.m10);
+                c1 = q;
+            }
+        }
+        pole_seen = pole_seen || __any_sync(0xffffffffu, first_bad <= S);
+        if (i0 < S) store_rows<STREAM>(out, i0, S, y);
+    }
+
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        first_bad = min(first_bad, __shfl_xor_sync(0xffffffffu, first_bad, off));
+        nonfinite += __shfl_xor_sync(0xffffffffu, nonfinite, off);
+        if (TRACK) last_need = max(last_need, __shfl_xor_sync(0xffffffffu, last_need, off));
+    }
+    bool defer = false;     // FP32 pass of a ray that the refined pass redoes
+    if (TRACK) {
+        // rows up to the pole's (which the refined pass decides again), or
+        // up to the last row whose conditioning needs the refined states
+        const int cover = first_bad <= S ? first_bad - 1 : last_need;
+        const int segs = cover >= 0 ? cover / kSeg + 1 : 0;
+        defer = segs > 0;
+        if (lane == 0) {
+            out.rinfo[0] = make_int2(segs, first_bad <= S ? first_bad : S + 1);
+            if (defer) {
+                out.rlist[atomicAdd(out.rcount, 1u)] = out.rid;
+                if (out.status) atomicAdd(out.status + 3, 1u);
+            }
+        }
+    }
+    if (lane == 0 && !defer) {
+        bool bad = first_bad <= S;
+        if (out.valid) out.valid[0] = bad ? first_bad - 1 : S;
+        if (out.status) {
+            if (bad) atomicAdd(out.status + 0, 1u);
+            if (nonfinite) atomicAdd(out.status + 1, (uint32_t)nonfinite);
+        }
+    }
+}
+
+// The refined pass of one ray by one warp (buf: kSegPad floats, dbuf: kSegPad
+// float pairs of shared memory; line64: the ray's FP64 line; rinfo: what the
+// FP32 pass recorded).  It redoes the first segments of the ray with one
+// iterative-refinement pass of the depth recurrence b_{i+1} = b_i M_i,
+// D_{i+1} = D_i delta_i: the FP32 states are kept, their residuals
+// rho_{i+1} = b_i M*_i - b_{i+1} are computed in double-single precision
+// (about 47 bits, ff.cuh) with M*_i the coefficients of double-single samples
+// at the FP64 line's positions (sample_z_ff), the error recurrence
+// e_{i+1} = e_i M_i + rho_{i+1} (e_0 = 0) of e_i = b*_i - b_i (b* the states
+// of the exact coefficients) is solved in FP32 with the same scan (affine
+// maps), and the echoes use the corrected states b_i + e_i and the refined
+// coefficient x*_i.  It covers rinfo.x segments, and goes on while the FP32
+// pass saw a pole there that the refined states do not confirm; rows beyond
+// keep the FP32 pass's values.
+template <typename T, bool STREAM>
+__device__ void march_refine_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg, const RayOut &out,
+                                 float *__restrict__ buf, float2 *__restrict__ dbuf, const RayLine64 &line64,
+                                 int2 rinfo)
+{
+    const int lane = threadIdx.x & 31;
+    const int S = rg.S;
+    const uint32_t pose = A.sp.pose_ctr + (uint32_t)rg.pose;
+    const int nseg = (S + kSeg - 1) / kSeg;
+
+    float czr, cdz, cor0[8];
+    sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz, nullptr, cor0);
+    const RayLineFF line_f = line_ff(line64);
+    FF czf = sample_z_ff(cor0, A.g, rg.X0[0], rg.X0[1], rg.X0[2], line_f.x0[0], line_f.x0[1], line_f.x0[2]);
+    const FF a2f = ff_from_double(A.a2d);
+    float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;   // bottom row and det at segment start
+    int first_bad = 0x7fffffff;
+    int nonfinite = 0;
+    float es0 = 0.0f, es1 = 0.0f, esD = 0.0f;  // correction at segment start
+    // segments to redo; extended while the FP32 pass's pole lies
+    // before the end and the refined states have not found one
+    const bool fp32_pole = rinfo.y <= S;
+    int seg = 0;
+    for (; seg < nseg; seg++) {
+        if (seg >= rinfo.x) {
+            const bool pole_seen = __shfl_sync(0xffffffffu, first_bad, 0) <= S;   // lane 0 holds the reduced value
+            if (!(fp32_pole && !pole_seen)) break;
+        }
+        const int base = seg * kSeg;
+        if (out.ckpt && lane == 0) out.ckpt[seg] = make_float4(bs0 + es0, bs1 + es1, Ds + esD, 0.0f);
+        seg_reflections_ff<T>(vol, A.g, rg, base, czr, cdz, buf, dbuf, line_f, czf);
+        __syncwarp();
+        const int i0 = base + lane * kChunk;
+        float rr[kChunk];
+#pragma unroll
+        for (int t = 0; t < kChunk; t++) rr[t] = buf[smem_idx(lane * kChunk + t)];
+        Mat2 Q, E, Qall;
+        float dq, de, dall;
+        chunk_product_ref(rr, i0, S, A.a2, A.mode, Q, dq);
+        warp_scan_prefix(Q, dq, E, de, Qall, dall);
+        float b0 = fmaf(bs0, E.a, bs1 * E.c);
+        float b1 = fmaf(bs0, E.b, bs1 * E.d);
+        float D = Ds * de;
+        {
+            float n0 = fmaf(bs0, Qall.a, bs1 * Qall.c);
+            float n1 = fmaf(bs0, Qall.b, bs1 * Qall.d);
+            bs0 = n0;
+            bs1 = n1;
+            Ds *= dall;
+        }
+        float m[kChunk];
+        if (A.sp.on) {
             chunk_speckle(A.sp, i0, S, rg.ray, pose, m);
         } else {
 #pragma unroll
             for (int t = 0; t < kChunk; t++) m[t] = 1.0f;
         }
-        if (!REFINE && out.mrow) {
-#pragma unroll
-            for (int t = 0; t < kChunk; t++)
-                if (i0 + t < S) __stcs(out.mrow + i0 + t, m[t]);
-        }
         float y[kChunk];
-        if (!REFINE) {
-            // TRACK: the FP32 pass of a refined render also finds the last
-            // row whose conditioning needs the refined states
-            auto echoes = [&](auto track) {
-                constexpr bool TRACK = decltype(track)::value;
-#pragma unroll
-                for (int t = 0; t < kChunk; t++) {
-                    const int i = i0 + t;
-                    y[t] = 0.0f;
-                    if (i < S) {
-                        Xfer x = xfer(rr[t], A.a2, A.mode);
-                        float q = fmaf(b0, x.m01, b1);          // det(A_{i+1})
-                        float e = x.m01 * D * frcp(b1 * q);
-                        if (!(q >= kPoleEps)) first_bad = min(first_bad, i + 1);
-                        if (TRACK && fminf(b1, q) < need_md) last_need = i;
-                        float nb0 = fmaf(b0, x.m00, b1 * x.m10);
-                        b1 = q;
-                        b0 = nb0;
-                        D *= x.delta;
-                        y[t] = m[t] * e;
-                        nonfinite += !isfinite(y[t]);
-                    }
-                }
-            };
-            if (out.rinfo)
-                echoes(std::true_type{});
-            else
-                echoes(std::false_type{});
-        } else {
+        {
             // FP32 states b_i, D_i of the chunk as the unrefined path computes them
             float sb0[kChunk + 1], sb1[kChunk + 1], sD[kChunk + 1];
             sb0[0] = b0;
@@ -525,64 +726,24 @@ __device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
                 }
             }
         }
-        if (vec4 && i0 + kChunk <= S) {
-            // STREAM (the batched kernel: gigabytes of one-pass rows):
-            // evict-first; ordinary stores for small single-pose rows
-            float4 *dst = reinterpret_cast<float4 *>(out.row + i0);
-            if (STREAM) {
-                __stcs(dst, make_float4(y[0], y[1], y[2], y[3]));
-                __stcs(dst + 1, make_float4(y[4], y[5], y[6], y[7]));
-            } else {
-                dst[0] = make_float4(y[0], y[1], y[2], y[3]);
-                dst[1] = make_float4(y[4], y[5], y[6], y[7]);
-            }
-        } else {
+        if (i0 < S) store_rows<STREAM>(out, i0, S, y);
+        // the pole decision so far, for the loop's stopping rule
 #pragma unroll
-            for (int t = 0; t < kChunk; t++)
-                if (i0 + t < S) {
-                    if (STREAM)
-                        __stcs(out.row + i0 + t, y[t]);
-                    else
-                        out.row[i0 + t] = y[t];
-                }
-        }
-        if (REFINE) {   // the pole decision so far, for the loop's stopping rule
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1)
-                first_bad = min(first_bad, __shfl_xor_sync(0xffffffffu, first_bad, off));
-        }
+        for (int off = 16; off > 0; off >>= 1)
+            first_bad = min(first_bad, __shfl_xor_sync(0xffffffffu, first_bad, off));
         __syncwarp();
     }
-    if (REFINE) {
-        // the carry of the first segment the refined pass left alone, so the
-        // adjoint starts from corrected states there too; then the FP32
-        // pass's rows beyond, counted for non-finite values
-        if (seg < nseg && out.ckpt && lane == 0) out.ckpt[seg] = make_float4(bs0 + es0, bs1 + es1, Ds + esD, 0.0f);
-        for (int i = seg * kSeg + lane; i < S; i += kWarp) nonfinite += !isfinite(out.row[i]);
-    }
-
+    // the carry of the first segment the refined pass left alone, so the
+    // adjoint starts from corrected states there too; then the FP32 pass's
+    // rows beyond, counted for non-finite values
+    if (seg < nseg && out.ckpt && lane == 0) out.ckpt[seg] = make_float4(bs0 + es0, bs1 + es1, Ds + esD, 0.0f);
+    for (int i = seg * kSeg + lane; i < S; i += kWarp) nonfinite += !isfinite(out.row[i]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         first_bad = min(first_bad, __shfl_xor_sync(0xffffffffu, first_bad, off));
         nonfinite += __shfl_xor_sync(0xffffffffu, nonfinite, off);
-        if (!REFINE) last_need = max(last_need, __shfl_xor_sync(0xffffffffu, last_need, off));
     }
-    bool defer = false;     // FP32 pass of a ray that the refined pass redoes
-    if (!REFINE && out.rinfo) {
-        // rows up to the pole's (which the refined pass decides again), or
-        // up to the last row whose conditioning needs the refined states
-        const int cover = first_bad <= S ? first_bad - 1 : last_need;
-        const int segs = cover >= 0 ? cover / kSeg + 1 : 0;
-        defer = segs > 0;
-        if (lane == 0) {
-            out.rinfo[0] = make_int2(segs, first_bad <= S ? first_bad : S + 1);
-            if (defer) {
-                out.rlist[atomicAdd(out.rcount, 1u)] = out.rid;
-                if (out.status) atomicAdd(out.status + 3, 1u);
-            }
-        }
-    }
-    if (lane == 0 && !defer) {
+    if (lane == 0) {
         bool bad = first_bad <= S;
         if (out.valid) out.valid[0] = bad ? first_bad - 1 : S;
         if (out.status) {

@@ -22,10 +22,11 @@ namespace dfs {
 
 constexpr int kBwdPad = 289;   // smem_idx(256) + 1
 
-template <bool POSE>
+template <bool POSE, bool STORED = false>
 struct BwdSmem {
-    float zr[kBwdPad], dz[kBwdPad];   // samples base .. base+256 (zref + dz form; STORED: zref + dz, r before)
+    static constexpr int kZ = STORED ? 1 : kBwdPad;
     float4 eg[kSeg];                  // echo partials of interface lane*8+t at [t*32 + lane] (both reverse passes)
+    float zr[kZ], dz[kZ];             // samples base .. base+256 (zref + dz form; not STORED)
     float gx[POSE ? kBwdPad : 1], gy[POSE ? kBwdPad : 1], gz[POSE ? kBwdPad : 1];   // dZ/dp (POSE)
     double acc[POSE ? 6 : 1];         // the ray's pose-gradient sums (lane 0)
 };
@@ -55,31 +56,33 @@ __device__ __forceinline__ EchoGrad echo_grad(float b0, float b1, float D, float
 // mrow: speckle factors written by the forward of the same call (nullable;
 // recomputed from Philox when absent).
 // STORED (requires have_ckpt, not POSE): the forward of the same call kept,
-// per sample k, (zref + dz, r_{k-1}) in krow, so the march reads them instead
-// of resampling the volume (the same values bit for bit).
-template <typename T, bool POSE, bool STORED = false>
+// per sample k, zref + dz in zrow and r_{k-1} in rrow, so the march reads them
+// instead of resampling the volume (the same values bit for bit), each lane
+// its own chunk in 16-byte loads.
+// gy_vec: gy_row is an internal row (aligned, row_stride long); mrow always is.
+// gz_row, zrow and rrow lie kGzLead floats into an aligned block of
+// gz_stride(S).  Only the gather reads dL/dZ, so POSE (which runs without one)
+// does not write it.
+//
+// Past the ray's end r and the adjoint sources are 0, so the passes need no
+// row tests; only the Z1-role term of interface S, which would reach sample
+// S, is dropped explicitly.
+template <typename T, int MODE, bool POSE, bool STORED = false>
 __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg,
                               const float *__restrict__ gy_row, float *__restrict__ gz_row,
-                              double *__restrict__ pose_part, float4 *__restrict__ ckpt, BwdSmem<POSE> &sm,
-                              bool have_ckpt = false, const float *__restrict__ mrow = nullptr,
-                              const float2 *__restrict__ krow = nullptr)
+                              double *__restrict__ pose_part, float4 *__restrict__ ckpt, BwdSmem<POSE, STORED> &sm,
+                              bool gy_vec, bool have_ckpt = false, const float *__restrict__ mrow = nullptr,
+                              const float *__restrict__ zrow = nullptr, const float *__restrict__ rrow = nullptr)
 {
     static_assert(!(STORED && POSE), "the pose terms of the march need the sampled gradient");
     // The batched call (STORED) streams gigabytes of one-pass rows: evict-
     // first loads and stores keep them from displacing reused L2 lines.  The
     // small single-pose rows stay ordinary.
     auto ld_once = [](const float *p) { return STORED ? __ldcs(p) : __ldg(p); };
-    auto st_once = [](float *p, float v) {
-        if (STORED)
-            __stcs(p, v);
-        else
-            *p = v;
-    };
     const int lane = threadIdx.x & 31;
     const int S = rg.S;
-    const uint32_t pose = A.sp.pose_ctr + (uint32_t)rg.pose;
+    const float a2 = A.a2;
     const int nseg = (S + kSeg - 1) / kSeg;
-    float *buf = sm.zr;   // sweep 1 uses the first array for reflection coefficients
 
     // ---------------- sweep 1: forward, record the carry at segment starts
     if (!STORED && !have_ckpt) {
@@ -87,23 +90,19 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
         sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz);
         float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;
         for (int s = 0; s < nseg; s++) {
-            const int base = s * kSeg;
             if (lane == 0) ckpt[s] = make_float4(bs0, bs1, Ds, 0.0f);
-            seg_reflections<T>(vol, A.g, rg, base, czr, cdz, buf);
-            __syncwarp();
             float rr[kChunk];
-#pragma unroll
-            for (int t = 0; t < kChunk; t++) rr[t] = buf[smem_idx(lane * kChunk + t)];
+            seg_coefficients<T, false>(vol, A.g, rg, s * kSeg, czr, cdz, reinterpret_cast<float2 *>(sm.eg), nullptr,
+                                       rr);
             Mat2 Q, E, Qall;
             float dq, de, dall;
-            chunk_product(rr, base + lane * kChunk, S, A.a2, A.mode, Q, dq);
+            chunk_product<MODE>(rr, a2, Q, dq);
             warp_scan_prefix(Q, dq, E, de, Qall, dall);
             float n0 = fmaf(bs0, Qall.a, bs1 * Qall.c);
             float n1 = fmaf(bs0, Qall.b, bs1 * Qall.d);
             bs0 = n0;
             bs1 = n1;
             Ds *= dall;
-            __syncwarp();
         }
     }
     __syncwarp();
@@ -119,74 +118,79 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
 
     for (int s = nseg - 1; s >= 0; s--) {
         const int base = s * kSeg;
-        // A': samples base .. base+255 (with dZ/dp when POSE); sample base+256 carried
-        long long X, Y, Z;
-        sample_pos(rg, base + lane, X, Y, Z);
-        const long long sX = rg.DX[0] * kWarp, sY = rg.DX[1] * kWarp, sZ = rg.DX[2] * kWarp;
-#pragma unroll
-        for (int t = 0; t < kChunk; t++) {
-            int p = t * kWarp + lane;
-            int k = base + p;
-            float zr = 0.0f, dz = 0.0f, g3[3] = {0.0f, 0.0f, 0.0f};
-            if (k <= S) {
-                if (STORED) {   // zr <- the sample's impedance, dz <- r of the interface before it
-                    const float2 kv = __ldcs(krow + k);
-                    zr = kv.x;
-                    dz = kv.y;
-                } else if (POSE) {
-                    sample_z<T, true>(vol, A.g, X, Y, Z, zr, dz, g3);
-                } else {
-                    sample_z<T, false>(vol, A.g, X, Y, Z, zr, dz);
-                }
-            }
-            X += sX;
-            Y += sY;
-            Z += sZ;
-            int o = smem_idx(p);
-            sm.zr[o] = zr; sm.dz[o] = dz;
-            if (POSE) { sm.gx[o] = g3[0]; sm.gy[o] = g3[1]; sm.gz[o] = g3[2]; }
-        }
-        if (lane == 0) {
-            if (s == nseg - 1 && base + kSeg <= S) {
-                long long X, Y, Z;
-                float g3[3];
-                sample_pos(rg, base + kSeg, X, Y, Z);
-                if (STORED) {
-                    const float2 kv = __ldcs(krow + base + kSeg);
-                    czr = kv.x;
-                    cdz = kv.y;
-                } else if (POSE) {
-                    sample_z<T, true>(vol, A.g, X, Y, Z, czr, cdz, g3);
-                    cg0 = g3[0]; cg1 = g3[1]; cg2 = g3[2];
-                } else {
-                    sample_z<T, false>(vol, A.g, X, Y, Z, czr, cdz);
-                }
-            }
-            int o = smem_idx(kSeg);
-            sm.zr[o] = czr; sm.dz[o] = cdz;
-            if (POSE) { sm.gx[o] = cg0; sm.gy[o] = cg1; sm.gz[o] = cg2; }
-        }
-        __syncwarp();
-        {   // carry the first sample of this segment to the earlier one
-            int o = smem_idx(0);
-            czr = sm.zr[o]; cdz = sm.dz[o];
-            if (POSE) { cg0 = sm.gx[o]; cg1 = sm.gy[o]; cg2 = sm.gz[o]; }
-        }
-
-        // B': reflection coefficients of this lane's chunk and the forward scan
         const int i0 = base + lane * kChunk;
         float rr[kChunk];
+        if (STORED) {
+            load_chunk(rrow + i0 + 1, i0 < S, rr);   // r_{i0+t} is kept with sample i0+t+1, 0 past the ray
+        } else {
+            // A': samples base .. base+255 (with dZ/dp when POSE); sample base+256 carried
+            long long X, Y, Z;
+            sample_pos(rg, base + lane, X, Y, Z);
+            const long long sX = rg.DX[0] * kWarp, sY = rg.DX[1] * kWarp, sZ = rg.DX[2] * kWarp;
+            constexpr int kGroup = POSE ? 1 : kSampleGroup;
 #pragma unroll
-        for (int t = 0; t < kChunk; t++) {
-            int o = smem_idx(lane * kChunk + t), o1 = smem_idx(lane * kChunk + t + 1);
-            if (STORED)   // r_{i0+t} is kept with sample i0+t+1
-                rr[t] = (i0 + t < S) ? sm.dz[o1] : 0.0f;
-            else
+            for (int t0 = 0; t0 < kChunk; t0 += kGroup) {
+                if (base + t0 * kWarp <= S) {   // past the ray a lane samples at a clamped position
+#pragma unroll
+                    for (int t = t0; t < t0 + kGroup; t++) {
+                        float zr, dz, g3[3];
+                        sample_z<T, POSE>(vol, A.g, X, Y, Z, zr, dz, g3);
+                        X += sX;
+                        Y += sY;
+                        Z += sZ;
+                        int o = smem_idx(t * kWarp + lane);
+                        sm.zr[o] = zr; sm.dz[o] = dz;
+                        if (POSE) { sm.gx[o] = g3[0]; sm.gy[o] = g3[1]; sm.gz[o] = g3[2]; }
+                    }
+                }
+            }
+            if (lane == 0) {
+                if (s == nseg - 1 && base + kSeg <= S) {
+                    float g3[3];
+                    sample_pos(rg, base + kSeg, X, Y, Z);
+                    sample_z<T, POSE>(vol, A.g, X, Y, Z, czr, cdz, g3);
+                    if (POSE) { cg0 = g3[0]; cg1 = g3[1]; cg2 = g3[2]; }
+                }
+                int o = smem_idx(kSeg);
+                sm.zr[o] = czr; sm.dz[o] = cdz;
+                if (POSE) { sm.gx[o] = cg0; sm.gy[o] = cg1; sm.gz[o] = cg2; }
+            }
+            __syncwarp();
+            {   // carry the first sample of this segment to the earlier one
+                int o = smem_idx(0);
+                czr = sm.zr[o]; cdz = sm.dz[o];
+                if (POSE) { cg0 = sm.gx[o]; cg1 = sm.gy[o]; cg2 = sm.gz[o]; }
+            }
+#pragma unroll
+            for (int t = 0; t < kChunk; t++) {
+                int o = smem_idx(lane * kChunk + t), o1 = smem_idx(lane * kChunk + t + 1);
                 rr[t] = (i0 + t < S) ? refl(sm.zr[o], sm.dz[o], sm.zr[o1], sm.dz[o1]) : 0.0f;
+            }
         }
+        // adjoint sources of the echo rows
+        float m[kChunk];
+        if (mrow) {
+            load_chunk(mrow + i0, i0 < S, m);
+        } else if (!STORED && A.sp.on) {
+            chunk_speckle(A.sp, i0, S, rg.ray, A.sp.pose_ctr + (uint32_t)rg.pose, m);
+        } else {
+#pragma unroll
+            for (int t = 0; t < kChunk; t++) m[t] = 1.0f;
+        }
+        float ge[kChunk];
+        if (gy_vec) {
+            load_chunk(gy_row + i0, i0 < S, ge);
+        } else {
+#pragma unroll
+            for (int t = 0; t < kChunk; t++) ge[t] = (i0 + t < S) ? ld_once(gy_row + i0 + t) : 0.0f;
+        }
+#pragma unroll
+        for (int t = 0; t < kChunk; t++) ge[t] = (i0 + t < S) ? m[t] * ge[t] : 0.0f;
+
+        // B': the chunk's forward states
         Mat2 Q, E, Qall;
         float dq, de, dall;
-        chunk_product(rr, i0, S, A.a2, A.mode, Q, dq);
+        chunk_product<MODE>(rr, a2, Q, dq);
         warp_scan_prefix(Q, dq, E, de, Qall, dall);
         const float4 ck = ckpt[s];
         float b0s[kChunk], b1s[kChunk], Dsv[kChunk];
@@ -197,47 +201,35 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
 #pragma unroll
             for (int t = 0; t < kChunk; t++) {
                 b0s[t] = b0; b1s[t] = b1; Dsv[t] = D;
-                if (i0 + t < S) {
-                    Xfer x = xfer(rr[t], A.a2, A.mode);
-                    float nb0 = fmaf(b0, x.m00, b1 * x.m10);
-                    b1 = fmaf(b0, x.m01, b1);
-                    b0 = nb0;
-                    D *= x.delta;
-                }
+                const Xfer x = xfer_t<MODE>(rr[t], a2);
+                float nb0 = fmaf(b0, x.m00, b1 * x.m10);
+                b1 = fmaf(b0, x.m01, b1);
+                b0 = nb0;
+                D *= x.delta;
             }
         }
-        // adjoint sources of the echo rows
-        float m[kChunk];
-        if (mrow) {
-#pragma unroll
-            for (int t = 0; t < kChunk; t++) m[t] = (i0 + t < S) ? ld_once(mrow + i0 + t) : 1.0f;
-        } else if (A.sp.on) {
-            chunk_speckle(A.sp, i0, S, rg.ray, pose, m);
-        } else {
-#pragma unroll
-            for (int t = 0; t < kChunk; t++) m[t] = 1.0f;
-        }
-        float ge[kChunk];
-#pragma unroll
-        for (int t = 0; t < kChunk; t++) ge[t] = (i0 + t < S) ? m[t] * ld_once(gy_row + i0 + t) : 0.0f;
 
         // C': local reverse pass with zero adjoint at the chunk end; the
         // echo partials are kept for the true pass
         float c0 = 0.0f, c1 = 0.0f, dloc = 0.0f;
 #pragma unroll
         for (int t = kChunk - 1; t >= 0; t--) {
-            if (i0 + t < S) {
-                Xfer x = xfer(rr[t], A.a2, A.mode);
-                EchoGrad g = echo_grad(b0s[t], b1s[t], Dsv[t], x.m01, ge[t]);
-                sm.eg[t * kWarp + lane] = make_float4(g.gb0, g.gb1, g.gD, g.gx);
-                // explicit adds: the partials are not fused here either, as
-                // in the true pass, which reads them back
-                float n0 = __fadd_rn(g.gb0, fmaf(c0, x.m00, c1 * x.m01));
-                float n1 = __fadd_rn(g.gb1, fmaf(c0, x.m10, c1));
-                dloc = fmaf(dloc, x.delta, g.gD);
-                c0 = n0;
-                c1 = n1;
-            }
+            const Xfer x = xfer_t<MODE>(rr[t], a2);
+            EchoGrad g = echo_grad(b0s[t], b1s[t], Dsv[t], x.m01, ge[t]);
+            sm.eg[t * kWarp + lane] = make_float4(g.gb0, g.gb1, g.gD, g.gx);
+            // explicit adds: the partials are not fused here either, as
+            // in the true pass, which reads them back
+            float n0 = __fadd_rn(g.gb0, fmaf(c0, x.m00, c1 * x.m01));
+            float n1 = __fadd_rn(g.gb1, fmaf(c0, x.m10, c1));
+            dloc = fmaf(dloc, x.delta, g.gD);
+            c0 = n0;
+            c1 = n1;
+        }
+        // impedances of samples i0+1 .. i0+8 (and of i0), on their way during the scan
+        float zz[kChunk], z_first = 0.0f;
+        if (STORED) {
+            load_chunk(zrow + i0 + 1, i0 < S, zz);
+            if (lane == 0) z_first = __ldcs(zrow + base);
         }
         // D': warp suffix scan of the affine maps (lambda -> c + lambda Q^T, mu -> d + mu dq)
         Mat2 Pm = Q;          // chunk product (warp_scan_prefix took Q by value)
@@ -284,62 +276,66 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
         // dL/dZ of sample i0+t+1 (t < 7) is complete once interfaces t and
         // t+1 are done, so it is finalised inside the loop; sample i0+8 also
         // needs the next lane's interface and is finalised after it.
-        const float a2 = A.a2;
         float a[6] = {0, 0, 0, 0, 0, 0};
         float c_next = 0.0f;     // Z1-role contribution of interface t+1 to sample i0+t+1
         float n_last = 0.0f;     // Z2-role contribution of interface i0+7 to sample i0+8
         float c_first = 0.0f;    // Z1-role contribution of interface i0 to sample i0
-        auto add_pose = [&](int k, int o, float G) {
+        float G[kChunk];         // dL/dZ of samples i0+1 .. i0+8
+        auto add_pose = [&](int k, int o, float g) {
             if (!POSE) return;
             const float gx = sm.gx[o], gyv = sm.gy[o], gzv = sm.gz[o];
             const float sk = ((float)k + 0.5f) * ds;
-            a[0] = fmaf(G, gx, a[0]);
-            a[1] = fmaf(G, gyv, a[1]);
-            a[2] = fmaf(G, gzv, a[2]);
-            a[3] = fmaf(G * sk, gx, a[3]);
-            a[4] = fmaf(G * sk, gyv, a[4]);
-            a[5] = fmaf(G * sk, gzv, a[5]);
+            a[0] = fmaf(g, gx, a[0]);
+            a[1] = fmaf(g, gyv, a[1]);
+            a[2] = fmaf(g, gzv, a[2]);
+            a[3] = fmaf(g * sk, gx, a[3]);
+            a[4] = fmaf(g * sk, gyv, a[4]);
+            a[5] = fmaf(g * sk, gzv, a[5]);
         };
+        if (STORED) {
+            const float zl = __shfl_up_sync(0xffffffffu, zz[kChunk - 1], 1);
+            if (lane) z_first = zl;
+        }
 #pragma unroll
         for (int t = kChunk - 1; t >= 0; t--) {
-            float gzc = 0.0f, gzn = 0.0f;
-            if (i0 + t < S) {
-                const float r = rr[t];
-                Xfer x = xfer(r, a2, A.mode);
-                float gm00 = b0s[t] * le0, gm10 = b1s[t] * le0, gm01 = b0s[t] * le1;
-                float gdel = lmu * Dsv[t];
-                const float4 gv = sm.eg[t * kWarp + lane];   // written by this lane in C'
-                const EchoGrad g{gv.x, gv.y, gv.z, gv.w};
-                float gr;
-                if (A.mode == DIFFUS_MODE_LITERAL) {
-                    float R = fabsf(r);
-                    float gR = gm00 * (-4.0f * a2 * R) + (gm01 + g.gx) * a2 - gm10 + gdel * (-2.0f * a2 * R);
-                    gr = r > 0.0f ? gR : (r < 0.0f ? -gR : 0.0f);
-                } else {
-                    gr = (gm01 + g.gx) * a2 + gm10 + gdel * (-2.0f * a2 * r);
-                }
-                float n0 = g.gb0 + fmaf(le0, x.m00, le1 * x.m01);
-                float n1 = g.gb1 + fmaf(le0, x.m10, le1);
-                lmu = fmaf(lmu, x.delta, g.gD);
-                le0 = n0;
-                le1 = n1;
-                const int o1 = smem_idx(lane * kChunk + t), o2 = smem_idx(lane * kChunk + t + 1);
-                const float z1 = STORED ? sm.zr[o1] : sm.zr[o1] + sm.dz[o1];
-                const float z2 = STORED ? sm.zr[o2] : sm.zr[o2] + sm.dz[o2];
-                const float sz = z1 + z2;
-                const float is2 = frcp(sz * sz);
-                gzc = gr * (-2.0f * z2) * is2;
-                gzn = gr * (2.0f * z1) * is2;
+            const float r = rr[t];
+            const Xfer x = xfer_t<MODE>(r, a2);
+            float gm00 = b0s[t] * le0, gm10 = b1s[t] * le0, gm01 = b0s[t] * le1;
+            float gdel = lmu * Dsv[t];
+            const float4 gv = sm.eg[t * kWarp + lane];   // written by this lane in C'
+            const EchoGrad g{gv.x, gv.y, gv.z, gv.w};
+            float gr;
+            if (MODE == DIFFUS_MODE_LITERAL) {
+                float R = fabsf(r);
+                float gR = gm00 * (-4.0f * a2 * R) + (gm01 + g.gx) * a2 - gm10 + gdel * (-2.0f * a2 * R);
+                gr = r > 0.0f ? gR : (r < 0.0f ? -gR : 0.0f);
+            } else {
+                gr = (gm01 + g.gx) * a2 + gm10 + gdel * (-2.0f * a2 * r);
             }
+            float n0 = g.gb0 + fmaf(le0, x.m00, le1 * x.m01);
+            float n1 = g.gb1 + fmaf(le0, x.m10, le1);
+            lmu = fmaf(lmu, x.delta, g.gD);
+            le0 = n0;
+            le1 = n1;
+            float z1, z2;
+            if (STORED) {
+                z1 = t == 0 ? z_first : zz[t == 0 ? 0 : t - 1];
+                z2 = zz[t];
+            } else {
+                const int o1 = smem_idx(lane * kChunk + t), o2 = smem_idx(lane * kChunk + t + 1);
+                z1 = sm.zr[o1] + sm.dz[o1];
+                z2 = sm.zr[o2] + sm.dz[o2];
+            }
+            const float sz = z1 + z2;
+            const float is2 = frcp(sz * sz);
+            const float gzc = i0 + t < S ? gr * (-2.0f * z2) * is2 : 0.0f;
+            const float gzn = gr * (2.0f * z1) * is2;
             if (t == kChunk - 1) {
                 n_last = gzn;
             } else {
                 const int k = i0 + t + 1;
-                if (k <= S) {
-                    const float G = c_next + gzn;
-                    st_once(gz_row + k, G);
-                    add_pose(k, smem_idx(lane * kChunk + t + 1), G);
-                }
+                G[t] = c_next + gzn;
+                if (k <= S) add_pose(k, smem_idx(lane * kChunk + t + 1), G[t]);
             }
             c_next = gzc;
             if (t == 0) c_first = gzc;
@@ -354,14 +350,24 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
             float nextc = __shfl_down_sync(0xffffffffu, c_first, 1);
             if (lane == kWarp - 1) nextc = carry_gz1;
             const int k = i0 + kChunk;
-            if (k <= S) {
-                const float G = n_last + nextc;
-                st_once(gz_row + k, G);
-                add_pose(k, smem_idx(lane * kChunk + kChunk), G);
+            G[kChunk - 1] = n_last + nextc;
+            if (k <= S) add_pose(k, smem_idx(lane * kChunk + kChunk), G[kChunk - 1]);
+            if (!POSE && i0 < S) {
+                // samples i0+1 .. i0+8 lie on one aligned sector (samples past
+                // S fall into the block's padding)
+                float4 *dst = reinterpret_cast<float4 *>(gz_row + i0 + 1);
+                const float4 lo = make_float4(G[0], G[1], G[2], G[3]), hi = make_float4(G[4], G[5], G[6], G[7]);
+                if (STORED) {
+                    __stcs(dst, lo);
+                    __stcs(dst + 1, hi);
+                } else {
+                    dst[0] = lo;
+                    dst[1] = hi;
+                }
             }
         }
         if (s == 0 && lane == 0) {
-            st_once(gz_row, c_first);
+            if (!POSE) gz_row[0] = c_first;
             add_pose(0, smem_idx(0), c_first);
         }
         carry_gz1 = __shfl_sync(0xffffffffu, c_first, 0);

@@ -55,16 +55,20 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 // bcar: the forward's carries, (b0, b1, D) at rows 0, 16, 32, ... of every
 // ray, tile rays at tl.cb0 + lane * n_blocks(S).
-__device__ void march_bwd_tile(const MarchArgs &A, const TileDesc &tl, const float *__restrict__ gy,
+static __device__ void march_bwd_tile(const MarchArgs &A, const TileDesc &tl, const float *__restrict__ gy,
                                const float *__restrict__ mbuf, const float2 *__restrict__ kbuf,
-                               const float4 *__restrict__ bcar, float *__restrict__ gz, BwdTileSmem &sm)
+                               const float4 *__restrict__ bcar, float *__restrict__ gz, bool gy_padded,
+                               BwdTileSmem &sm)
 {
     const int lane = threadIdx.x & 31;
     const int S = tl.S, cnt = tl.cnt;
     const bool act = lane < cnt;
     const int nb = n_blocks(S);
     const float a2 = A.a2;
-    const int64_t kofs = tl.gz0 + (int64_t)(act ? lane : 0) * (S + 1);
+    const int ld = row_stride(S), ldz = gz_stride(S);
+    const int64_t gy0 = gy_padded ? tl.pad0 : tl.row0;
+    const int ldg = gy_padded ? ld : S;
+    const int64_t kofs = tl.gz0 + (int64_t)(act ? lane : 0) * ldz;
     float lam0 = 0.0f, lam1 = 0.0f, mu = 0.0f;   // adjoint of the state after the current interface
     float carry_c = 0.0f;                        // Z1-role term of interface i+1 for sample i+1
     const int e = lane & (kBlkRows - 1), h = lane >> 4;
@@ -76,10 +80,9 @@ __device__ void march_bwd_tile(const MarchArgs &A, const TileDesc &tl, const flo
         for (int t2 = 0; t2 < kWarp / 2; t2++) {
             const int rr = 2 * t2 + h;
             if (rr < cnt && e < n) {
-                const int64_t ro = tl.row0 + (int64_t)rr * S + i0 + e;
-                cp_async8(&sm.kp[st][rr * kBlkLd + e], kbuf + tl.gz0 + (int64_t)rr * (S + 1) + i0 + 1 + e);
-                cp_async4(&sm.gy[st][rr * kBlkLd + e], gy + ro);
-                if (mbuf) cp_async4(&sm.m[st][rr * kBlkLd + e], mbuf + ro);
+                cp_async8(&sm.kp[st][rr * kBlkLd + e], kbuf + tl.gz0 + (int64_t)rr * ldz + i0 + 1 + e);
+                cp_async4(&sm.gy[st][rr * kBlkLd + e], gy + gy0 + (int64_t)rr * ldg + i0 + e);
+                if (mbuf) cp_async4(&sm.m[st][rr * kBlkLd + e], mbuf + tl.pad0 + (int64_t)rr * ld + i0 + e);
             }
         }
         cp_async_commit();
@@ -157,7 +160,7 @@ __device__ void march_bwd_tile(const MarchArgs &A, const TileDesc &tl, const flo
 #pragma unroll 4
         for (int t2 = 0; t2 < kWarp / 2; t2++) {
             const int rr = 2 * t2 + h;
-            if (rr < cnt && e < n) __stcs(gz + tl.gz0 + (int64_t)rr * (S + 1) + i0 + 1 + e, gy_s[rr * kBlkLd + e]);
+            if (rr < cnt && e < n) __stcs(gz + tl.gz0 + (int64_t)rr * ldz + i0 + 1 + e, gy_s[rr * kBlkLd + e]);
         }
         __syncwarp();
     }

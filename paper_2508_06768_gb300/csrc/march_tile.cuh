@@ -26,10 +26,11 @@ constexpr int kTileWarps = 4;               // warps (tiles) per CTA
 
 // A tile of the batched forward (host-built, in the plan): rays j0 .. j0+cnt-1
 // of pose `pose`, whose global ray indices are rid0 .. rid0+cnt-1 and whose
-// rows, kept samples and scan carries start at row0, gz0 and ck0.
+// packed rows, internal rows (row_stride), samples (gz_stride) and scan
+// carries start at row0, pad0, gz0 and ck0.
 struct TileDesc {
     int32_t pose, j0, cnt, S;
-    int64_t row0, gz0, ck0, cb0;   // cb0: the rays' 16-row carries (backward), n_blocks(S) per ray
+    int64_t row0, pad0, gz0, ck0, cb0;   // cb0: the rays' 16-row carries (backward), n_blocks(S) per ray
     int32_t rid0, pad;
 };
 
@@ -59,7 +60,7 @@ __device__ void march_fwd_tile(const T *__restrict__ vol, const MarchArgs &A, co
                                const RayGeo *__restrict__ geo, float *__restrict__ out, int *__restrict__ valid,
                                uint32_t *__restrict__ status, float4 *__restrict__ ckpt, float *__restrict__ mbuf,
                                float2 *__restrict__ kbuf, float4 *__restrict__ bcar, const RefineSel &sel,
-                               TileSmem &sm)
+                               bool padded, TileSmem &sm)
 {
     const int lane = threadIdx.x & 31;
     const int S = tl.S, cnt = tl.cnt;
@@ -69,6 +70,9 @@ __device__ void march_fwd_tile(const T *__restrict__ vol, const MarchArgs &A, co
     const uint32_t pose = A.sp.pose_ctr + (uint32_t)tl.pose;
     const uint32_t ray = (uint32_t)(tl.j0 + lane);
     const int nseg = (S + kSeg - 1) / kSeg;
+    const int ld = row_stride(S), ldz = gz_stride(S);
+    const int64_t o0 = padded ? tl.pad0 : tl.row0;
+    const int ldo = padded ? ld : S;
     const bool spk = A.sp.on != 0;
     const bool keep = kbuf != nullptr, keep_m = mbuf != nullptr;
 
@@ -76,7 +80,7 @@ __device__ void march_fwd_tile(const T *__restrict__ vol, const MarchArgs &A, co
     const long long dX = rg.DX[0], dY = rg.DX[1], dZ = rg.DX[2];
     float pzr, pdz;
     sample_z<T, false>(vol, A.g, X, Y, Z, pzr, pdz);
-    if (keep && act) __stcs(kbuf + tl.gz0 + (int64_t)lane * (S + 1), make_float2(pzr + pdz, 0.0f));
+    if (keep && act) __stcs(kbuf + tl.gz0 + (int64_t)lane * ldz, make_float2(pzr + pdz, 0.0f));
     float b0 = 0.0f, b1 = 1.0f, D = 1.0f;
     int first_bad = 0x7fffffff, last_need = -1, nonfinite = 0;
     const float need_md = fmaxf(kNeedFloor, kNeedCoef * sqrtf((float)S));
@@ -177,10 +181,9 @@ __device__ void march_fwd_tile(const T *__restrict__ vol, const MarchArgs &A, co
         for (int t2 = 0; t2 < kWarp / 4; t2++) {
             const int rr = 4 * t2 + h;
             if (rr < cnt && e < nrow) {
-                const int64_t o = tl.row0 + (int64_t)rr * S + kb + e;
-                __stcs(out + o, sm.y[rr * kStageLd + e]);
-                if (keep_m) __stcs(mbuf + o, sm.m[rr * kStageLd + e]);
-                if (keep) __stcs(kbuf + tl.gz0 + (int64_t)rr * (S + 1) + kb + 1 + e, sm.k[rr * kStageLd + e]);
+                __stcs(out + o0 + (int64_t)rr * ldo + kb + e, sm.y[rr * kStageLd + e]);
+                if (keep_m) __stcs(mbuf + tl.pad0 + (int64_t)rr * ld + kb + e, sm.m[rr * kStageLd + e]);
+                if (keep) __stcs(kbuf + tl.gz0 + (int64_t)rr * ldz + kb + 1 + e, sm.k[rr * kStageLd + e]);
             }
         }
         __syncwarp();
@@ -235,14 +238,14 @@ struct SpkSmem {
 };
 
 // Speckle factors (Section 2.4) of rows k0 .. k0+63 of the tile's rays,
-// written to mbuf at the rays' image offsets.  The factors depend only on the
+// written to mbuf at the rays' internal rows.  The factors depend only on the
 // seed, the pose and ray indices, the row and S, never on the volume, so they
 // can be drawn before the march and read by it.  A lane runs its ray's rows
 // in order: the radial window from byte sums of Philox groups of four rows
 // (exact integer sums, as the march's own speckle), one grain normal per
 // grain cell, and the same factor arithmetic, so the factors equal the
 // march's bit for bit.
-__device__ void speckle_item(const Speckle &sp, const TileDesc &tl, int k0, float *__restrict__ mbuf, SpkSmem &sm)
+static __device__ void speckle_item(const Speckle &sp, const TileDesc &tl, int k0, float *__restrict__ mbuf, SpkSmem &sm)
 {
     const int lane = threadIdx.x & 31;
     const int S = tl.S, cnt = tl.cnt;
@@ -313,7 +316,7 @@ __device__ void speckle_item(const Speckle &sp, const TileDesc &tl, int k0, floa
     __syncwarp();
     // one ray's rows of the item per store instruction
     for (int rr = 0; rr < cnt; rr++) {
-        float *dst = mbuf + tl.row0 + (int64_t)rr * S + k0;
+        float *dst = mbuf + tl.pad0 + (int64_t)rr * row_stride(S) + k0;
         for (int e = lane; e < n; e += kWarp) __stcs(dst + e, sm.m[rr * kSpkLd + e]);
     }
     __syncwarp();

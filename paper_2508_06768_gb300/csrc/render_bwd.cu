@@ -9,14 +9,14 @@ using namespace dfs;
 
 namespace dfs {
 
-int launch_blur(const float *in, float *out, int n, int S, const diffus_params *prm, const diffus_fan *fan,
-                bool transpose, cudaStream_t s);
+int launch_blur(const float *in, float *out, int n, int S, int si, int so, const diffus_params *prm,
+                const diffus_fan *fan, bool transpose, cudaStream_t s);
 int check_common(const void *vol, const diffus_volume_desc *vd, const float *pose, const diffus_fan *fan,
                  const diffus_params *prm);
 
 constexpr int kWarpsBwd = 4;
 
-template <typename T, bool POSE>
+template <typename T, bool POSE, int MODE>
 __global__ void __launch_bounds__(kWarpsBwd * 32) k_march_bwd(const T *__restrict__ vol, MarchArgs A,
                                                               const RayGeo *__restrict__ geo, int n_rays,
                                                               const float *__restrict__ gy,
@@ -25,15 +25,15 @@ __global__ void __launch_bounds__(kWarpsBwd * 32) k_march_bwd(const T *__restric
                                                               const long long *__restrict__ gz_off,
                                                               double *__restrict__ pose_part,
                                                               float4 *__restrict__ ckpt,
-                                                              const long long *__restrict__ ckpt_off)
+                                                              const long long *__restrict__ ckpt_off, bool gy_vec)
 {
     __shared__ BwdSmem<POSE> sm[kWarpsBwd];
     const int w = threadIdx.x >> 5;
     const int j = blockIdx.x * kWarpsBwd + w;
     if (j >= n_rays) return;
     RayGeo rg = geo[j];
-    march_bwd_ray<T, POSE>(vol, A, rg, gy + row_off[j], gz + gz_off[j], pose_part + 6 * (size_t)j, ckpt + ckpt_off[j],
-                     sm[w]);
+    march_bwd_ray<T, MODE, POSE>(vol, A, rg, gy + row_off[j], gz + gz_off[j], pose_part + 6 * (size_t)j, ckpt + ckpt_off[j],
+                           sm[w], gy_vec);
 }
 
 // Deterministic per-pose sum of per-ray pose partials: one warp per pose,
@@ -56,12 +56,13 @@ static __global__ void k_pose_reduce(const double *__restrict__ part, const int 
 }
 
 static __global__ void k_offsets(long long *__restrict__ row_off, long long *__restrict__ gz_off,
-                                 long long *__restrict__ ck_off, int *__restrict__ ray0, int n, int S)
+                                 long long *__restrict__ ck_off, int *__restrict__ ray0, int n, int S,
+                                 int row_ld)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n) {
-        row_off[j] = (long long)j * S;
-        gz_off[j] = (long long)j * (S + 1);
+        row_off[j] = (long long)j * row_ld;
+        gz_off[j] = (long long)j * gz_stride(S) + kGzLead;
         ck_off[j] = (long long)j * ((S + kSeg - 1) / kSeg);
     }
     if (j == 0) {
@@ -91,8 +92,8 @@ static BwdLayout bwd_layout(void *ws, const diffus_volume_desc *vd, const diffus
     size_t nseg = (S + kSeg - 1) / kSeg;
     L.geo = c.take<RayGeo>(n);
     L.frame = c.take<PoseFrame>(1);
-    L.gy = (prm->blur || prm->atten) ? c.take<float>(n * S) : nullptr;
-    L.gz = c.take<float>(n * (S + 1));
+    L.gy = (prm->blur || prm->atten) ? c.take<float>(n * row_stride((int)S)) : nullptr;
+    L.gz = c.take<float>(n * gz_stride((int)S));
     L.part = c.take<double>(6 * n);
     L.ckpt = c.take<float4>(n * nseg);
     L.row_off = c.take<long long>(n);
@@ -106,21 +107,25 @@ static BwdLayout bwd_layout(void *ws, const diffus_volume_desc *vd, const diffus
 
 template <typename T, bool POSE>
 static void launch_march_bwd_t(const void *vol, const MarchArgs &A, const BwdLayout &L, int n, const float *gy,
-                               int grid, cudaStream_t s)
+                               bool gy_vec, int grid, cudaStream_t s)
 {
-    k_march_bwd<T, POSE><<<grid, kWarpsBwd * 32, 0, s>>>((const T *)vol, A, L.geo, n, gy, L.row_off, L.gz, L.gz_off,
-                                                         L.part, L.ckpt, L.ck_off);
+    if (A.mode == DIFFUS_MODE_LITERAL)
+        k_march_bwd<T, POSE, DIFFUS_MODE_LITERAL><<<grid, kWarpsBwd * 32, 0, s>>>(
+            (const T *)vol, A, L.geo, n, gy, L.row_off, L.gz, L.gz_off, L.part, L.ckpt, L.ck_off, gy_vec);
+    else
+        k_march_bwd<T, POSE, DIFFUS_MODE_SIGNED><<<grid, kWarpsBwd * 32, 0, s>>>(
+            (const T *)vol, A, L.geo, n, gy, L.row_off, L.gz, L.gz_off, L.part, L.ckpt, L.ck_off, gy_vec);
 }
 
 static int launch_march_bwd(const void *vol, int dtype, bool pose, const MarchArgs &A, const BwdLayout &L, int n,
-                            const float *gy, int grid, cudaStream_t s)
+                            const float *gy, bool gy_vec, int grid, cudaStream_t s)
 {
     if (dtype == DIFFUS_F32) {
-        if (pose) launch_march_bwd_t<float, true>(vol, A, L, n, gy, grid, s);
-        else launch_march_bwd_t<float, false>(vol, A, L, n, gy, grid, s);
+        if (pose) launch_march_bwd_t<float, true>(vol, A, L, n, gy, gy_vec, grid, s);
+        else launch_march_bwd_t<float, false>(vol, A, L, n, gy, gy_vec, grid, s);
     } else {
-        if (pose) launch_march_bwd_t<unsigned short, true>(vol, A, L, n, gy, grid, s);
-        else launch_march_bwd_t<unsigned short, false>(vol, A, L, n, gy, grid, s);
+        if (pose) launch_march_bwd_t<unsigned short, true>(vol, A, L, n, gy, gy_vec, grid, s);
+        else launch_march_bwd_t<unsigned short, false>(vol, A, L, n, gy, gy_vec, grid, s);
     }
     return launch_status();
 }
@@ -153,10 +158,11 @@ extern "C" int diffus_render_bwd(const void *vol, const diffus_volume_desc *vd, 
     FanDev fd{n, S, fan->fov_rad, fan->depth_mm};
     k_pose_frames<<<1, 32, 0, s>>>(pose, 1, L.frame);
     k_ray_setup<<<(n + 127) / 128, 128, 0, s>>>(L.frame, fd, make_place(vd), L.geo);
-    k_offsets<<<(n + 127) / 128, 128, 0, s>>>(L.row_off, L.gz_off, L.ck_off, L.ray0, n, S);
+    k_offsets<<<(n + 127) / 128, 128, 0, s>>>(L.row_off, L.gz_off, L.ck_off, L.ray0, n, S,
+                                                  prm->blur ? row_stride(S) : S);
     const float *gy = grad_image;
     if (prm->blur) {
-        if ((rc = launch_blur(grad_image, L.gy, n, S, prm, fan, true, s))) return rc;
+        if ((rc = launch_blur(grad_image, L.gy, n, S, S, row_stride(S), prm, fan, true, s))) return rc;
         gy = L.gy;
     }
     if (prm->atten && !prm->blur) {   // the depth gain is its own adjoint (with blur it rides on the blur)
@@ -169,7 +175,7 @@ extern "C" int diffus_render_bwd(const void *vol, const diffus_volume_desc *vd, 
     MarchArgs A = make_march_args(vd, fan, prm);
     int grid = (n + kWarpsBwd - 1) / kWarpsBwd;
     const bool march_pose = grad_pose && !grad_vol;
-    if ((rc = launch_march_bwd(vol, vd->dtype, march_pose, A, L, n, gy, grid, s))) return rc;
+    if ((rc = launch_march_bwd(vol, vd->dtype, march_pose, A, L, n, gy, prm->blur != 0, grid, s))) return rc;
     if (grad_vol &&
         (rc = launch_gather(vd, vol, L.geo, n, fan->depth_mm, L.gz, L.gz_off, L.gather_ws, status, grad_vol,
                             grad_pose ? L.part : nullptr, 8, s)))

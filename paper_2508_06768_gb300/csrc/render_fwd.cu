@@ -83,23 +83,29 @@ int launch_fwd_march(const void *vol, const diffus_volume_desc *vd, const float 
     const bool refine = prm->refine && sel.rinfo;
     if (refine && cudaMemsetAsync(sel.rcount, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
     // the FP32 pass, then the refined pass over the rays it listed
-#define DFS_FWD(T)                                                                                               \
-    k_march_fwd<T><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, fan->n_rays, out, ray_valid, status, \
-                                                   refine ? sel : RefineSel{nullptr, nullptr, nullptr, nullptr}); \
-    if (refine)                                                                                                  \
-        k_march_refine<T><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, frame, fd, make_place(vd), out, \
-                                                          ray_valid, status, sel);
+#define DFS_FWD(T, MODE)                                                                                             \
+    if (refine) {                                                                                                    \
+        k_march_fwd<T, MODE, true><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, fan->n_rays, out,        \
+                                                                   ray_valid, status, sel);                         \
+        k_march_refine<T><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, frame, fd, make_place(vd), out,   \
+                                                          ray_valid, status, sel);                                  \
+    } else {                                                                                                         \
+        k_march_fwd<T, MODE, false><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, fan->n_rays, out,       \
+                                                                    ray_valid, status,                              \
+                                                                    RefineSel{nullptr, nullptr, nullptr, nullptr}); \
+    }
+    const bool literal = prm->mode == DIFFUS_MODE_LITERAL;
     if (vd->dtype == DIFFUS_F32) {
-        DFS_FWD(float)
+        if (literal) { DFS_FWD(float, DIFFUS_MODE_LITERAL) } else { DFS_FWD(float, DIFFUS_MODE_SIGNED) }
     } else {
-        DFS_FWD(unsigned short)
+        if (literal) { DFS_FWD(unsigned short, DIFFUS_MODE_LITERAL) } else { DFS_FWD(unsigned short, DIFFUS_MODE_SIGNED) }
     }
 #undef DFS_FWD
     return launch_status();
 }
 
-int launch_blur(const float *in, float *out, int n, int S, const diffus_params *prm, const diffus_fan *fan,
-                bool transpose, cudaStream_t s)
+int launch_blur(const float *in, float *out, int n, int S, int si, int so, const diffus_params *prm,
+                const diffus_fan *fan, bool transpose, cudaStream_t s)
 {
     BlurArgs b{(float)prm->sigma0, (float)prm->sigma1, blur_halfwidth(prm), prm->atten};
     float hi = 0.0f, lo = 0.0f;
@@ -108,9 +114,9 @@ int launch_blur(const float *in, float *out, int n, int S, const diffus_params *
     const dim3 grid((strips + kBlurWarps - 1) / kBlurWarps, (n + kBlurSegRays - 1) / kBlurSegRays);
 #define DFS_BLUR(WT)                                                        \
     if (transpose)                                                          \
-        k_blur<true, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, b, hi, lo); \
+        k_blur<true, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, si, so, b, hi, lo); \
     else                                                                    \
-        k_blur<false, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, b, hi, lo);
+        k_blur<false, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, si, so, b, hi, lo);
     switch (b.W) {
     case 0: DFS_BLUR(0) break;
     case 1: DFS_BLUR(1) break;
@@ -155,6 +161,7 @@ extern "C" int diffus_render_fwd(const void *vol, const diffus_volume_desc *vd, 
         k_row_gain<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(march_out, march_out, fan->n_rays, fan->n_samples, hi,
                                                                 lo);
     }
-    if (prm->blur) rc = launch_blur(L.y, image, fan->n_rays, fan->n_samples, prm, fan, false, s);
+    if (prm->blur) rc = launch_blur(L.y, image, fan->n_rays, fan->n_samples, fan->n_samples, fan->n_samples, prm, fan,
+                                  false, s);
     return rc;
 }
