@@ -10,7 +10,7 @@
 //             i * n_rays + r), are sorted by brick with a stable radix sort,
 //             so every brick's runs appear in slot order whatever the launch
 //             schedule.
-//  3. units:  each brick's runs are cut into units of at most kUnitRuns runs
+//  3. units:  each brick's runs are cut into units of at most unit_runs() runs
 //             (hot bricks crossed by many poses spread over many CTAs).
 //  4. gather: one warp per unit accumulates its samples into the 9^3 voxels
 //             the brick's cells touch, in a shared-memory copy of its own.
@@ -40,7 +40,17 @@ constexpr int kBrick = 8;
 constexpr int kBrickV = kBrick + 1;            // voxels touched by a brick's cells, per axis
 constexpr int kBrickVox = kBrickV * kBrickV * kBrickV;
 constexpr int kGatherWarps = 4;
-constexpr int kUnitRuns = 256;
+// Runs per unit.  A warp walks a unit's runs 32 at a time, so a unit of n
+// runs is n/32 run walks in series (about 20 us each); more units cost more
+// partials (729 floats each).  Large problems fill the GPU with units of 256;
+// below, units shrink to one run per lane, for as long as the slots (about
+// four per run) make no more units than twice the resident warps (152 x 28).
+// Measured with 256 and with 32: a 251-ray frame's unit kernel 182 and 43 us,
+// nine small frames' 132 and 45 us; 512 frames stay at 256.
+__host__ __device__ inline int unit_runs(size_t slots)
+{
+    return slots <= (1u << 20) ? 32 : slots <= (1u << 21) ? 64 : slots <= (1u << 22) ? 128 : 256;
+}
 
 struct GatherArgs {
     int nx, ny, nz;
