@@ -8,17 +8,17 @@ namespace dfs {
 namespace {
 
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;                  // items per thread per tile
+constexpr int kSortItems = 16;                 // items per thread per tile
 constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kScanChunk = 4096;
 
 // ------------------------------------------------------------------ runs
 
+// One thread per ray: many rays, or rays of more than kRunMax brick changes.
 __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__restrict__ gz_off, int n_rays,
-                           GatherArgs G, int cap, uint32_t sentinel,
-                           Run *__restrict__ runs, uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
-                           int *__restrict__ nrun, unsigned long long *__restrict__ brick_work,
-                           uint32_t *__restrict__ status)
+                           GatherArgs G, int cap, Run *__restrict__ runs, uint32_t *__restrict__ keys,
+                           int *__restrict__ nrun, uint32_t *__restrict__ bcount,
+                           unsigned long long *__restrict__ brick_work, uint32_t *__restrict__ status)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_rays) return;
@@ -54,15 +54,17 @@ __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__re
             const size_t slot = (size_t)cnt * n_rays + r;
             runs[slot] = run;
             keys[slot] = brick;
-            vals[slot] = (uint32_t)slot;
-            {   // for the unit order only: lanes on the same brick add once, through
-                // their lowest lane (integer sums, so the order does not matter)
+            {   // lanes on the same brick add once, through their lowest lane
+                // (integer sums, so the order does not matter)
                 const unsigned act = __activemask();
                 const unsigned grp = __match_any_sync(act, brick);
                 unsigned long long sum = 0;
                 for (unsigned m = grp; m; m &= m - 1)
                     sum += (unsigned long long)__shfl_sync(grp, run.len, __ffs(m) - 1);
-                if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) atomicAdd(brick_work + brick, sum);
+                if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) {
+                    atomicAdd(brick_work + brick, sum);
+                    atomicAdd(bcount + brick, (uint32_t)__popc(grp));
+                }
             }
             cnt++;
         } else if (status) {
@@ -79,12 +81,132 @@ __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__re
             }
         }
     }
-    for (int i = cnt; i < cap; i++) {
-        const size_t slot = (size_t)i * n_rays + r;
-        keys[slot] = sentinel;
-        vals[slot] = (uint32_t)slot;
-    }
     nrun[r] = cnt;
+}
+
+// The same runs with one warp per ray, for rays of at most kRunMax brick
+// changes.  The brick index of an axis is monotone along the ray, so its
+// changes can be found independently: lanes solve one crossing each, the three
+// axes' ordered lists are merged by rank, and equal crossings (a sample that
+// enters a new brick on two axes) become one.  One thread per ray walks up to
+// 80 dependent steps of 64-bit arithmetic, which is latency-bound for a frame
+// of a few hundred rays: 48 us for 251, 5.4 us here.  With many rays the walk
+// is hidden and its aggregated counter updates win: 147 K rays 160 us, 227 us
+// here; the two lines cross near kRunWarpRays rays.
+//
+// bcount receives the runs of each brick.  ARRIVE keeps each run's arrival
+// number in its brick (any order; ranked by slot afterwards), else brick_work
+// receives the samples of each brick for the unit order.
+constexpr int kRunWarps = 8;
+constexpr int kRunMax = 255;
+constexpr int kRunWarpRays = 50000;
+
+__device__ __forceinline__ int count_below(const int *k, int n, int v, bool or_equal)
+{
+    int lo = 0;
+    while (n > 0) {
+        const int h = n >> 1;
+        const int m = k[lo + h];
+        if (m < v || (or_equal && m == v)) {
+            lo += h + 1;
+            n -= h + 1;
+        } else {
+            n = h;
+        }
+    }
+    return lo;
+}
+
+template <bool ARRIVE>
+__global__ void __launch_bounds__(kRunWarps * 32)
+    k_ray_runs_warp(const RayGeo *__restrict__ geo, const long long *__restrict__ gz_off, int n_rays, GatherArgs G,
+                    int cap, Run *__restrict__ runs, uint32_t *__restrict__ keys, int *__restrict__ nrun,
+                    uint32_t *__restrict__ bcount, uint32_t *__restrict__ arrival,
+                    unsigned long long *__restrict__ brick_work, uint32_t *__restrict__ status)
+{
+    __shared__ int sk[kRunWarps][kRunMax + 1], sm[kRunWarps][kRunMax + 1];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int r = blockIdx.x * kRunWarps + w;
+    if (r >= n_rays) return;
+    const RayGeo rg = geo[r];
+    const int S = rg.S;
+    const int n[3] = {G.nx, G.ny, G.nz};
+    int b0[3], off[4];
+    off[0] = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        b0[a] = cell_of(rg.X0[a], n[a]) / kBrick;
+        const int b1 = cell_of(rg.X0[a] + (long long)S * rg.DX[a], n[a]) / kBrick;
+        off[a + 1] = off[a] + abs(b1 - b0[a]);
+    }
+    const int m = min(off[3], kRunMax);        // off[3] <= cap - 1 <= kRunMax
+    int *k = sk[w], *start = sm[w];
+    for (int e = lane; e < m; e += 32) {
+        const int a = e < off[1] ? 0 : (e < off[2] ? 1 : 2);
+        const int j = e - (a == 0 ? 0 : (a == 1 ? off[1] : off[2]));
+        const long long X0 = a == 0 ? rg.X0[0] : (a == 1 ? rg.X0[1] : rg.X0[2]);
+        const long long DX = a == 0 ? rg.DX[0] : (a == 1 ? rg.DX[1] : rg.DX[2]);
+        const int b = a == 0 ? b0[0] : (a == 1 ? b0[1] : b0[2]);
+        long long kk;
+        if (DX > 0)
+            kk = first_at_or_above(X0, DX, (long long)((b + j + 1) * kBrick) << 32, S);
+        else   // cell < 8c  <=>  -X >= -(8c << 32) + 1
+            kk = first_at_or_above(-X0, -DX, -((long long)((b - j) * kBrick) << 32) + 1, S);
+        k[e] = (int)kk;
+    }
+    __syncwarp();
+    int *order = start;                         // merged, with repeats
+    for (int e = lane; e < m; e += 32) {
+        const int a = e < off[1] ? 0 : (e < off[2] ? 1 : 2);
+        const int v = k[e];
+        int pos = e - (a == 0 ? 0 : (a == 1 ? off[1] : off[2]));
+        if (a != 0) pos += count_below(k, off[1], v, true);
+        if (a != 1) pos += count_below(k + off[1], off[2] - off[1], v, a == 2);
+        if (a != 2) pos += count_below(k + off[2], m - off[2], v, false);
+        order[pos] = v;
+    }
+    __syncwarp();
+    // distinct crossings: the first sample of every run after the first
+    int cnt = 1;
+    for (int e0 = 0; e0 < m; e0 += 32) {
+        const int e = e0 + lane;
+        const int v = e < m ? order[e] : 0;
+        const bool first = e < m && (e == 0 || order[e - 1] != v);
+        const unsigned bal = __ballot_sync(0xffffffffu, first);
+        if (first) k[cnt - 1 + __popc(bal & ((1u << lane) - 1u))] = v;   // k[i]: start of run i + 1
+        cnt += __popc(bal);
+    }
+    __syncwarp();
+    if (cnt > cap) {
+        if (status && lane == 0) atomicOr(status + 2, (uint32_t)DIFFUS_STATUS_QUEUE);
+        cnt = cap;
+    }
+    const long long go = gz_off[r];
+    for (int i = lane; i < cnt; i += 32) {
+        const int ka = i ? k[i - 1] : 0, kb = i + 1 < cnt ? k[i] : S + 1;
+        Run run;
+        run.X = rg.X0[0] + (long long)ka * rg.DX[0];
+        run.Y = rg.X0[1] + (long long)ka * rg.DX[1];
+        run.Z = rg.X0[2] + (long long)ka * rg.DX[2];
+        run.dX = rg.DX[0];
+        run.dY = rg.DX[1];
+        run.dZ = rg.DX[2];
+        run.g_off = go + ka;
+        run.len = kb - ka;
+        run.k0 = ka;
+        const uint32_t brick = (uint32_t)(((cell_of(run.Z, n[2]) / kBrick) * G.nby + cell_of(run.Y, n[1]) / kBrick) * G.nbx +
+                                          cell_of(run.X, n[0]) / kBrick);
+        const size_t slot = (size_t)i * n_rays + r;
+        runs[slot] = run;
+        keys[slot] = brick;
+        if (ARRIVE) {
+            arrival[slot] = atomicAdd(bcount + brick, 1u);
+        } else {
+            atomicAdd(bcount + brick, 1u);
+            atomicAdd(brick_work + brick, (unsigned long long)run.len);
+        }
+    }
+    if (lane == 0) nrun[r] = cnt;
 }
 
 // ------------------------------------------------------------ exclusive scan
@@ -162,16 +284,37 @@ __global__ void k_chunk_scan(const uint32_t *__restrict__ in, size_t n, const ui
 
 // ------------------------------------------------------- stable radix sort
 
-__global__ void k_digit_hist(const uint32_t *__restrict__ keys, size_t n, int shift, int nblk,
-                             uint32_t *__restrict__ hist)
+// The first pass reads the slots (n = all of them; kNoRun marks a slot without
+// a run) and drops the empty ones, about three in four; the later passes run
+// over the *n_used runs that are left.
+constexpr uint32_t kNoRun = 0xffffffffu;
+
+template <bool FIRST>
+__global__ void __launch_bounds__(kSortThreads) k_digit_hist(const uint32_t *__restrict__ keys, size_t slots,
+                                                             const uint32_t *__restrict__ n_used, int shift, int nblk,
+                                                             uint32_t *__restrict__ hist)
 {
     __shared__ uint32_t cnt[256];
+    const size_t n = FIRST ? slots : (size_t)*n_used;
     cnt[threadIdx.x] = 0;
     __syncthreads();
     const size_t b0 = (size_t)blockIdx.x * kSortTile;
-    for (int s = 0; s < kSortItems; s++) {
-        size_t i = b0 + (size_t)s * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 255u], 1u);   // integer counts: order-free
+    if (b0 < n) {
+        uint32_t key[kSortItems];
+#pragma unroll
+        for (int s = 0; s < kSortItems; s++) {
+            const size_t i = b0 + (size_t)s * kSortThreads + threadIdx.x;
+            key[s] = i < n ? keys[i] : kNoRun;
+        }
+#pragma unroll
+        for (int s = 0; s < kSortItems; s++) {
+            // neighbouring slots are the same run of neighbouring rays and
+            // mostly lie in one brick: one shared add per distinct digit
+            const uint32_t d = key[s] != kNoRun ? ((key[s] >> shift) & 255u) : 256u;
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            if (d < 256u && (peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0)
+                atomicAdd(&cnt[d], (uint32_t)__popc(peers));   // integer counts: order-free
+        }
     }
     __syncthreads();
     hist[(size_t)threadIdx.x * nblk + blockIdx.x] = cnt[threadIdx.x];
@@ -179,9 +322,11 @@ __global__ void k_digit_hist(const uint32_t *__restrict__ keys, size_t n, int sh
 
 // Stable scatter: an item's position is its digit's offset for this tile,
 // plus the items of the same digit earlier in the tile (earlier sub-tiles,
-// earlier warps, lower lanes).
+// earlier warps, lower lanes).  FIRST: the values are the slot numbers.
+template <bool FIRST>
 __global__ void __launch_bounds__(kSortThreads) k_digit_scatter(const uint32_t *__restrict__ kin,
-                                                                const uint32_t *__restrict__ vin, size_t n, int shift,
+                                                                const uint32_t *__restrict__ vin, size_t slots,
+                                                                const uint32_t *__restrict__ n_used, int shift,
                                                                 int nblk, const uint32_t *__restrict__ offs,
                                                                 uint32_t *__restrict__ kout,
                                                                 uint32_t *__restrict__ vout)
@@ -189,18 +334,21 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_scatter(const uint32_t *
     constexpr int W = kSortThreads / 32;
     __shared__ uint32_t run[256];
     __shared__ uint32_t wcnt[W][257];
+    const size_t n = FIRST ? slots : (size_t)*n_used;
+    const size_t b0 = (size_t)blockIdx.x * kSortTile;
+    if (b0 >= n) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     run[threadIdx.x] = offs[(size_t)threadIdx.x * nblk + blockIdx.x];
     for (int q = 0; q < W; q++) wcnt[q][threadIdx.x] = 0;
     if (threadIdx.x == 0)
         for (int q = 0; q < W; q++) wcnt[q][256] = 0;
     __syncthreads();
-    const size_t b0 = (size_t)blockIdx.x * kSortTile;
     for (int s = 0; s < kSortItems; s++) {
         const size_t i = b0 + (size_t)s * kSortThreads + threadIdx.x;
-        const bool valid = i < n;
-        const uint32_t key = valid ? kin[i] : 0u;
-        const uint32_t val = valid ? vin[i] : 0u;
+        const uint32_t key = i < n ? kin[i] : kNoRun;
+        const bool valid = key != kNoRun;
+        if (FIRST && !__syncthreads_or(valid)) continue;   // a stretch of empty slots
+        const uint32_t val = FIRST ? (uint32_t)i : (valid ? vin[i] : 0u);
         const uint32_t d = valid ? ((key >> shift) & 255u) : 256u;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const int wrank = __popc(peers & ((1u << lane) - 1u));
@@ -227,35 +375,115 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_scatter(const uint32_t *
 
 // --------------------------------------------------------------- units
 
-// brick -> [start, end) of its runs in the sorted order
-__global__ void k_brick_bounds(const uint32_t *__restrict__ keys, size_t n, uint32_t sentinel,
-                               uint32_t *__restrict__ bstart, uint32_t *__restrict__ bend)
+// Per brick, from its run count: its runs [bstart, bend) in sorted order and
+// its units ustart .. ustart + ucount - 1 (with the unit -> brick table).  A
+// block owns 1024 bricks and adds up the counts before its own by itself, so
+// the two prefix sums take one launch and no block waits for another; beyond
+// kPlanDirect bricks (a quarter of a MB of counts from L2 per block) it adds up
+// per-block sums that k_brick_sums wrote first.
+constexpr int kPlanThreads = 1024;
+constexpr int kPlanDirect = 65536;
+
+__device__ __forceinline__ unsigned long long block_sum2(unsigned long long v, unsigned long long *red)
 {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t k = keys[i];
-    if (k == sentinel) return;
-    if (i == 0 || keys[i - 1] != k) bstart[k] = (uint32_t)i;
-    if (i + 1 == n || keys[i + 1] != k) bend[k] = (uint32_t)(i + 1);
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    unsigned long long t = red[threadIdx.x & 31];
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    __syncthreads();
+    return t;
 }
 
-__global__ void k_unit_counts(const uint32_t *__restrict__ bstart, const uint32_t *__restrict__ bend, int nb,
-                              int unit, uint32_t *__restrict__ ucount)
+// Runs (high word) and units (low word) of a brick with c runs; unit is a
+// power of two.
+__device__ __forceinline__ unsigned long long runs_units(uint32_t c, int unit)
 {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    uint32_t c = bend[b] - bstart[b];
-    ucount[b] = (c + unit - 1) / unit;
+    return ((unsigned long long)c << 32) | ((c + (uint32_t)unit - 1) >> (31 - __clz(unit)));
 }
 
-// Unit -> brick table: brick b owns units ustart[b] .. ustart[b] + ucount[b] - 1.
-__global__ void k_unit_bricks(const uint32_t *__restrict__ ustart, const uint32_t *__restrict__ ucount, int nb,
-                              uint32_t *__restrict__ unit_brick)
+__global__ void __launch_bounds__(kPlanThreads)
+    k_brick_sums(const uint32_t *__restrict__ bcount, int nb, int unit, unsigned long long *__restrict__ sums)
 {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    const uint32_t u0 = ustart[b], c = ucount[b];
-    for (uint32_t i = 0; i < c; i++) unit_brick[u0 + i] = (uint32_t)b;
+    __shared__ unsigned long long red[32];
+    const int b = blockIdx.x * kPlanThreads + threadIdx.x;
+    const unsigned long long t = block_sum2(runs_units(b < nb ? bcount[b] : 0u, unit), red);
+    if (threadIdx.x == 0) sums[blockIdx.x] = t;
+}
+
+__global__ void __launch_bounds__(kPlanThreads)
+    k_brick_plan(const uint32_t *__restrict__ bcount, const unsigned long long *__restrict__ sums, int nb, int unit,
+                 uint32_t *__restrict__ bstart, uint32_t *__restrict__ bend, uint32_t *__restrict__ ucount,
+                 uint32_t *__restrict__ ustart, uint32_t *__restrict__ unit_brick, uint32_t *__restrict__ n_units,
+                 uint32_t *__restrict__ n_runs)
+{
+    __shared__ unsigned long long red[32], wsum[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int b0 = blockIdx.x * kPlanThreads, b = b0 + threadIdx.x;
+    unsigned long long before = 0;
+    if (sums) {
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += kPlanThreads) before += sums[i];
+    } else {
+        for (int i = threadIdx.x * 4; i < b0; i += kPlanThreads * 4) {
+            const uint4 c = *reinterpret_cast<const uint4 *>(bcount + i);
+            before += (runs_units(c.x, unit) + runs_units(c.y, unit)) + (runs_units(c.z, unit) + runs_units(c.w, unit));
+        }
+    }
+    before = block_sum2(before, red);
+    const uint32_t c = b < nb ? bcount[b] : 0u;
+    const unsigned long long v = runs_units(c, unit);
+    unsigned long long x = v;
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    unsigned long long base = before;
+    for (int q = 0; q < w; q++) base += wsum[q];
+    const unsigned long long ex = base + x - v;
+    if (b < nb) {
+        const uint32_t r0 = (uint32_t)(ex >> 32), u0 = (uint32_t)ex, nu = (uint32_t)v;
+        bstart[b] = r0;
+        bend[b] = r0 + c;
+        ustart[b] = u0;
+        ucount[b] = nu;
+        for (uint32_t i = 0; i < nu; i++) unit_brick[u0 + i] = (uint32_t)b;
+    }
+    if (b == nb - 1) {
+        *n_units = (uint32_t)(ex + v);
+        *n_runs = (uint32_t)((ex + v) >> 32);
+    }
+}
+
+// Small problems (a frame, a few frames) are sorted by place and rank instead
+// of the radix passes: every run goes to its arrival place in its brick's
+// range, then each counts the runs of its brick with a smaller slot.  The
+// result is the same order (by brick, then slot); the work is the sum of the
+// squared brick counts.  Grid y: run number along the ray.
+__global__ void k_place_runs(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ arrival,
+                             const int *__restrict__ nrun, int n_rays, const uint32_t *__restrict__ bstart,
+                             uint2 *__restrict__ list)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n_rays || (int)blockIdx.y >= nrun[r]) return;
+    const uint32_t slot = blockIdx.y * (uint32_t)n_rays + (uint32_t)r;
+    const uint32_t b = keys[slot];
+    list[bstart[b] + arrival[slot]] = make_uint2(slot, b);
+}
+
+__global__ void k_rank_runs(const uint2 *__restrict__ list, const uint32_t *__restrict__ n_runs,
+                            const uint32_t *__restrict__ bstart, const uint32_t *__restrict__ bend,
+                            uint32_t *__restrict__ sorted)
+{
+    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= *n_runs) return;
+    const uint2 me = list[p];
+    const uint32_t q0 = bstart[me.y], q1 = bend[me.y];
+    uint32_t rank = 0;
+#pragma unroll 8
+    for (uint32_t q = q0; q < q1; q++) rank += list[q].x < me.x;
+    sorted[q0 + rank] = me.x;
 }
 
 // Work class of each unit, one thread per unit: its share of its brick's
@@ -327,7 +555,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32)
         if (lane == 0) u = atomicAdd(queue, 1u);
         u = __shfl_sync(0xffffffffu, u, 0);
         if (u >= total) break;
-        u = order[u];   // longest-first
+        if (order) u = order[u];   // longest-first
         const int b = (int)unit_brick[u];
         const uint32_t part = u - ustart[b];
         const uint32_t r0 = bstart[b] + part * (uint32_t)unit;
@@ -499,9 +727,14 @@ __global__ void k_ray_pose(const float *__restrict__ rpart, size_t slots, const 
 int sort_bits(int nb)
 {
     int bits = 1;
-    while ((1u << bits) <= (uint32_t)nb) bits++;   // sentinel (2^bits - 1) > every brick id
+    while ((1u << bits) < (uint32_t)nb) bits++;
     return bits;
 }
+
+// Place and rank instead of the radix passes: up to 32 K slots (12 launches and
+// about 50 us less for a frame; ranking grows with the runs per brick), unless
+// a few bricks hold so many runs that ranking is dearer.
+bool sort_by_rank(size_t slots, size_t nb) { return slots <= 32768 && slots * slots <= nb << 26; }
 
 }  // namespace
 
@@ -532,11 +765,14 @@ int runs_per_ray(const diffus_volume_desc *vd, double max_path_mm)
 
 struct GatherLayout {
     Run *runs;
-    uint32_t *keys[2], *vals[2];
-    uint32_t *hist, *sums, *misc;   // misc: [0] units total, [1] scan total, [2] unit queue
+    uint32_t *keys[2], *vals[2];    // radix passes; by rank: keys[1] arrivals, vals[0..1] the placed list
+    uint32_t *hist, *sums, *misc;   // misc: [0] units total, [1] runs in use
     uint32_t *bstart, *bend, *ucount, *ustart, *unit_brick;
-    uint32_t *uclass, *uorder, *classes;   // unit work classes, the longest-first order, 32 class counters
-    unsigned long long *bwork;             // samples of each brick's runs
+    uint32_t *uclass, *uorder;             // unit work classes, the longest-first order
+    // zeroed by one memset: 64 counters (0..31 unit classes, 32 unit queue),
+    // runs of each brick, samples of each brick's runs
+    uint32_t *zero, *bcount;
+    unsigned long long *bwork, *bsums;
     float *upart;
     float *rpart;   // per-run pose-gradient sums, 6 x slots
     int *nrun;      // runs of each ray
@@ -552,13 +788,13 @@ static GatherLayout gather_layout(void *ws, const diffus_volume_desc *vd, long l
     size_t slots = (size_t)n_rays * cap;
     size_t nblk = (slots + kSortTile - 1) / kSortTile;
     size_t nhist = 256 * nblk;
-    size_t nsums = (std::max(nhist, nb) + kScanChunk - 1) / kScanChunk;
+    size_t nsums = (nhist + kScanChunk - 1) / kScanChunk;
     size_t max_units = slots / unit_runs(slots) + nb;
     L.runs = c.take<Run>(slots);
     L.keys[0] = c.take<uint32_t>(slots);
     L.keys[1] = c.take<uint32_t>(slots);
-    L.vals[0] = c.take<uint32_t>(slots);
-    L.vals[1] = c.take<uint32_t>(slots);
+    L.vals[0] = c.take<uint32_t>(2 * slots);
+    L.vals[1] = L.vals[0] ? L.vals[0] + slots : nullptr;
     L.hist = c.take<uint32_t>(nhist);
     L.sums = c.take<uint32_t>(nsums + 1);
     L.misc = c.take<uint32_t>(4);
@@ -569,8 +805,10 @@ static GatherLayout gather_layout(void *ws, const diffus_volume_desc *vd, long l
     L.unit_brick = c.take<uint32_t>(max_units);
     L.uclass = c.take<uint32_t>(max_units);
     L.uorder = c.take<uint32_t>(max_units);
-    L.classes = c.take<uint32_t>(32);
+    L.zero = c.take<uint32_t>(64);
+    L.bcount = c.take<uint32_t>(nb);
     L.bwork = c.take<unsigned long long>(nb);
+    L.bsums = c.take<unsigned long long>((nb + kPlanThreads - 1) / kPlanThreads);
     L.upart = c.take<float>(max_units * kBrickVox);
     L.rpart = c.take<float>(6 * slots);
     L.nrun = c.take<int>((size_t)n_rays);
@@ -592,12 +830,12 @@ static void launch_scan(const uint32_t *in, uint32_t *out, size_t n, uint32_t *s
 }
 
 template <typename T, bool POSE>
-static void launch_units(const float *gz, const GatherLayout &L, int cur, const GatherArgs &G, const void *vol,
+static void launch_units(const float *gz, const GatherLayout &L, const uint32_t *sorted, const uint32_t *order, const GatherArgs &G, const void *vol,
                          const PoseOut &po, int unit, int grid, cudaStream_t s)
 {
-    k_gather_units<T, POSE><<<grid, kGatherWarps * 32, 0, s>>>(gz, L.runs, L.vals[cur], L.bstart, L.bend, L.ustart,
-                                                             L.unit_brick, L.misc + 0, G, unit, L.upart, L.misc + 2,
-                                                             L.uorder, (const T *)vol, po);
+    k_gather_units<T, POSE><<<grid, kGatherWarps * 32, 0, s>>>(gz, L.runs, sorted, L.bstart, L.bend, L.ustart,
+                                                             L.unit_brick, L.misc + 0, G, unit, L.upart, L.zero + 32,
+                                                             order, (const T *)vol, po);
 }
 
 int launch_gather(const diffus_volume_desc *vd, const void *vol, const RayGeo *geo, long long n_rays,
@@ -610,47 +848,77 @@ int launch_gather(const diffus_volume_desc *vd, const void *vol, const RayGeo *g
     GatherLayout L = gather_layout(ws, vd, n_rays, cap);
     const size_t slots = (size_t)n_rays * cap;
     const int unit = unit_runs(slots);
-    const int bits = sort_bits(nb);
-    const uint32_t sentinel = (1u << bits) - 1u;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
 
-    if (cudaMemsetAsync(L.bwork, 0, sizeof(unsigned long long) * nb, s) != cudaSuccess) return DIFFUS_E_LAUNCH;
-    k_ray_runs<<<(unsigned)((n_rays + 127) / 128), 128, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, sentinel, L.runs,
-                                                               L.keys[0], L.vals[0], L.nrun, L.bwork, status);
-    // stable LSD radix sort by brick
-    const int nblk = (int)((slots + kSortTile - 1) / kSortTile);
-    int cur = 0;
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_digit_hist<<<nblk, kSortThreads, 0, s>>>(L.keys[cur], slots, shift, nblk, L.hist);
-        launch_scan(L.hist, L.hist, (size_t)256 * nblk, L.sums, L.misc + 1, s);
-        k_digit_scatter<<<nblk, kSortThreads, 0, s>>>(L.keys[cur], L.vals[cur], slots, shift, nblk, L.hist,
-                                                      L.keys[cur ^ 1], L.vals[cur ^ 1]);
-        cur ^= 1;
+    const bool by_rank = cap - 1 <= kRunMax && sort_by_rank(slots, (size_t)nb);
+    const size_t zbytes = (by_rank ? (char *)(L.bcount + nb) : (char *)(L.bwork + nb)) - (char *)L.zero;
+    if (cudaMemsetAsync(L.zero, 0, zbytes, s) != cudaSuccess) return DIFFUS_E_LAUNCH;
+    const int wgrid = (int)((n_rays + kRunWarps - 1) / kRunWarps);
+    const int pgrid = (nb + kPlanThreads - 1) / kPlanThreads;
+    const uint32_t *sorted, *order = nullptr;
+    auto brick_plan = [&] {
+        if (nb > kPlanDirect) k_brick_sums<<<pgrid, kPlanThreads, 0, s>>>(L.bcount, nb, unit, L.bsums);
+        k_brick_plan<<<pgrid, kPlanThreads, 0, s>>>(L.bcount, nb > kPlanDirect ? L.bsums : nullptr, nb, unit, L.bstart,
+                                                    L.bend, L.ucount, L.ustart, L.unit_brick, L.misc + 0, L.misc + 1);
+    };
+    if (by_rank) {
+        k_ray_runs_warp<true><<<wgrid, kRunWarps * 32, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs, L.keys[0],
+                                                              L.nrun, L.bcount, L.keys[1], nullptr, status);
+        brick_plan();
+        uint2 *list = reinterpret_cast<uint2 *>(L.vals[0]);
+        k_place_runs<<<dim3((unsigned)((n_rays + 127) / 128), (unsigned)cap), 128, 0, s>>>(
+            L.keys[0], L.keys[1], L.nrun, (int)n_rays, L.bstart, list);
+        // the ranked order replaces the arrivals, which the list has absorbed
+        k_rank_runs<<<(unsigned)((slots + 127) / 128), 128, 0, s>>>(list, L.misc + 1, L.bstart, L.bend, L.keys[1]);
+        sorted = L.keys[1];
+    } else {
+        if (cudaMemsetAsync(L.keys[0], 0xff, sizeof(uint32_t) * slots, s) != cudaSuccess) return DIFFUS_E_LAUNCH;
+        if (cap - 1 <= kRunMax && n_rays <= kRunWarpRays)
+            k_ray_runs_warp<false><<<wgrid, kRunWarps * 32, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs,
+                                                                   L.keys[0], L.nrun, L.bcount, nullptr, L.bwork,
+                                                                   status);
+        else
+            k_ray_runs<<<(unsigned)((n_rays + 127) / 128), 128, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs,
+                                                                       L.keys[0], L.nrun, L.bcount, L.bwork, status);
+        brick_plan();
+        // stable LSD radix sort by brick
+        const int bits = sort_bits(nb);
+        const int nblk = (int)((slots + kSortTile - 1) / kSortTile);
+        int cur = 0;
+        for (int shift = 0; shift < bits; shift += 8) {
+            if (shift == 0)
+                k_digit_hist<true><<<nblk, kSortThreads, 0, s>>>(L.keys[cur], slots, L.misc + 1, shift, nblk, L.hist);
+            else
+                k_digit_hist<false><<<nblk, kSortThreads, 0, s>>>(L.keys[cur], slots, L.misc + 1, shift, nblk, L.hist);
+            launch_scan(L.hist, L.hist, (size_t)256 * nblk, L.sums, nullptr, s);
+            if (shift == 0)
+                k_digit_scatter<true><<<nblk, kSortThreads, 0, s>>>(L.keys[cur], L.vals[cur], slots, L.misc + 1, shift,
+                                                                    nblk, L.hist, L.keys[cur ^ 1], L.vals[cur ^ 1]);
+            else
+                k_digit_scatter<false><<<nblk, kSortThreads, 0, s>>>(L.keys[cur], L.vals[cur], slots, L.misc + 1,
+                                                                     shift, nblk, L.hist, L.keys[cur ^ 1],
+                                                                     L.vals[cur ^ 1]);
+            cur ^= 1;
+        }
+        sorted = L.vals[cur];
+        // longest-first unit order (by classes of work), so that no long unit starts last
+        k_unit_work<<<sms, 256, 0, s>>>(L.bwork, L.bstart, L.bend, L.ustart, L.unit_brick, L.misc + 0, unit, L.uclass,
+                                        L.zero);
+        k_class_cursors<<<1, 32, 0, s>>>(L.zero);
+        k_unit_order<<<sms * 4, 256, 0, s>>>(L.uclass, L.misc + 0, L.zero, L.uorder);
+        order = L.uorder;
     }
-    if (cudaMemsetAsync(L.bstart, 0, sizeof(uint32_t) * nb, s) != cudaSuccess) return DIFFUS_E_LAUNCH;
-    if (cudaMemsetAsync(L.bend, 0, sizeof(uint32_t) * nb, s) != cudaSuccess) return DIFFUS_E_LAUNCH;
-    k_brick_bounds<<<(unsigned)((slots + 255) / 256), 256, 0, s>>>(L.keys[cur], slots, sentinel, L.bstart, L.bend);
-    k_unit_counts<<<(nb + 255) / 256, 256, 0, s>>>(L.bstart, L.bend, nb, unit, L.ucount);
-    launch_scan(L.ucount, L.ustart, (size_t)nb, L.sums, L.misc + 0, s);
-    k_unit_bricks<<<(nb + 255) / 256, 256, 0, s>>>(L.ustart, L.ucount, nb, L.unit_brick);
-    // longest-first unit order (by classes of work), so that no long unit starts last
-    if (cudaMemsetAsync(L.classes, 0, 32 * sizeof(uint32_t), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
-    k_unit_work<<<sms, 256, 0, s>>>(L.bwork, L.bstart, L.bend, L.ustart, L.unit_brick, L.misc + 0, unit, L.uclass,
-                                    L.classes);
-    k_class_cursors<<<1, 32, 0, s>>>(L.classes);
-    k_unit_order<<<sms * 4, 256, 0, s>>>(L.uclass, L.misc + 0, L.classes, L.uorder);
     record_mark(marks.units, marks.external, s);
-    if (cudaMemsetAsync(L.misc + 2, 0, sizeof(uint32_t), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
     const int grid = sms * ctas_per_sm;
     const PoseOut po{L.rpart, slots};
     if (!pose_part)
-        launch_units<float, false>(gz, L, cur, G, vol, po, unit, grid, s);
+        launch_units<float, false>(gz, L, sorted, order, G, vol, po, unit, grid, s);
     else if (vd->dtype == DIFFUS_F32)
-        launch_units<float, true>(gz, L, cur, G, vol, po, unit, grid, s);
+        launch_units<float, true>(gz, L, sorted, order, G, vol, po, unit, grid, s);
     else
-        launch_units<unsigned short, true>(gz, L, cur, G, vol, po, unit, grid, s);
+        launch_units<unsigned short, true>(gz, L, sorted, order, G, vol, po, unit, grid, s);
     record_mark(marks.reduce, marks.external, s);
     const bool rvec = vd->nx % kRedVox == 0 && (uintptr_t)grad_vol % 16 == 0;
     int rx = 4;
