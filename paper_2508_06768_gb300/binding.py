@@ -9,7 +9,10 @@ library is missing or no GPU is present the calls raise.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
+import struct
 import threading
 
 import numpy as np
@@ -19,6 +22,7 @@ from . import build as _build
 
 _lock = threading.Lock()
 _lib = None
+_node = None
 
 
 class VolumeDesc(C.Structure):
@@ -107,6 +111,27 @@ def load(build_if_missing: bool = True):
         return lib
 
 
+def load_node():
+    """Load the native autograd node of render() (a torch extension module
+    linked against libdiffus.so)."""
+    global _node
+    if _node is not None:
+        return _node
+    load()
+    with _lock:
+        if _node is None:
+            if not os.path.exists(_build.NODE):
+                _build.build()
+            spec = importlib.util.spec_from_file_location(
+                _build.NODE_NAME, _build.NODE, loader=importlib.machinery.ExtensionFileLoader(_build.NODE_NAME,
+                                                                                             _build.NODE))
+            mod = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(mod)
+            mod.set_error(DiffusError)
+            _node = mod
+    return _node
+
+
 def _check(rc: int, what: str):
     if rc != 0:
         msg = load().diffus_strerror(rc).decode()
@@ -137,6 +162,19 @@ def params_desc(p, pose_ctr: int = 0) -> ParamsDesc:
                       float(p.Ag), float(p.pg), int(p.Lr), int(p.gshift), int(p.blur),
                       int(getattr(p, "refine", 0)), float(p.sigma0), float(p.sigma1), int(pose_ctr) & 0xFFFFFFFF,
                       int(getattr(p, "atten", 0)))
+
+
+# spacing, origin, diffus_fan and diffus_params as the native node takes them
+_CALL = struct.Struct("@6d ii4d Qii4diiiiddIi")
+
+
+def pack_call(spacing, origin, f, p, pose_ctr: int = 0):
+    """The descriptors of one single-pose call as bytes, with the conversions
+    of fan_desc and params_desc; struct.error if a value does not fit as it is."""
+    return _CALL.pack(*spacing, *origin, f.n_rays, f.n_samples, f.fov, f.depth, f.f_mhz, f.alpha,
+                      int(p.seed) & (2**64 - 1), int(p.mode), int(p.speckle), p.Ar, p.pr, p.Ag, p.pg, int(p.Lr),
+                      int(p.gshift), int(p.blur), int(getattr(p, "refine", 0)), p.sigma0, p.sigma1,
+                      int(pose_ctr) & 0xFFFFFFFF, int(getattr(p, "atten", 0)))
 
 
 def _ptr(t):

@@ -1,14 +1,17 @@
 """User-facing API: differentiable rendering through the C ABI.
 
 ``render(volume, pose, fan, params)`` renders one pose and is differentiable
-with respect to the impedance volume and the 6-DoF pose (a
-``torch.autograd.Function`` whose backward calls ``diffus_render_bwd``).
+with respect to the impedance volume and the 6-DoF pose (an autograd node
+whose backward calls ``diffus_render_bwd``: native, csrc/torch_node.cpp, for
+plain CUDA tensors; the same in Python for everything else).
 ``BatchRenderer`` renders many poses with their own fans in persistent
 launches and can capture a whole forward+backward step in a CUDA graph.
 PyTorch supplies device memory and streams only; every step runs in
 libdiffus.so.
 """
 from __future__ import annotations
+
+import struct
 
 import numpy as np
 import torch
@@ -41,9 +44,30 @@ class _Render(torch.autograd.Function):
         return gv, gp, None, None, None, None, None
 
 
+_PLAIN = (torch.Tensor, torch.nn.Parameter)
+
+
+def _native_call(volume, pose, fan, params, spacing, origin, pose_ctr):
+    """The packed descriptors if the native node takes this call as the Python
+    function does: plain CUDA tensors outside of tracing and functorch
+    transforms (which the Python function refuses or traces), values that fit
+    the C descriptors.  None otherwise."""
+    if (type(volume) not in _PLAIN or type(pose) not in _PLAIN or not volume.is_cuda or pose.device != volume.device
+            or volume.dim() != 3 or volume.dtype not in (torch.float32, torch.bfloat16)
+            or torch._C._are_functorch_transforms_active() or torch.compiler.is_compiling()):
+        return None
+    try:
+        return B.pack_call(spacing, origin, fan, params, pose_ctr)
+    except (struct.error, TypeError):
+        return None
+
+
 def render(volume: torch.Tensor, pose: torch.Tensor, fan, params, spacing=(1.0, 1.0, 1.0),
            origin=(0.0, 0.0, 0.0), pose_ctr: int = 0):
     """Render one pose: returns (image [n_rays][S] float32, ray_valid int32)."""
+    call = _native_call(volume, pose, fan, params, spacing, origin, pose_ctr)
+    if call is not None:
+        return B.load_node().render(volume, pose, call)
     return _Render.apply(volume, pose, tuple(spacing), tuple(origin), fan, params, int(pose_ctr))
 
 
