@@ -15,31 +15,35 @@ struct VolPlace {
 };
 
 // Rotation R = Rz Ry Rx of ZYX Euler angles and its three partial
-// derivatives, in double precision (pose angles are float inputs).
-__device__ __forceinline__ void rotation_zyx(const double r[3], double R[3][3], double dR[3][3][3])
+// derivatives, in double precision (pose angles are float inputs), from the
+// angles' sines and cosines.  Every product and sum of the geometry is
+// rounded as written (explicit intrinsics), so that every kernel that sets
+// rays up gets the same positions bit for bit.
+__device__ __forceinline__ double mul3(double a, double b, double c) { return __dmul_rn(__dmul_rn(a, b), c); }
+__device__ __forceinline__ double mul3_add(double a, double b, double c, double d, double e)
 {
-    double sx, cx, sy, cy, sz, cz;
-    sincos(r[0], &sx, &cx);
-    sincos(r[1], &sy, &cy);
-    sincos(r[2], &sz, &cz);
+    return __fma_rn(__dmul_rn(a, b), c, __dmul_rn(d, e));   // abc + de
+}
+
+__device__ __forceinline__ void rotation_zyx(const double sn[3], const double cs[3], double R[3][3], double dR[3][3][3])
+{
+    const double sx = sn[0], sy = sn[1], sz = sn[2], cx = cs[0], cy = cs[1], cz = cs[2];
     // R = Rz Ry Rx expanded
-    R[0][0] = cz * cy; R[0][1] = cz * sy * sx - sz * cx; R[0][2] = cz * sy * cx + sz * sx;
-    R[1][0] = sz * cy; R[1][1] = sz * sy * sx + cz * cx; R[1][2] = sz * sy * cx - cz * sx;
-    R[2][0] = -sy;     R[2][1] = cy * sx;                R[2][2] = cy * cx;
-    if (dR) {
-        // d/drx: differentiate the Rx factor
-        dR[0][0][0] = 0; dR[0][0][1] = cz * sy * cx + sz * sx; dR[0][0][2] = -cz * sy * sx + sz * cx;
-        dR[0][1][0] = 0; dR[0][1][1] = sz * sy * cx - cz * sx; dR[0][1][2] = -sz * sy * sx - cz * cx;
-        dR[0][2][0] = 0; dR[0][2][1] = cy * cx;                dR[0][2][2] = -cy * sx;
-        // d/dry
-        dR[1][0][0] = -cz * sy; dR[1][0][1] = cz * cy * sx; dR[1][0][2] = cz * cy * cx;
-        dR[1][1][0] = -sz * sy; dR[1][1][1] = sz * cy * sx; dR[1][1][2] = sz * cy * cx;
-        dR[1][2][0] = -cy;      dR[1][2][1] = -sy * sx;     dR[1][2][2] = -sy * cx;
-        // d/drz
-        dR[2][0][0] = -sz * cy; dR[2][0][1] = -sz * sy * sx - cz * cx; dR[2][0][2] = -sz * sy * cx + cz * sx;
-        dR[2][1][0] = cz * cy;  dR[2][1][1] = cz * sy * sx - sz * cx;  dR[2][1][2] = cz * sy * cx + sz * sx;
-        dR[2][2][0] = 0;        dR[2][2][1] = 0;                       dR[2][2][2] = 0;
-    }
+    R[0][0] = __dmul_rn(cz, cy); R[0][1] = mul3_add(cz, sy, sx, -sz, cx); R[0][2] = mul3_add(cz, sy, cx, sz, sx);
+    R[1][0] = __dmul_rn(sz, cy); R[1][1] = mul3_add(sz, sy, sx, cz, cx);  R[1][2] = mul3_add(sz, sy, cx, -cz, sx);
+    R[2][0] = -sy;               R[2][1] = __dmul_rn(cy, sx);             R[2][2] = __dmul_rn(cy, cx);
+    // d/drx: differentiate the Rx factor
+    dR[0][0][0] = 0; dR[0][0][1] = R[0][2]; dR[0][0][2] = -R[0][1];
+    dR[0][1][0] = 0; dR[0][1][1] = R[1][2]; dR[0][1][2] = -R[1][1];
+    dR[0][2][0] = 0; dR[0][2][1] = R[2][2]; dR[0][2][2] = -R[2][1];
+    // d/dry
+    dR[1][0][0] = __dmul_rn(-cz, sy); dR[1][0][1] = mul3(cz, cy, sx);     dR[1][0][2] = mul3(cz, cy, cx);
+    dR[1][1][0] = __dmul_rn(-sz, sy); dR[1][1][1] = mul3(sz, cy, sx);     dR[1][1][2] = mul3(sz, cy, cx);
+    dR[1][2][0] = -cy;                dR[1][2][1] = __dmul_rn(-sy, sx);   dR[1][2][2] = __dmul_rn(-sy, cx);
+    // d/drz
+    dR[2][0][0] = -R[1][0]; dR[2][0][1] = -R[1][1]; dR[2][0][2] = -R[1][2];
+    dR[2][1][0] = R[0][0];  dR[2][1][1] = R[0][1];  dR[2][1][2] = R[0][2];
+    dR[2][2][0] = 0;        dR[2][2][1] = 0;        dR[2][2][2] = 0;
 }
 
 __device__ __forceinline__ long long to_fixed(double x)
@@ -59,11 +63,11 @@ struct PoseFrame {
     double t[3];
 };
 
-__device__ __forceinline__ void pose_frame(const float *__restrict__ pose6, PoseFrame &f)
+__device__ __forceinline__ void pose_frame(const float *__restrict__ pose6, const double sn[3], const double cs[3],
+                                           PoseFrame &f)
 {
-    const double r[3] = {(double)pose6[3], (double)pose6[4], (double)pose6[5]};
     double R[3][3], dR[3][3][3];
-    rotation_zyx(r, R, dR);
+    rotation_zyx(sn, cs, R, dR);
     for (int i = 0; i < 3; i++) {
         f.Rc[i][0] = R[i][0];
         f.Rc[i][1] = R[i][2];
@@ -80,25 +84,46 @@ static __global__ void k_pose_frames(const float *__restrict__ poses, int P, Pos
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= P) return;
     PoseFrame f;
-    pose_frame(poses + 6 * (size_t)p, f);
+    double sn[3], cs[3];
+    for (int a = 0; a < 3; a++) sincos((double)poses[6 * (size_t)p + 3 + a], &sn[a], &cs[a]);
+    pose_frame(poses + 6 * (size_t)p, sn, cs, f);
     frames[p] = f;
 }
 
 // FP64 voxel coordinates of sample 0 of ray `ray` and the step between
 // samples (Section 2.4): sample k lies at x0 + k dx = (t + (k + 1/2) ds u -
 // origin) / spacing.  st, ct: sin and cos of the beam angle.
+__device__ __forceinline__ void beam_sincos(int ray, const FanDev &fan, double &st, double &ct)
+{
+    const double th = fan.n_rays > 1 ? __fma_rn(-0.5, fan.fov, __ddiv_rn(__dmul_rn(fan.fov, (double)ray),
+                                                                         (double)(fan.n_rays - 1)))
+                                     : 0.0;
+    sincos(th, &st, &ct);
+}
+
+// One axis of the line: Rc, t: the pose frame's row of that axis.
+__device__ __forceinline__ void axis_line(const double Rc[2], double t, double ds, double sp, double org, double st,
+                                          double ct, double &x0, double &dx)
+{
+    const double u = __fma_rn(Rc[0], st, __dmul_rn(Rc[1], ct));
+    x0 = __ddiv_rn(__dsub_rn(__fma_rn(__dmul_rn(0.5, ds), u, t), org), sp);
+    dx = __ddiv_rn(__dmul_rn(ds, u), sp);
+}
+
 __device__ __forceinline__ void ray_line(const PoseFrame &f, int ray, const FanDev &fan, const VolPlace &vp,
                                          double x0[3], double dx[3], double &st, double &ct)
 {
-    double th = fan.n_rays > 1 ? -0.5 * fan.fov + fan.fov * (double)ray / (double)(fan.n_rays - 1) : 0.0;
-    sincos(th, &st, &ct);
-    double ds = fan.depth / (double)fan.S;
-    double sp[3] = {vp.sx, vp.sy, vp.sz}, org[3] = {vp.ox, vp.oy, vp.oz};
-    for (int i = 0; i < 3; i++) {
-        const double u = f.Rc[i][0] * st + f.Rc[i][1] * ct;
-        x0[i] = (f.t[i] + 0.5 * ds * u - org[i]) / sp[i];
-        dx[i] = ds * u / sp[i];
-    }
+    beam_sincos(ray, fan, st, ct);
+    const double ds = __ddiv_rn(fan.depth, (double)fan.S);
+    const double sp[3] = {vp.sx, vp.sy, vp.sz}, org[3] = {vp.ox, vp.oy, vp.oz};
+    for (int i = 0; i < 3; i++) axis_line(f.Rc[i], f.t[i], ds, sp[i], org[i], st, ct, x0[i], dx[i]);
+}
+
+__device__ __forceinline__ long long step_fixed(double dx) { return __double2ll_rn(__dmul_rn(dx, 4294967296.0)); }
+
+__device__ __forceinline__ float dir_derivative(const double dRc[2], double st, double ct)
+{
+    return (float)__fma_rn(dRc[0], st, __dmul_rn(dRc[1], ct));
 }
 
 // Geometry of ray `ray` of pose `pose_idx` (Section 2.4): FP64 direction and
@@ -110,25 +135,103 @@ __device__ __forceinline__ void setup_ray(const PoseFrame &f, int pose_idx, int 
     ray_line(f, ray, fan, vp, x0, dx, st, ct);
     for (int i = 0; i < 3; i++) {
         out.X0[i] = to_fixed(x0[i]);
-        out.DX[i] = __double2ll_rn(dx[i] * 4294967296.0);
+        out.DX[i] = step_fixed(dx[i]);
     }
-    const double ds = fan.depth / (double)fan.S;
     for (int q = 0; q < 3; q++)
-        for (int i = 0; i < 3; i++) out.v[q][i] = (float)(f.dRc[q][i][0] * st + f.dRc[q][i][1] * ct);
+        for (int i = 0; i < 3; i++) out.v[q][i] = dir_derivative(f.dRc[q][i], st, ct);
     out.pose = pose_idx;
     out.ray = ray;
     out.S = fan.S;
-    out.ds = (float)ds;
+    out.ds = (float)__ddiv_rn(fan.depth, (double)fan.S);
+}
+
+// Setup of one pose's rays in one launch: the pose frame, the ray table and
+// (rows not null) the offsets that the backward's kernels read.  FP64 runs at
+// two operations per clock and SM, so a warp's FP64 instruction takes 16 clocks
+// whatever its lanes do: a block takes ten rays with one lane per ray and
+// axis (two divisions in series instead of six) while a second warp works out
+// the pose frame.  Frame kernel, ray kernel and offset kernel took 6.5 + 8.5 +
+// 2 us for a frame; this one 7.0 us.  Above kSetupFrameRays rays the blocks'
+// repeated pose frames cost more than the separate kernel.
+constexpr int kSetupRays = 10;
+constexpr int kSetupFrameRays = 4096;
+
+struct RowOffsets {
+    long long *row, *gz, *ck;
+    int *ray0;
+    int row_ld;
+};
+
+__device__ __forceinline__ void write_offsets(const RowOffsets &o, int j, int n, int S)
+{
+    o.row[j] = (long long)j * o.row_ld;
+    o.gz[j] = (long long)j * gz_stride(S) + kGzLead;
+    o.ck[j] = (long long)j * ((S + kSeg - 1) / kSeg);
+    if (j == 0) {
+        o.ray0[0] = 0;
+        o.ray0[1] = n;
+    }
+}
+
+static __global__ void __launch_bounds__(64) k_setup_frame(const float *__restrict__ pose6, FanDev fan, VolPlace vp,
+                                                           PoseFrame *__restrict__ frame, RayGeo *__restrict__ geo,
+                                                           RowOffsets off)
+{
+    __shared__ PoseFrame f;
+    __shared__ double sn[3], cs[3];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j = blockIdx.x * kSetupRays + lane / 3, a = lane % 3;
+    const bool on = lane < 3 * kSetupRays && j < fan.n_rays;
+    double st = 0.0, ct = 1.0;
+    if (w == 1) {
+        if (lane < 3) sincos((double)pose6[3 + lane], &sn[lane], &cs[lane]);
+        __syncwarp();
+        if (lane == 0) {
+            pose_frame(pose6, sn, cs, f);
+            if (blockIdx.x == 0) *frame = f;
+        }
+    } else if (on) {
+        beam_sincos(j, fan, st, ct);
+    }
+    __syncthreads();
+    if (w == 1 || !on) return;
+    const double ds = __ddiv_rn(fan.depth, (double)fan.S);
+    double x0, dx;
+    axis_line(f.Rc[a], f.t[a], ds, a == 0 ? vp.sx : (a == 1 ? vp.sy : vp.sz), a == 0 ? vp.ox : (a == 1 ? vp.oy : vp.oz),
+              st, ct, x0, dx);
+    RayGeo &g = geo[j];
+    g.X0[a] = to_fixed(x0);
+    g.DX[a] = step_fixed(dx);
+    for (int q = 0; q < 3; q++) g.v[q][a] = dir_derivative(f.dRc[q][a], st, ct);
+    if (a == 0) {
+        g.pose = 0;
+        g.ray = j;
+        g.S = fan.S;
+        g.ds = (float)ds;
+        if (off.row) write_offsets(off, j, fan.n_rays, fan.S);
+    }
 }
 
 static __global__ void k_ray_setup(const PoseFrame *__restrict__ frame, FanDev fan, VolPlace vp,
-                                   RayGeo *__restrict__ geo)
+                                   RayGeo *__restrict__ geo, RowOffsets off)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= fan.n_rays) return;
     RayGeo rg;
     setup_ray(*frame, 0, j, fan, vp, rg);
     geo[j] = rg;
+    if (off.row) write_offsets(off, j, fan.n_rays, fan.S);
+}
+
+inline void launch_setup(const float *pose, const FanDev &fd, const VolPlace &vp, PoseFrame *frame, RayGeo *geo,
+                         const RowOffsets &off, cudaStream_t s)
+{
+    if (fd.n_rays <= kSetupFrameRays) {
+        k_setup_frame<<<(fd.n_rays + kSetupRays - 1) / kSetupRays, 64, 0, s>>>(pose, fd, vp, frame, geo, off);
+    } else {
+        k_pose_frames<<<1, 32, 0, s>>>(pose, 1, frame);
+        k_ray_setup<<<(fd.n_rays + 127) / 128, 128, 0, s>>>(frame, fd, vp, geo, off);
+    }
 }
 
 // One warp per ray, kWarpsFwd warps per CTA.
@@ -164,6 +267,28 @@ __global__ void __launch_bounds__(kWarpsFwd * 32) k_march_fwd(const T *__restric
     RayOut o{out + (size_t)j * rg.S, valid ? valid + j : nullptr, status, nullptr, nullptr, nullptr, nullptr,
              sel.rinfo ? sel.rinfo + j : nullptr, sel.rlist, sel.rcount, j, false};
     march_fwd_ray<T, MODE, TRACK, true, false>(vol, A, rg, o, buf[w]);
+}
+
+// One block per ray, up to kMultiWarps of its segments side by side: for fans
+// too small to fill the GPU with one warp per ray, whose time is one ray's
+// chain of segments (256 rays x 1024 rows: 24 us with one warp per ray, 9.4
+// us with four).  The rows are the same bits (march_fwd_multi).
+constexpr int kMultiWarps = 8;
+constexpr int kMultiRays = 2432;     // 16 warps per SM: beyond, one warp per ray fills the GPU
+
+template <typename T, int MODE, bool TRACK>
+__global__ void __launch_bounds__(kMultiWarps * 32) k_march_fwd_multi(const T *__restrict__ vol, MarchArgs A,
+                                                                     const RayGeo *__restrict__ geo,
+                                                                     float *__restrict__ out, int *__restrict__ valid,
+                                                                     uint32_t *__restrict__ status, RefineSel sel)
+{
+    __shared__ float2 buf[kMultiWarps][kSegPad];
+    __shared__ MultiSmem<kMultiWarps> ms;
+    const int j = blockIdx.x;
+    const RayGeo rg = geo[j];
+    RayOut o{out + (size_t)j * rg.S, valid ? valid + j : nullptr, status, nullptr, nullptr, nullptr, nullptr,
+             sel.rinfo ? sel.rinfo + j : nullptr, sel.rlist, sel.rcount, j, false};
+    march_fwd_multi<T, MODE, TRACK>(vol, A, rg, o, buf[threadIdx.x >> 5], ms);
 }
 
 // The refined pass of one ray that the FP32 pass listed: its FP64 line from
@@ -355,15 +480,25 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
 // Single-pose blur: one warp per strip and range of kBlurSegRays rays (one
 // pose alone is too small a grid for whole-fan strips).
 constexpr int kBlurSegRays = 64;
+// Rays per warp: fewer for small images, which are bound by one warp's sweep
+// (64 rays x 256 rows: 14.6 us with 64 rays a warp, 5.6 us with 8), as long as the
+// image does not fill the GPU's 608 schedulers; a range also reads 2W halo rays.
+inline int blur_seg_rays(int strips, int n)
+{
+    int seg = kBlurSegRays;
+    while (seg > kBlurStep && (int64_t)strips * ((n + seg - 1) / seg) < 608) seg /= 2;
+    return seg;
+}
 
 template <bool TRANSPOSE, int WT>
 __global__ void __launch_bounds__(kBlurWarps * 32) k_blur(const float *__restrict__ in, float *__restrict__ out,
-                                                          int n, int S, int si, int so, BlurArgs b, float l2_hi, float l2_lo)
+                                                          int n, int S, int si, int so, int seg, BlurArgs b, float l2_hi,
+                                                          float l2_lo)
 {
     const int strip = blockIdx.x * kBlurWarps + (threadIdx.x >> 5);
     if (strip * kBlurRows >= S) return;
-    const int j0 = blockIdx.y * kBlurSegRays;
-    blur_strip<TRANSPOSE, WT>(in, out, n, S, si, so, b, strip * kBlurRows, j0, min(n, j0 + kBlurSegRays), l2_hi, l2_lo);
+    const int j0 = blockIdx.y * seg;
+    blur_strip<TRANSPOSE, WT>(in, out, n, S, si, so, b, strip * kBlurRows, j0, min(n, j0 + seg), l2_hi, l2_lo);
 }
 
 }  // namespace dfs

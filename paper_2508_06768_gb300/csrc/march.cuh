@@ -434,61 +434,22 @@ __device__ __forceinline__ void store_rows(const RayOut &out, int i0, int S, con
     }
 }
 
-// Forward march of one ray by one warp.  buf: this warp's shared row of
-// kSegPad float pairs.  SPK_INLINE draws the speckle here (when it is on and
-// no factors are passed in out.min); without it the factors come from out.min
-// or there are none.  STREAM writes one-pass rows with evict-first stores
-// (the batched kernel).
-//
-// TRACK (the FP32 pass of a refined render, out.rinfo set) also decides
-// whether the ray needs the refined pass (rows whose md falls below
-// kNeedCoef sqrt(S), or a pole): such a ray is appended to out.rlist, and its
-// valid-row count and status are left to the refined pass.
-//
-// The rows carry no per-row tests: a chunk keeps the smallest determinant
-// and a sum that is NaN once any row is not finite, and only a chunk that
-// fails either is walked again for the first ill-posed row and the count.
-template <typename T, int MODE, bool TRACK, bool SPK_INLINE, bool STREAM>
-__device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg, const RayOut &out,
-                              float2 *__restrict__ buf)
+// What a ray's lanes found on the way: the first ill-posed depth, the rows
+// that are not finite, the last row that needs the refined states.
+struct RowFinds {
+    int first_bad = 0x7fffffff, nonfinite = 0, last_need = -1;
+};
+
+// Echo rows of this lane's chunk from its coefficients and the state at its
+// start.  pole_seen: an earlier segment met a pole (its row is the one that
+// counts).
+template <int MODE, bool TRACK, bool SPK_INLINE, bool STREAM>
+__device__ __forceinline__ void chunk_rows(const MarchArgs &A, const RayGeo &rg, const RayOut &out, int i0,
+                                           const float (&rr)[kChunk], float b0, float b1, float D, float need_md,
+                                           bool pole_seen, RowFinds &f)
 {
-    const int lane = threadIdx.x & 31;
     const int S = rg.S;
     const float a2 = A.a2;
-    float czr, cdz;
-    sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz);
-    if (out.zrow && lane == 0) out.zrow[0] = czr + cdz;
-    float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;   // bottom row and det at segment start
-    int first_bad = 0x7fffffff;
-    int nonfinite = 0;
-    int last_need = -1;                         // TRACK: last row with md below the threshold
-    const float need_md = TRACK ? fmaxf(kNeedFloor, kNeedCoef * sqrtf((float)S)) : 0.0f;
-    bool pole_seen = false;                     // in an earlier segment
-
-    for (int base = 0; base < S; base += kSeg) {
-        if (out.ckpt && lane == 0) out.ckpt[base / kSeg] = make_float4(bs0, bs1, Ds, 0.0f);
-        const int i0 = base + lane * kChunk;
-        float rr[kChunk];
-        seg_coefficients<T, STREAM>(vol, A.g, rg, base, czr, cdz, buf, out.zrow, rr);
-        if (out.rrow && i0 < S) {
-            float4 *dst = reinterpret_cast<float4 *>(out.rrow + i0 + 1);   // r_{i0} belongs to sample i0 + 1
-            __stcs(dst, make_float4(rr[0], rr[1], rr[2], rr[3]));
-            __stcs(dst + 1, make_float4(rr[4], rr[5], rr[6], rr[7]));
-        }
-        Mat2 Q, E, Qall;
-        float dq, de, dall;
-        chunk_product<MODE>(rr, a2, Q, dq);
-        warp_scan_prefix(Q, dq, E, de, Qall, dall);
-        float b0 = fmaf(bs0, E.a, bs1 * E.c);
-        float b1 = fmaf(bs0, E.b, bs1 * E.d);
-        float D = Ds * de;
-        {
-            float n0 = fmaf(bs0, Qall.a, bs1 * Qall.c);
-            float n1 = fmaf(bs0, Qall.b, bs1 * Qall.d);
-            bs0 = n0;
-            bs1 = n1;
-            Ds *= dall;
-        }
         float m[kChunk];
         if (out.min) {
             load_chunk(out.min + i0, i0 < S, m);
@@ -506,7 +467,7 @@ __device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
             const Xfer x = xfer_t<MODE>(rr[t], a2);
             const float q = fmaf(b0, x.m01, b1);          // det(A_{i+1})
             const float e = x.m01 * D * frcp(b1 * q);
-            if (TRACK && i0 + t < S && fminf(b1, q) < need_md) last_need = i0 + t;
+            if (TRACK && i0 + t < S && fminf(b1, q) < need_md) f.last_need = i0 + t;
             minq = fminf(minq, q);
             const float nb0 = fmaf(b0, x.m00, b1 * x.m10);
             b1 = q;
@@ -523,17 +484,23 @@ __device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
                 const Xfer x = xfer_t<MODE>(rr[t], a2);
                 const float q = fmaf(c0, x.m01, c1);
                 if (i0 + t < S) {
-                    if (!(q >= kPoleEps)) first_bad = min(first_bad, i0 + t + 1);
-                    nonfinite += !isfinite(y[t]);
+                    if (!(q >= kPoleEps)) f.first_bad = min(f.first_bad, i0 + t + 1);
+                    f.nonfinite += !isfinite(y[t]);
                 }
                 c0 = fmaf(c0, x.m00, c1 * x.m10);
                 c1 = q;
             }
         }
-        pole_seen = pole_seen || __any_sync(0xffffffffu, first_bad <= S);
         if (i0 < S) store_rows<STREAM>(out, i0, S, y);
-    }
+}
 
+// The ray's counts after its last segment (called by one warp; f holds each
+// lane's finds).
+template <bool TRACK>
+__device__ __forceinline__ void finish_ray(const RayOut &out, int S, RowFinds f)
+{
+    const int lane = threadIdx.x & 31;
+    int first_bad = f.first_bad, nonfinite = f.nonfinite, last_need = f.last_need;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         first_bad = min(first_bad, __shfl_xor_sync(0xffffffffu, first_bad, off));
@@ -563,6 +530,141 @@ __device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
             if (nonfinite) atomicAdd(out.status + 1, (uint32_t)nonfinite);
         }
     }
+}
+
+// Forward march of one ray by one warp.  buf: this warp's shared row of
+// kSegPad float pairs.  SPK_INLINE draws the speckle here (when it is on and
+// no factors are passed in out.min); without it the factors come from out.min
+// or there are none.  STREAM writes one-pass rows with evict-first stores
+// (the batched kernel).
+//
+// TRACK (the FP32 pass of a refined render, out.rinfo set) also decides
+// whether the ray needs the refined pass (rows whose md falls below
+// kNeedCoef sqrt(S), or a pole): such a ray is appended to out.rlist, and its
+// valid-row count and status are left to the refined pass.
+//
+// The rows carry no per-row tests: a chunk keeps the smallest determinant
+// and a sum that is NaN once any row is not finite, and only a chunk that
+// fails either is walked again for the first ill-posed row and the count.
+template <typename T, int MODE, bool TRACK, bool SPK_INLINE, bool STREAM>
+__device__ void march_fwd_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg, const RayOut &out,
+                              float2 *__restrict__ buf)
+{
+    const int lane = threadIdx.x & 31;
+    const int S = rg.S;
+    const float a2 = A.a2;
+    float czr, cdz;
+    sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz);
+    if (out.zrow && lane == 0) out.zrow[0] = czr + cdz;
+    float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;   // bottom row and det at segment start
+    RowFinds f;
+    const float need_md = TRACK ? fmaxf(kNeedFloor, kNeedCoef * sqrtf((float)S)) : 0.0f;
+    bool pole_seen = false;                     // in an earlier segment
+
+    for (int base = 0; base < S; base += kSeg) {
+        if (out.ckpt && lane == 0) out.ckpt[base / kSeg] = make_float4(bs0, bs1, Ds, 0.0f);
+        const int i0 = base + lane * kChunk;
+        float rr[kChunk];
+        seg_coefficients<T, STREAM>(vol, A.g, rg, base, czr, cdz, buf, out.zrow, rr);
+        if (out.rrow && i0 < S) {
+            float4 *dst = reinterpret_cast<float4 *>(out.rrow + i0 + 1);   // r_{i0} belongs to sample i0 + 1
+            __stcs(dst, make_float4(rr[0], rr[1], rr[2], rr[3]));
+            __stcs(dst + 1, make_float4(rr[4], rr[5], rr[6], rr[7]));
+        }
+        Mat2 Q, E, Qall;
+        float dq, de, dall;
+        chunk_product<MODE>(rr, a2, Q, dq);
+        warp_scan_prefix(Q, dq, E, de, Qall, dall);
+        float b0 = fmaf(bs0, E.a, bs1 * E.c);
+        float b1 = fmaf(bs0, E.b, bs1 * E.d);
+        float D = Ds * de;
+        {
+            float n0 = fmaf(bs0, Qall.a, bs1 * Qall.c);
+            float n1 = fmaf(bs0, Qall.b, bs1 * Qall.d);
+            bs0 = n0;
+            bs1 = n1;
+            Ds *= dall;
+        }
+        chunk_rows<MODE, TRACK, SPK_INLINE, STREAM>(A, rg, out, i0, rr, b0, b1, D, need_md, pole_seen, f);
+        pole_seen = pole_seen || __any_sync(0xffffffffu, f.first_bad <= S);
+    }
+    finish_ray<TRACK>(out, S, f);
+}
+
+// The march of one ray by all warps of a block, a segment each: a warp
+// samples its segment, forms its chunk products and scan, and learns the
+// state at its start from the totals of the segments before, composed in
+// order with march_fwd_ray's own arithmetic, so the rows are the same bits.
+template <int WARPS>
+struct MultiSmem {
+    float4 q[WARPS];       // segment totals
+    float d[WARPS];
+    RowFinds f[32];        // lanes' finds over all warps
+};
+
+template <typename T, int MODE, bool TRACK>
+__device__ void march_fwd_multi(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg, const RayOut &out,
+                                float2 *__restrict__ buf, MultiSmem<8> &ms)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int S = rg.S;
+    RowFinds f;
+    const float need_md = TRACK ? fmaxf(kNeedFloor, kNeedCoef * sqrtf((float)S)) : 0.0f;
+    float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;   // state at the start of the round
+    auto advance = [&](int v) {
+        const float4 q = ms.q[v];
+        const float n0 = fmaf(bs0, q.x, bs1 * q.z);
+        const float n1 = fmaf(bs0, q.y, bs1 * q.w);
+        bs0 = n0;
+        bs1 = n1;
+        Ds *= ms.d[v];
+    };
+    for (int base0 = 0; base0 < S; base0 += nw * kSeg) {
+        const int base = base0 + w * kSeg;
+        const bool on = base < S;
+        float rr[kChunk];
+        Mat2 E = mat_ident(), Qall;
+        float de = 1.0f, dall;
+        if (on) {
+            long long X, Y, Z;
+            float czr, cdz;
+            sample_pos(rg, base, X, Y, Z);
+            sample_z<T, false>(vol, A.g, X, Y, Z, czr, cdz);
+            seg_coefficients<T, false>(vol, A.g, rg, base, czr, cdz, buf, nullptr, rr);
+            Mat2 Q;
+            float dq;
+            chunk_product<MODE>(rr, A.a2, Q, dq);
+            warp_scan_prefix(Q, dq, E, de, Qall, dall);
+            if (lane == 0) {
+                ms.q[w] = make_float4(Qall.a, Qall.b, Qall.c, Qall.d);
+                ms.d[w] = dall;
+            }
+        }
+        __syncthreads();
+        const int nv = min(nw, (S - base0 + kSeg - 1) / kSeg);
+        for (int v = 0; v < min(w, nv); v++) advance(v);
+        if (on) {
+            const float b0 = fmaf(bs0, E.a, bs1 * E.c);
+            const float b1 = fmaf(bs0, E.b, bs1 * E.d);
+            const float D = Ds * de;
+            chunk_rows<MODE, TRACK, true, false>(A, rg, out, base + lane * kChunk, rr, b0, b1, D, need_md, false, f);
+        }
+        for (int v = w; v < nv; v++) advance(v);
+        __syncthreads();
+    }
+    // one lane's finds of all warps, then the ray's
+    if (w == 0) ms.f[lane] = f;
+    for (int v = 1; v < nw; v++) {
+        __syncthreads();
+        if (w == v) {
+            RowFinds &g = ms.f[lane];
+            g.first_bad = min(g.first_bad, f.first_bad);
+            g.nonfinite += f.nonfinite;
+            g.last_need = max(g.last_need, f.last_need);
+        }
+    }
+    __syncthreads();
+    if (w == 0) finish_ray<TRACK>(out, S, ms.f[lane]);
 }
 
 // The refined pass of one ray by one warp (buf: kSegPad floats, dbuf: kSegPad

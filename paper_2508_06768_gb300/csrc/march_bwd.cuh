@@ -64,16 +64,30 @@ __device__ __forceinline__ EchoGrad echo_grad(float b0, float b1, float D, float
 // gz_stride(S).  Only the gather reads dL/dZ, so POSE (which runs without one)
 // does not write it.
 //
+// MULTI (not STORED; mm is the block's): all warps of the block march one ray,
+// a segment each, side by side up to the true reverse pass, which runs in turn
+// from the last segment to the first and hands the adjoint on through shared
+// memory: the same arithmetic in the same order, for fans too small to fill
+// the GPU with one warp per ray.
+//
 // Past the ray's end r and the adjoint sources are 0, so the passes need no
 // row tests; only the Z1-role term of interface S, which would reach sample
 // S, is dropped explicitly.
-template <typename T, int MODE, bool POSE, bool STORED = false>
+struct BwdMulti {
+    float4 q[32];            // segment totals (first sweep)
+    float d[32];
+    float lam0, lam1, mu, carry;   // adjoint at the end of the segment whose turn it is
+};
+
+template <typename T, int MODE, bool POSE, bool STORED = false, bool MULTI = false>
 __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, const RayGeo &rg,
                               const float *__restrict__ gy_row, float *__restrict__ gz_row,
                               double *__restrict__ pose_part, float4 *__restrict__ ckpt, BwdSmem<POSE, STORED> &sm,
                               bool gy_vec, bool have_ckpt = false, const float *__restrict__ mrow = nullptr,
-                              const float *__restrict__ zrow = nullptr, const float *__restrict__ rrow = nullptr)
+                              const float *__restrict__ zrow = nullptr, const float *__restrict__ rrow = nullptr,
+                              BwdMulti *mm = nullptr, double *macc = nullptr)
 {
+    static_assert(!(STORED && MULTI), "the batched march takes one ray per warp");
     static_assert(!(STORED && POSE), "the pose terms of the march need the sampled gradient");
     // The batched call (STORED) streams gigabytes of one-pass rows: evict-
     // first loads and stores keep them from displacing reused L2 lines.  The
@@ -84,39 +98,73 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
     const float a2 = A.a2;
     const int nseg = (S + kSeg - 1) / kSeg;
 
+    const int w = MULTI ? (int)(threadIdx.x >> 5) : 0, nw = MULTI ? (int)(blockDim.x >> 5) : 1;
+
     // ---------------- sweep 1: forward, record the carry at segment starts
+    // (the last segment's totals reach no carry)
     if (!STORED && !have_ckpt) {
         float czr, cdz;
-        sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz);
+        if (!MULTI) sample_z<T, false>(vol, A.g, rg.X0[0], rg.X0[1], rg.X0[2], czr, cdz);
         float bs0 = 0.0f, bs1 = 1.0f, Ds = 1.0f;
-        for (int s = 0; s < nseg; s++) {
-            if (lane == 0) ckpt[s] = make_float4(bs0, bs1, Ds, 0.0f);
-            float rr[kChunk];
-            seg_coefficients<T, false>(vol, A.g, rg, s * kSeg, czr, cdz, reinterpret_cast<float2 *>(sm.eg), nullptr,
-                                       rr);
-            Mat2 Q, E, Qall;
-            float dq, de, dall;
-            chunk_product<MODE>(rr, a2, Q, dq);
-            warp_scan_prefix(Q, dq, E, de, Qall, dall);
-            float n0 = fmaf(bs0, Qall.a, bs1 * Qall.c);
-            float n1 = fmaf(bs0, Qall.b, bs1 * Qall.d);
-            bs0 = n0;
-            bs1 = n1;
-            Ds *= dall;
+        if (lane == 0 && w == 0) ckpt[0] = make_float4(bs0, bs1, Ds, 0.0f);
+        for (int s0 = 0; s0 < nseg - 1; s0 += nw) {
+            const int s = s0 + w;
+            Mat2 Qall;
+            float dall;
+            if (s < nseg - 1) {
+                if (MULTI) {
+                    long long X, Y, Z;
+                    sample_pos(rg, s * kSeg, X, Y, Z);
+                    sample_z<T, false>(vol, A.g, X, Y, Z, czr, cdz);
+                }
+                float rr[kChunk];
+                seg_coefficients<T, false>(vol, A.g, rg, s * kSeg, czr, cdz, reinterpret_cast<float2 *>(sm.eg),
+                                           nullptr, rr);
+                Mat2 Q, E;
+                float dq, de;
+                chunk_product<MODE>(rr, a2, Q, dq);
+                warp_scan_prefix(Q, dq, E, de, Qall, dall);
+                if (MULTI && lane == 0) {
+                    mm->q[w] = make_float4(Qall.a, Qall.b, Qall.c, Qall.d);
+                    mm->d[w] = dall;
+                }
+            }
+            if (MULTI) __syncthreads();
+            for (int v = 0; v < nw && s0 + v < nseg - 1; v++) {
+                if (MULTI) {
+                    const float4 q = mm->q[v];
+                    Qall = {q.x, q.y, q.z, q.w};
+                    dall = mm->d[v];
+                }
+                float n0 = fmaf(bs0, Qall.a, bs1 * Qall.c);
+                float n1 = fmaf(bs0, Qall.b, bs1 * Qall.d);
+                bs0 = n0;
+                bs1 = n1;
+                Ds *= dall;
+                if (lane == 0 && w == 0) ckpt[s0 + v + 1] = make_float4(bs0, bs1, Ds, 0.0f);
+            }
+            if (MULTI) __syncthreads();
         }
     }
-    __syncwarp();
+    if (MULTI) {
+        if (threadIdx.x == 0) mm->lam0 = mm->lam1 = mm->mu = mm->carry = 0.0f;
+        __syncthreads();
+    } else {
+        __syncwarp();
+    }
 
     // ---------------- sweep 2: reverse over segments
     float lam0 = 0.0f, lam1 = 0.0f, mus = 0.0f;   // adjoint at the end of the current segment
     float carry_gz1 = 0.0f;                       // dL/dZ of sample base+256 from interface base+256
     float czr = 0.0f, cdz = 0.0f, cg0 = 0.0f, cg1 = 0.0f, cg2 = 0.0f;   // sample base+256
-    double *acc = sm.acc;
-    if (POSE && lane == 0)
+    double *acc = MULTI ? macc : sm.acc;
+    if (POSE && lane == 0 && w == 0)
         for (int q = 0; q < 6; q++) acc[q] = 0.0;
     const float ds = rg.ds;
 
-    for (int s = nseg - 1; s >= 0; s--) {
+    for (int s0 = nseg - 1; s0 >= 0; s0 -= nw) {
+        const bool on = !MULTI || s0 >= w;   // a warp without a segment repeats segment 0 and writes nothing
+        const int s = on ? s0 - w : 0;
         const int base = s * kSeg;
         const int i0 = base + lane * kChunk;
         float rr[kChunk];
@@ -145,7 +193,7 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
                 }
             }
             if (lane == 0) {
-                if (s == nseg - 1 && base + kSeg <= S) {
+                if ((MULTI || s == nseg - 1) && base + kSeg <= S) {
                     float g3[3];
                     sample_pos(rg, base + kSeg, X, Y, Z);
                     sample_z<T, POSE>(vol, A.g, X, Y, Z, czr, cdz, g3);
@@ -253,6 +301,15 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
                 Pm = mat_mul(Pm, Po);
                 pal *= oal;
             }
+        }
+        for (int turn = 0; turn < nw; turn++) {
+        if (MULTI) {
+            __syncthreads();
+            if (turn != w || !on) continue;
+            lam0 = mm->lam0;
+            lam1 = mm->lam1;
+            mus = mm->mu;
+            carry_gz1 = mm->carry;
         }
         // adjoint at this lane's chunk end = G_{lane+1}(lambda_seg)
         float le0, le1, lmu;
@@ -380,9 +437,17 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
                 if (lane == 0) acc[q] += (double)v;
             }
         }
+        if (MULTI && lane == 0) {
+            mm->lam0 = lam0;
+            mm->lam1 = lam1;
+            mm->mu = mus;
+            mm->carry = carry_gz1;
+        }
+        }
         __syncwarp();
     }
-    if (POSE && lane == 0) {
+    if (MULTI) __syncthreads();
+    if (POSE && lane == 0 && w == 0) {
         pose_part[0] = acc[0];
         pose_part[1] = acc[1];
         pose_part[2] = acc[2];

@@ -36,6 +36,29 @@ __global__ void __launch_bounds__(kWarpsBwd * 32) k_march_bwd(const T *__restric
                            sm[w], gy_vec);
 }
 
+// One block per ray, up to kWarpsBwd of its segments side by side, for fans
+// too small to fill the GPU (251 rays x 1021 rows: 39 us with one warp per
+// ray, 16.7 us with four).
+template <typename T, bool POSE, int MODE>
+__global__ void __launch_bounds__(kWarpsBwd * 32) k_march_bwd_multi(const T *__restrict__ vol, MarchArgs A,
+                                                                   const RayGeo *__restrict__ geo,
+                                                                   const float *__restrict__ gy,
+                                                                   const long long *__restrict__ row_off,
+                                                                   float *__restrict__ gz,
+                                                                   const long long *__restrict__ gz_off,
+                                                                   double *__restrict__ pose_part,
+                                                                   float4 *__restrict__ ckpt,
+                                                                   const long long *__restrict__ ckpt_off, bool gy_vec)
+{
+    __shared__ BwdSmem<POSE> sm[kWarpsBwd];
+    __shared__ BwdMulti mm;
+    const int j = blockIdx.x;
+    const RayGeo rg = geo[j];
+    march_bwd_ray<T, MODE, POSE, false, true>(vol, A, rg, gy + row_off[j], gz + gz_off[j], pose_part + 6 * (size_t)j,
+                                              ckpt + ckpt_off[j], sm[threadIdx.x >> 5], gy_vec, false, nullptr,
+                                              nullptr, nullptr, &mm, sm[0].acc);
+}
+
 // Deterministic per-pose sum of per-ray pose partials: one warp per pose,
 // lanes stride over the pose's rays, then a fixed shuffle tree.
 static __global__ void k_pose_reduce(const double *__restrict__ part, const int *__restrict__ ray0, int P,
@@ -52,22 +75,6 @@ static __global__ void k_pose_reduce(const double *__restrict__ part, const int 
         double v = s[q];
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
         if (lane == 0) grad_pose[6 * p + q] = (float)v;
-    }
-}
-
-static __global__ void k_offsets(long long *__restrict__ row_off, long long *__restrict__ gz_off,
-                                 long long *__restrict__ ck_off, int *__restrict__ ray0, int n, int S,
-                                 int row_ld)
-{
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) {
-        row_off[j] = (long long)j * row_ld;
-        gz_off[j] = (long long)j * gz_stride(S) + kGzLead;
-        ck_off[j] = (long long)j * ((S + kSeg - 1) / kSeg);
-    }
-    if (j == 0) {
-        ray0[0] = 0;
-        ray0[1] = n;
     }
 }
 
@@ -106,26 +113,36 @@ static BwdLayout bwd_layout(void *ws, const diffus_volume_desc *vd, const diffus
 }
 
 template <typename T, bool POSE>
-static void launch_march_bwd_t(const void *vol, const MarchArgs &A, const BwdLayout &L, int n, const float *gy,
+static void launch_march_bwd_t(const void *vol, const MarchArgs &A, const BwdLayout &L, int n, int S, const float *gy,
                                bool gy_vec, int grid, cudaStream_t s)
 {
-    if (A.mode == DIFFUS_MODE_LITERAL)
-        k_march_bwd<T, POSE, DIFFUS_MODE_LITERAL><<<grid, kWarpsBwd * 32, 0, s>>>(
-            (const T *)vol, A, L.geo, n, gy, L.row_off, L.gz, L.gz_off, L.part, L.ckpt, L.ck_off, gy_vec);
-    else
-        k_march_bwd<T, POSE, DIFFUS_MODE_SIGNED><<<grid, kWarpsBwd * 32, 0, s>>>(
-            (const T *)vol, A, L.geo, n, gy, L.row_off, L.gz, L.gz_off, L.part, L.ckpt, L.ck_off, gy_vec);
+    const int nseg = (S + kSeg - 1) / kSeg;
+    const bool multi = nseg > 1 && n <= kMultiRays;
+    const int mthreads = 32 * (nseg < kWarpsBwd ? nseg : kWarpsBwd);
+#define DFS_BWD(MODE)                                                                                               \
+    if (multi)                                                                                                      \
+        k_march_bwd_multi<T, POSE, MODE><<<n, mthreads, 0, s>>>((const T *)vol, A, L.geo, gy, L.row_off, L.gz,      \
+                                                                L.gz_off, L.part, L.ckpt, L.ck_off, gy_vec);        \
+    else                                                                                                            \
+        k_march_bwd<T, POSE, MODE><<<grid, kWarpsBwd * 32, 0, s>>>((const T *)vol, A, L.geo, n, gy, L.row_off, L.gz, \
+                                                                   L.gz_off, L.part, L.ckpt, L.ck_off, gy_vec)
+    if (A.mode == DIFFUS_MODE_LITERAL) {
+        DFS_BWD(DIFFUS_MODE_LITERAL);
+    } else {
+        DFS_BWD(DIFFUS_MODE_SIGNED);
+    }
+#undef DFS_BWD
 }
 
-static int launch_march_bwd(const void *vol, int dtype, bool pose, const MarchArgs &A, const BwdLayout &L, int n,
+static int launch_march_bwd(const void *vol, int dtype, bool pose, const MarchArgs &A, const BwdLayout &L, int n, int S,
                             const float *gy, bool gy_vec, int grid, cudaStream_t s)
 {
     if (dtype == DIFFUS_F32) {
-        if (pose) launch_march_bwd_t<float, true>(vol, A, L, n, gy, gy_vec, grid, s);
-        else launch_march_bwd_t<float, false>(vol, A, L, n, gy, gy_vec, grid, s);
+        if (pose) launch_march_bwd_t<float, true>(vol, A, L, n, S, gy, gy_vec, grid, s);
+        else launch_march_bwd_t<float, false>(vol, A, L, n, S, gy, gy_vec, grid, s);
     } else {
-        if (pose) launch_march_bwd_t<unsigned short, true>(vol, A, L, n, gy, gy_vec, grid, s);
-        else launch_march_bwd_t<unsigned short, false>(vol, A, L, n, gy, gy_vec, grid, s);
+        if (pose) launch_march_bwd_t<unsigned short, true>(vol, A, L, n, S, gy, gy_vec, grid, s);
+        else launch_march_bwd_t<unsigned short, false>(vol, A, L, n, S, gy, gy_vec, grid, s);
     }
     return launch_status();
 }
@@ -156,10 +173,8 @@ extern "C" int diffus_render_bwd(const void *vol, const diffus_volume_desc *vd, 
     if (status && cudaMemsetAsync(status, 0, 4 * sizeof(uint32_t), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
     const int n = fan->n_rays, S = fan->n_samples;
     FanDev fd{n, S, fan->fov_rad, fan->depth_mm};
-    k_pose_frames<<<1, 32, 0, s>>>(pose, 1, L.frame);
-    k_ray_setup<<<(n + 127) / 128, 128, 0, s>>>(L.frame, fd, make_place(vd), L.geo);
-    k_offsets<<<(n + 127) / 128, 128, 0, s>>>(L.row_off, L.gz_off, L.ck_off, L.ray0, n, S,
-                                                  prm->blur ? row_stride(S) : S);
+    launch_setup(pose, fd, make_place(vd), L.frame, L.geo,
+                 RowOffsets{L.row_off, L.gz_off, L.ck_off, L.ray0, prm->blur ? row_stride(S) : S}, s);
     const float *gy = grad_image;
     if (prm->blur) {
         if ((rc = launch_blur(grad_image, L.gy, n, S, S, row_stride(S), prm, fan, true, s))) return rc;
@@ -175,7 +190,7 @@ extern "C" int diffus_render_bwd(const void *vol, const diffus_volume_desc *vd, 
     MarchArgs A = make_march_args(vd, fan, prm);
     int grid = (n + kWarpsBwd - 1) / kWarpsBwd;
     const bool march_pose = grad_pose && !grad_vol;
-    if ((rc = launch_march_bwd(vol, vd->dtype, march_pose, A, L, n, gy, prm->blur != 0, grid, s))) return rc;
+    if ((rc = launch_march_bwd(vol, vd->dtype, march_pose, A, L, n, S, gy, prm->blur != 0, grid, s))) return rc;
     if (grad_vol &&
         (rc = launch_gather(vd, vol, L.geo, n, fan->depth_mm, L.gz, L.gz_off, L.gather_ws, status, grad_vol,
                             grad_pose ? L.part : nullptr, 8, s)))

@@ -76,23 +76,30 @@ int launch_fwd_march(const void *vol, const diffus_volume_desc *vd, const float 
                      uint32_t *status, const RefineSel &sel, cudaStream_t s)
 {
     FanDev fd{fan->n_rays, fan->n_samples, fan->fov_rad, fan->depth_mm};
-    k_pose_frames<<<1, 32, 0, s>>>(pose, 1, frame);
-    k_ray_setup<<<(fan->n_rays + 127) / 128, 128, 0, s>>>(frame, fd, make_place(vd), geo);
+    launch_setup(pose, fd, make_place(vd), frame, geo, RowOffsets{nullptr, nullptr, nullptr, nullptr, 0}, s);
     MarchArgs A = make_march_args(vd, fan, prm);
     const int grid = (fan->n_rays + kWarpsFwd - 1) / kWarpsFwd;
     const bool refine = prm->refine && sel.rinfo;
     if (refine && cudaMemsetAsync(sel.rcount, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
     // the FP32 pass, then the refined pass over the rays it listed
+    const int nseg = (fan->n_samples + kSeg - 1) / kSeg;
+    const bool multi = nseg > 1 && fan->n_rays <= kMultiRays;
+    const int mthreads = 32 * (nseg < kMultiWarps ? nseg : kMultiWarps);
+    const RefineSel none{nullptr, nullptr, nullptr, nullptr};
+#define DFS_MARCH(T, MODE, TRACK, SEL)                                                                               \
+    if (multi)                                                                                                       \
+        k_march_fwd_multi<T, MODE, TRACK><<<fan->n_rays, mthreads, 0, s>>>((const T *)vol, A, geo, out, ray_valid,   \
+                                                                           status, SEL);                             \
+    else                                                                                                             \
+        k_march_fwd<T, MODE, TRACK><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, fan->n_rays, out,        \
+                                                                    ray_valid, status, SEL)
 #define DFS_FWD(T, MODE)                                                                                             \
     if (refine) {                                                                                                    \
-        k_march_fwd<T, MODE, true><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, fan->n_rays, out,        \
-                                                                   ray_valid, status, sel);                         \
-        k_march_refine<T><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, frame, fd, make_place(vd), out,   \
-                                                          ray_valid, status, sel);                                  \
+        DFS_MARCH(T, MODE, true, sel);                                                                               \
+        k_march_refine<T><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, frame, fd, make_place(vd), out,    \
+                                                          ray_valid, status, sel);                                   \
     } else {                                                                                                         \
-        k_march_fwd<T, MODE, false><<<grid, kWarpsFwd * 32, 0, s>>>((const T *)vol, A, geo, fan->n_rays, out,       \
-                                                                    ray_valid, status,                              \
-                                                                    RefineSel{nullptr, nullptr, nullptr, nullptr}); \
+        DFS_MARCH(T, MODE, false, none);                                                                             \
     }
     const bool literal = prm->mode == DIFFUS_MODE_LITERAL;
     if (vd->dtype == DIFFUS_F32) {
@@ -101,6 +108,7 @@ int launch_fwd_march(const void *vol, const diffus_volume_desc *vd, const float 
         if (literal) { DFS_FWD(unsigned short, DIFFUS_MODE_LITERAL) } else { DFS_FWD(unsigned short, DIFFUS_MODE_SIGNED) }
     }
 #undef DFS_FWD
+#undef DFS_MARCH
     return launch_status();
 }
 
@@ -111,12 +119,13 @@ int launch_blur(const float *in, float *out, int n, int S, int si, int so, const
     float hi = 0.0f, lo = 0.0f;
     if (prm->atten) gain_l2(attenuation_a(fan), hi, lo);
     const int strips = (S + kBlurRows - 1) / kBlurRows;
-    const dim3 grid((strips + kBlurWarps - 1) / kBlurWarps, (n + kBlurSegRays - 1) / kBlurSegRays);
+    const int seg = blur_seg_rays(strips, n);
+    const dim3 grid((strips + kBlurWarps - 1) / kBlurWarps, (n + seg - 1) / seg);
 #define DFS_BLUR(WT)                                                        \
     if (transpose)                                                          \
-        k_blur<true, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, si, so, b, hi, lo); \
+        k_blur<true, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, si, so, seg, b, hi, lo); \
     else                                                                    \
-        k_blur<false, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, si, so, b, hi, lo);
+        k_blur<false, WT><<<grid, kBlurWarps * 32, 0, s>>>(in, out, n, S, si, so, seg, b, hi, lo);
     switch (b.W) {
     case 0: DFS_BLUR(0) break;
     case 1: DFS_BLUR(1) break;
