@@ -287,25 +287,6 @@ void launch_batch_blur(const float *in, float *out, const PlanPose *poses, const
 
 }  // namespace
 
-namespace dfs {
-__global__ void k_pose_reduce_batch(const double *__restrict__ part, const int *__restrict__ ray0, int P,
-                                    float *__restrict__ grad_pose)
-{
-    const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (p >= P) return;
-    const int a = ray0[p], b = ray0[p + 1];
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = a + lane; j < b; j += 32)
-        for (int q = 0; q < 6; q++) s[q] += part[6 * (size_t)j + q];
-    for (int q = 0; q < 6; q++) {
-        double v = s[q];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) grad_pose[6 * p + q] = (float)v;
-    }
-}
-}  // namespace dfs
-
 // ---------------------------------------------------------------- entry points
 
 extern "C" size_t diffus_batch_plan_bytes(const diffus_fan *fans, int32_t P)
@@ -721,7 +702,7 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
     }
     mark(DIFFUS_TR_POSE);
     const int32_t *ray0 = at<int32_t>(plan_dev, H.off_ray0);
-    if (grad_poses) k_pose_reduce_batch<<<(H.P + 3) / 4, 128, 0, s>>>(L.part, ray0, H.P, grad_poses);
+    if (grad_poses) k_pose_reduce<<<H.P, 192, 0, s>>>(L.part, ray0, grad_poses);
     mark(DIFFUS_TR_END);
     return launch_status();
 }

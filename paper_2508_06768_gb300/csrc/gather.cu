@@ -14,10 +14,33 @@ constexpr int kScanChunk = 4096;
 
 // ------------------------------------------------------------------ runs
 
+// The run's 40 bytes in use.
+__device__ __forceinline__ void store_run(Run *dst, const Run &r)
+{
+    longlong2 *p = reinterpret_cast<longlong2 *>(dst);
+    p[0] = make_longlong2(r.X, r.Y);
+    p[1] = make_longlong2(r.Z, (long long)(unsigned)r.ray | ((long long)r.k0 << 32));
+    reinterpret_cast<uint2 *>(dst)[4] = make_uint2((uint32_t)r.len, r.next);
+}
+
+__device__ __forceinline__ void store_steps(RayStep *dst, const long long d[3], long long g_off)
+{
+    RayStep s;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        s.d[a] = d[a];
+        s.qr[a] = cell_steps(d[a]);
+        s.v[a] = slope_of(d[a]);
+        s.pad[a] = 0.0f;
+    }
+    s.g_off = g_off;
+    *dst = s;
+}
+
 // One thread per ray: many rays, or rays of more than kRunMax brick changes.
 __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__restrict__ gz_off, int n_rays,
-                           GatherArgs G, int cap, Run *__restrict__ runs, uint32_t *__restrict__ keys,
-                           int *__restrict__ nrun, uint32_t *__restrict__ bcount,
+                           GatherArgs G, int cap, Run *__restrict__ runs, RayStep *__restrict__ steps,
+                           uint32_t *__restrict__ keys, int *__restrict__ nrun, uint32_t *__restrict__ bcount,
                            unsigned long long *__restrict__ brick_work, uint32_t *__restrict__ status)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -31,6 +54,7 @@ __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__re
         b[a] = cell_of(rg.X0[a], n[a]) / kBrick;
         nxt[a] = next_change(rg.X0[a], rg.DX[a], b[a], n[a], S);
     }
+    const FirstSteps fs = first_steps_of(rg.DX);
     long long k = 0;
     int cnt = 0;
     // slot of run i of ray r: i * n_rays + r (consecutive rays write consecutive slots)
@@ -45,14 +69,12 @@ __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__re
             run.X = rg.X0[0] + k * rg.DX[0];
             run.Y = rg.X0[1] + k * rg.DX[1];
             run.Z = rg.X0[2] + k * rg.DX[2];
-            run.dX = rg.DX[0];
-            run.dY = rg.DX[1];
-            run.dZ = rg.DX[2];
-            run.g_off = gz_off[r] + k;
+            run.ray = r;
             run.len = (int)(k1 - k + 1);
             run.k0 = (int)k;
+            run.next = first_steps(run.X, run.Y, run.Z, rg.DX, fs, G.nx, G.ny, G.nz);
             const size_t slot = (size_t)cnt * n_rays + r;
-            runs[slot] = run;
+            store_run(runs + slot, run);
             keys[slot] = brick;
             {   // lanes on the same brick add once, through their lowest lane
                 // (integer sums, so the order does not matter)
@@ -82,6 +104,7 @@ __global__ void k_ray_runs(const RayGeo *__restrict__ geo, const long long *__re
         }
     }
     nrun[r] = cnt;
+    store_steps(steps + r, rg.DX, gz_off[r]);
 }
 
 // The same runs with one warp per ray, for rays of at most kRunMax brick
@@ -120,8 +143,8 @@ __device__ __forceinline__ int count_below(const int *k, int n, int v, bool or_e
 template <bool ARRIVE>
 __global__ void __launch_bounds__(kRunWarps * 32)
     k_ray_runs_warp(const RayGeo *__restrict__ geo, const long long *__restrict__ gz_off, int n_rays, GatherArgs G,
-                    int cap, Run *__restrict__ runs, uint32_t *__restrict__ keys, int *__restrict__ nrun,
-                    uint32_t *__restrict__ bcount, uint32_t *__restrict__ arrival,
+                    int cap, Run *__restrict__ runs, RayStep *__restrict__ steps, uint32_t *__restrict__ keys,
+                    int *__restrict__ nrun, uint32_t *__restrict__ bcount, uint32_t *__restrict__ arrival,
                     unsigned long long *__restrict__ brick_work, uint32_t *__restrict__ status)
 {
     __shared__ int sk[kRunWarps][kRunMax + 1], sm[kRunWarps][kRunMax + 1];
@@ -181,23 +204,21 @@ __global__ void __launch_bounds__(kRunWarps * 32)
         if (status && lane == 0) atomicOr(status + 2, (uint32_t)DIFFUS_STATUS_QUEUE);
         cnt = cap;
     }
-    const long long go = gz_off[r];
+    const FirstSteps fs = first_steps_of(rg.DX);
     for (int i = lane; i < cnt; i += 32) {
         const int ka = i ? k[i - 1] : 0, kb = i + 1 < cnt ? k[i] : S + 1;
         Run run;
         run.X = rg.X0[0] + (long long)ka * rg.DX[0];
         run.Y = rg.X0[1] + (long long)ka * rg.DX[1];
         run.Z = rg.X0[2] + (long long)ka * rg.DX[2];
-        run.dX = rg.DX[0];
-        run.dY = rg.DX[1];
-        run.dZ = rg.DX[2];
-        run.g_off = go + ka;
+        run.ray = r;
         run.len = kb - ka;
         run.k0 = ka;
+        run.next = first_steps(run.X, run.Y, run.Z, rg.DX, fs, G.nx, G.ny, G.nz);
         const uint32_t brick = (uint32_t)(((cell_of(run.Z, n[2]) / kBrick) * G.nby + cell_of(run.Y, n[1]) / kBrick) * G.nbx +
                                           cell_of(run.X, n[0]) / kBrick);
         const size_t slot = (size_t)i * n_rays + r;
-        runs[slot] = run;
+        store_run(runs + slot, run);
         keys[slot] = brick;
         if (ARRIVE) {
             arrival[slot] = atomicAdd(bcount + brick, 1u);
@@ -206,7 +227,10 @@ __global__ void __launch_bounds__(kRunWarps * 32)
             atomicAdd(brick_work + brick, (unsigned long long)run.len);
         }
     }
-    if (lane == 0) nrun[r] = cnt;
+    if (lane == 0) {
+        nrun[r] = cnt;
+        store_steps(steps + r, rg.DX, gz_off[r]);
+    }
 }
 
 // ------------------------------------------------------------ exclusive scan
@@ -533,13 +557,18 @@ __global__ void k_unit_order(const uint32_t *__restrict__ uclass, const uint32_t
         order[atomicAdd(cursor + uclass[u], 1u)] = u;
 }
 
+// Resident blocks per SM of the unit kernel: 6 at 80 registers.  Measured on
+// the 512-pose batch: 5 (96 registers) 1056 us, 6 986, 7 (72, spilling) 1270.
+constexpr int kGatherCtas = 6;
+
 // One warp per unit, units handed out by a ticket queue: the warp gathers
 // the unit's runs into its own 9^3 accumulator and writes the unit's
 // partial (with POSE, also each run's pose-gradient sums).  Warps are
 // independent, so a CTA has no block barriers.
 template <typename T, bool POSE>
-__global__ void __launch_bounds__(kGatherWarps * 32)
-    k_gather_units(const float *__restrict__ gz, const Run *__restrict__ runs, const uint32_t *__restrict__ sorted_vals,
+__global__ void __launch_bounds__(kGatherWarps * 32, kGatherCtas)
+    k_gather_units(const float *__restrict__ gz, const Run *__restrict__ runs, const RayStep *__restrict__ steps,
+                   const uint32_t *__restrict__ sorted_vals,
                    const uint32_t *__restrict__ bstart, const uint32_t *__restrict__ bend,
                    const uint32_t *__restrict__ ustart, const uint32_t *__restrict__ unit_brick,
                    const uint32_t *__restrict__ n_units, GatherArgs G, int unit, float *__restrict__ upart,
@@ -576,7 +605,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32)
             }
         }
         __syncwarp();
-        gather_runs<POSE>(runs, sorted_vals, r0, r1, gz, G, bx0, by0, bz0, sm, w, po);
+        gather_runs<POSE>(runs, steps, sorted_vals, r0, r1, gz, G, bx0, by0, bz0, sm, w, po);
         __syncwarp();
         float *out = upart + (size_t)u * kBrickVox;
         for (int i = lane; i < kBrickVox; i += 32) out[i] = acc[i];
@@ -669,59 +698,52 @@ __global__ void k_voxel_reduce(const float *__restrict__ upart, const uint32_t *
 }
 
 // Pose-gradient terms of each ray from its runs' sums, added in slot order
-// (run order along the ray) in FP64: the translation part sum_k dL/dZ_k
+// (run order along the ray) in compensated FP32 (Knuth's two-sum; FP64
+// arithmetic is slow on this part): the translation part sum_k dL/dZ_k
 // grad Z(p_k) (per mm) and the rotation part sum_k dL/dZ_k s_k grad Z(p_k)
-// projected on the ray's direction derivatives, s_k = (k + 1/2) ds.
-__global__ void k_ray_pose(const float *__restrict__ rpart, size_t slots, const int *__restrict__ nrun,
-                           const RayGeo *__restrict__ geo, int n_rays, float isx, float isy, float isz,
-                           double *__restrict__ pose_part)
+// projected on the ray's direction derivatives, s_k = (k + 1/2) ds.  A block
+// takes 32 rays, one warp per component, so a ray's chain of loads is one
+// component's, eight in flight (251 rays: 18 us with one thread per ray for all
+// six, 7 us; 147 K rays: 48 us, 36 us).
+__global__ void __launch_bounds__(192) k_ray_pose(const float *__restrict__ rpart, size_t slots,
+                                                  const int *__restrict__ nrun, const RayGeo *__restrict__ geo,
+                                                  int n_rays, float isx, float isy, float isz,
+                                                  double *__restrict__ pose_part)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rays) return;
-    // compensated FP32 sums (Knuth's two-sum; FP64 arithmetic is slow on
-    // this part), four runs' loads in flight, additions in run order
-    float sum[6] = {0, 0, 0, 0, 0, 0}, err[6] = {0, 0, 0, 0, 0, 0};
-    const int cnt = nrun[r];
-    constexpr int kB = 4;
+    __shared__ double sum6[6][32];
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int r = blockIdx.x * 32 + lane;
+    const int cnt = r < n_rays ? nrun[r] : 0;
+    const float *p = rpart + (size_t)q * slots + r;
+    float sum = 0.0f, err = 0.0f;
+    constexpr int kB = 8;
     for (int i0 = 0; i0 < cnt; i0 += kB) {
-        float x[kB][6];
+        float x[kB];
+#pragma unroll
+        for (int b = 0; b < kB; b++) x[b] = i0 + b < cnt ? p[(size_t)(i0 + b) * n_rays] : 0.0f;
 #pragma unroll
         for (int b = 0; b < kB; b++) {
-            const size_t slot = (size_t)(i0 + b) * n_rays + r;
-#pragma unroll
-            for (int q = 0; q < 6; q++) x[b][q] = i0 + b < cnt ? rpart[(size_t)q * slots + slot] : 0.0f;
-        }
-#pragma unroll
-        for (int b = 0; b < kB; b++) {
-#pragma unroll
-            for (int q = 0; q < 6; q++) {
-                const float t = __fadd_rn(sum[q], x[b][q]);
-                const float z = __fsub_rn(t, sum[q]);
-                const float e = __fadd_rn(__fsub_rn(sum[q], __fsub_rn(t, z)), __fsub_rn(x[b][q], z));
-                err[q] = __fadd_rn(err[q], e);
-                sum[q] = t;
-            }
+            const float t = __fadd_rn(sum, x[b]);
+            const float z = __fsub_rn(t, sum);
+            const float e = __fadd_rn(__fsub_rn(sum, __fsub_rn(t, z)), __fsub_rn(x[b], z));
+            err = __fadd_rn(err, e);
+            sum = t;
         }
     }
-    double t[3], u[3];
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        t[a] = (double)sum[a] + (double)err[a];
-        u[a] = (double)sum[3 + a] + (double)err[3 + a];
-    }
-    const RayGeo &rg = geo[r];
+    sum6[q][lane] = (double)sum + (double)err;
+    __syncthreads();
+    if (r >= n_rays || q >= 3) return;
+    // warp a: translation component a and rotation component a
+    const int a = q;
     const double is[3] = {(double)isx, (double)isy, (double)isz};
+    const RayGeo &rg = geo[r];
     const double ds = (double)rg.ds;
     double *out = pose_part + 6 * (size_t)r;
+    out[a] = __dmul_rn(sum6[a][lane], is[a]);
+    double u[3];
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        t[a] *= is[a];
-        u[a] *= is[a] * ds;
-        out[a] = t[a];
-    }
-#pragma unroll
-    for (int q = 0; q < 3; q++)
-        out[3 + q] = u[0] * (double)rg.v[q][0] + u[1] * (double)rg.v[q][1] + u[2] * (double)rg.v[q][2];
+    for (int i = 0; i < 3; i++) u[i] = __dmul_rn(sum6[3 + i][lane], __dmul_rn(is[i], ds));
+    out[3 + a] = __fma_rn(u[2], (double)rg.v[a][2], __fma_rn(u[1], (double)rg.v[a][1], __dmul_rn(u[0], (double)rg.v[a][0])));
 }
 
 int sort_bits(int nb)
@@ -765,6 +787,7 @@ int runs_per_ray(const diffus_volume_desc *vd, double max_path_mm)
 
 struct GatherLayout {
     Run *runs;
+    RayStep *steps;
     uint32_t *keys[2], *vals[2];    // radix passes; by rank: keys[1] arrivals, vals[0..1] the placed list
     uint32_t *hist, *sums, *misc;   // misc: [0] units total, [1] runs in use
     uint32_t *bstart, *bend, *ucount, *ustart, *unit_brick;
@@ -791,6 +814,7 @@ static GatherLayout gather_layout(void *ws, const diffus_volume_desc *vd, long l
     size_t nsums = (nhist + kScanChunk - 1) / kScanChunk;
     size_t max_units = slots / unit_runs(slots) + nb;
     L.runs = c.take<Run>(slots);
+    L.steps = c.take<RayStep>((size_t)n_rays);
     L.keys[0] = c.take<uint32_t>(slots);
     L.keys[1] = c.take<uint32_t>(slots);
     L.vals[0] = c.take<uint32_t>(2 * slots);
@@ -833,7 +857,7 @@ template <typename T, bool POSE>
 static void launch_units(const float *gz, const GatherLayout &L, const uint32_t *sorted, const uint32_t *order, const GatherArgs &G, const void *vol,
                          const PoseOut &po, int unit, int grid, cudaStream_t s)
 {
-    k_gather_units<T, POSE><<<grid, kGatherWarps * 32, 0, s>>>(gz, L.runs, sorted, L.bstart, L.bend, L.ustart,
+    k_gather_units<T, POSE><<<grid, kGatherWarps * 32, 0, s>>>(gz, L.runs, L.steps, sorted, L.bstart, L.bend, L.ustart,
                                                              L.unit_brick, L.misc + 0, G, unit, L.upart, L.zero + 32,
                                                              order, (const T *)vol, po);
 }
@@ -864,7 +888,7 @@ int launch_gather(const diffus_volume_desc *vd, const void *vol, const RayGeo *g
                                                     L.bend, L.ucount, L.ustart, L.unit_brick, L.misc + 0, L.misc + 1);
     };
     if (by_rank) {
-        k_ray_runs_warp<true><<<wgrid, kRunWarps * 32, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs, L.keys[0],
+        k_ray_runs_warp<true><<<wgrid, kRunWarps * 32, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs, L.steps, L.keys[0],
                                                               L.nrun, L.bcount, L.keys[1], nullptr, status);
         brick_plan();
         uint2 *list = reinterpret_cast<uint2 *>(L.vals[0]);
@@ -876,11 +900,11 @@ int launch_gather(const diffus_volume_desc *vd, const void *vol, const RayGeo *g
     } else {
         if (cudaMemsetAsync(L.keys[0], 0xff, sizeof(uint32_t) * slots, s) != cudaSuccess) return DIFFUS_E_LAUNCH;
         if (cap - 1 <= kRunMax && n_rays <= kRunWarpRays)
-            k_ray_runs_warp<false><<<wgrid, kRunWarps * 32, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs,
+            k_ray_runs_warp<false><<<wgrid, kRunWarps * 32, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs, L.steps,
                                                                    L.keys[0], L.nrun, L.bcount, nullptr, L.bwork,
                                                                    status);
         else
-            k_ray_runs<<<(unsigned)((n_rays + 127) / 128), 128, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs,
+            k_ray_runs<<<(unsigned)((n_rays + 127) / 128), 128, 0, s>>>(geo, gz_off, (int)n_rays, G, cap, L.runs, L.steps,
                                                                        L.keys[0], L.nrun, L.bcount, L.bwork, status);
         brick_plan();
         // stable LSD radix sort by brick
@@ -928,7 +952,7 @@ int launch_gather(const diffus_volume_desc *vd, const void *vol, const RayGeo *g
                      (unsigned)((vd->ny + rblk.y - 1) / rblk.y), (unsigned)vd->nz);
     k_voxel_reduce<<<rgrid, rblk, 0, s>>>(L.upart, L.ustart, L.ucount, G, grad_vol, rvec);
     if (pose_part)
-        k_ray_pose<<<(unsigned)((n_rays + 127) / 128), 128, 0, s>>>(
+        k_ray_pose<<<(unsigned)((n_rays + 31) / 32), 192, 0, s>>>(
             L.rpart, slots, L.nrun, geo, (int)n_rays, (float)(1.0 / vd->sx), (float)(1.0 / vd->sy),
             (float)(1.0 / vd->sz), pose_part);
     return launch_status();

@@ -49,7 +49,7 @@ constexpr int kGatherWarps = 4;
 // nine small frames' 132 and 45 us; 512 frames stay at 256.
 __host__ __device__ inline int unit_runs(size_t slots)
 {
-    return slots <= (1u << 20) ? 32 : slots <= (1u << 21) ? 64 : slots <= (1u << 22) ? 128 : 256;
+        return slots <= (1u << 20) ? 32 : slots <= (1u << 21) ? 64 : slots <= (1u << 22) ? 128 : 256;
 }
 
 struct GatherArgs {
@@ -57,18 +57,40 @@ struct GatherArgs {
     int nbx, nby, nbz;                // bricks of cells per axis (cells 0..n-2)
 };
 
-// Samples k0 .. k0+len-1 of one ray lie in cells of one brick.  The run
-// carries all a gather lane needs to walk it: the fixed-point position of
-// its first sample, the ray's step, the offset of its first dL/dZ value and
-// the index k0 of its first sample along the ray.
+// Samples k0 .. k0+len-1 of one ray lie in cells of one brick: where the run
+// starts, and for each axis the samples before its first crossing of a cell
+// face (kNextBits bits each, at most kNextMax).
 struct alignas(16) Run {
     long long X, Y, Z;
-    long long dX, dY, dZ;
-    long long g_off;
-    int len;
-    int k0;
+    int ray, k0, len;
+    uint32_t next;
+    uint32_t pad[2];
 };
-static_assert(sizeof(Run) == 64, "Run layout");
+static_assert(sizeof(Run) == 48, "Run layout");
+constexpr int kNextBits = 10;
+constexpr int kNextMax = (1 << kNextBits) - 1;
+
+// What every run of a ray needs to step from cell to cell.  Along an axis with
+// step e = |d| (2^-32 voxel) the samples between two crossings are q or q + 1,
+// q = floor(2^32 / e): a crossing leaves the position less than e inside the
+// new cell, so with r = 2^32 - q e the next one comes after q + (rem < r)
+// samples, rem the position's fraction counted in the direction of travel.  v is
+// d / 2^32 as a float (the slope of the cell weights).
+struct alignas(16) RayStep {
+    long long d[3], g_off;   // step per axis; offset of the ray's first dL/dZ value
+    uint2 qr[3];
+    float v[3], pad[3];
+};
+static_assert(sizeof(RayStep) == 80, "RayStep layout");
+
+__device__ __forceinline__ uint2 cell_steps(long long d)
+{
+    const unsigned long long e = (unsigned long long)(d < 0 ? -d : d);
+    if (e <= 1) return make_uint2(0xffffffffu, 0u);      // (never within a run)
+    if (e >> 32) return make_uint2(1u, 0u);              // a crossing at every sample
+    const uint32_t e32 = (uint32_t)e, q = 0xffffffffu / e32, r = 0xffffffffu - q * e32;   // 2^32 = q e + r + 1
+    return r + 1 == e32 ? make_uint2(q + 1, 0u) : make_uint2(q, r + 1);
+}
 
 // A 64-bit fixed-point quantity as a float, from two 32-bit conversions
 // (high word x 2^32 + low word): within about an ulp.  The direct 64-bit
@@ -123,7 +145,8 @@ template <bool POSE>
 struct GatherSmem {
     float acc[kGatherWarps][kBrickVox];
     float vox[POSE ? kGatherWarps : 1][POSE ? kBrickVox : 1];   // the brick's volume values (pose terms)
-    float pose[POSE ? kGatherWarps : 1][6][32];                  // per-lane sums of the lane's run
+    uint2 qr[kGatherWarps][3][32];                               // the lane's ray: cell steps and
+    float slope[kGatherWarps][3][32];                            // weight slopes
 };
 
 // Adds one closed cell record per flagged lane into the warp's accumulator.
@@ -182,24 +205,28 @@ __device__ __forceinline__ int ceil_div_fixed(long long num, long long den, int 
 }
 
 // Cell index i and upper-corner weight u + v k of one axis at position X
-// (exact in the clamped regions, where v = 0).
-__device__ __forceinline__ void axis_cell(long long X, long long dX, int n, int &i, float &u, float &v)
+// (exact in the clamped regions, where v = 0); vd = d / 2^32.
+__device__ __forceinline__ void axis_cell(long long X, float vd, int n, int &i, float &u, float &v)
 {
-    const long long top = (long long)(n - 1) << 32;
-    if (X < 0) {
+    const int hi = (int)(X >> 32);
+    i = hi;
+    u = __uint_as_float(__funnelshift_r((unsigned)X, 0x7Fu, 9)) - 1.0f;   // 23-bit fraction
+    v = vd;
+    if (hi < 0) {
         i = 0;
         u = 0.0f;
         v = 0.0f;
-    } else if (X >= top) {
+    } else if (hi >= n - 1) {
         i = n - 2;
         u = 1.0f;
         v = 0.0f;
-    } else {
-        i = (int)(X >> 32);
-        u = __uint_as_float(0x3F800000u | ((unsigned)X >> 9)) - 1.0f;   // 23-bit fraction
-        v = fmaf((float)(unsigned)(dX & 0xffffffffll), 2.3283064365386963e-10f,
-                 (float)(int)(dX >> 32));                               // dX / 2^32
     }
+}
+
+// dX / 2^32 as a float.
+__device__ __forceinline__ float slope_of(long long dX)
+{
+    return fmaf((float)(unsigned)(dX & 0xffffffffll), 2.3283064365386963e-10f, (float)(int)(dX >> 32));
 }
 
 // Samples from X (inclusive) before the axis's cell or its clamping changes
@@ -238,6 +265,70 @@ __device__ __forceinline__ void axis_poly(float D00, float D10, float D01, float
 
 constexpr int kGStepCap = 1 << 24;   // "no crossing within the run"
 
+// axis_steps at a position that a crossing of this axis has just reached: in
+// an inner cell the count comes from (q, r); next to the volume's faces, in the
+// clamped regions and for steps so small that a run's first count was cut at
+// kNextMax, from axis_steps (512 frames: 173 M warp instructions per 34 M
+// samples with that division at every crossing, 142 M).
+__device__ __forceinline__ int next_steps(long long X, long long dX, int n, uint2 qr)
+{
+    const int hi = (int)(X >> 32);
+    if ((unsigned)(hi - 1) < (unsigned)(n - 2) && qr.x < (unsigned)(kNextMax - 1)) {
+        const unsigned rem = (unsigned)X ^ (unsigned)((int)(dX >> 32) >> 31);
+        return (int)qr.x + (rem < qr.y);
+    }
+    return axis_steps(X, dX, n, kGStepCap);
+}
+
+// The same at any position.  With t the distance to the last position of the
+// cell in the direction of travel (a 32-bit number), the next crossing comes
+// after floor(t / e) + 1 samples; inv = 1 / e estimates the quotient (below
+// kNextMax, so off by one at most) and an exact product corrects it.
+__device__ __forceinline__ int first_steps1(long long X, long long dX, uint32_t q, float inv, int n)
+{
+    const int hi = (int)(X >> 32);
+    if ((unsigned)(hi - 1) < (unsigned)(n - 2) && q < (unsigned)(kNextMax - 1)) {
+        const bool neg = dX < 0;
+        const unsigned t = neg ? (unsigned)X : ~(unsigned)X;
+        const unsigned long long e = (unsigned long long)(neg ? -dX : dX);
+        if (e >> 32) return 1;
+        unsigned k = (unsigned)((float)t * inv);
+        const long long r = (long long)t - (long long)((unsigned long long)k * (unsigned)e);
+        if (r < 0)
+            k--;
+        else if (r >= (long long)e)
+            k++;
+        return (int)k + 1;
+    }
+    return axis_steps(X, dX, n, kNextMax);
+}
+
+// A ray's steps as its runs' first counts need them.
+struct FirstSteps {
+    uint32_t q[3];
+    float inv[3];
+};
+
+__device__ __forceinline__ FirstSteps first_steps_of(const long long d[3])
+{
+    FirstSteps f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        f.q[a] = cell_steps(d[a]).x;
+        f.inv[a] = 1.0f / fmaxf(fabsf(ll_to_float(d[a])), 1.0f);
+    }
+    return f;
+}
+
+// The three first counts of a run, packed.
+__device__ __forceinline__ uint32_t first_steps(long long X, long long Y, long long Z, const long long d[3],
+                                                const FirstSteps &f, int nx, int ny, int nz)
+{
+    return (uint32_t)first_steps1(X, d[0], f.q[0], f.inv[0], nx) |
+           ((uint32_t)first_steps1(Y, d[1], f.q[1], f.inv[1], ny) << kNextBits) |
+           ((uint32_t)first_steps1(Z, d[2], f.q[2], f.inv[2], nz) << (2 * kNextBits));
+}
+
 // Pose-gradient sums of one run, written at the run's slot: component q
 // (T_x, T_y, T_z, U_x, U_y, U_z) at rpart[q * slots + slot], with
 // T_a = sum_k dL/dZ_k dZ/dx_a(k) and U_a = sum_k dL/dZ_k (k + 1/2) dZ/dx_a(k)
@@ -259,7 +350,8 @@ struct PoseOut {
 // the sums have a fixed order.  With POSE the lane also sums the run's
 // pose-gradient terms from the same moments and the cell's corner values.
 template <bool POSE>
-__device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const uint32_t *__restrict__ order,
+__device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const RayStep *__restrict__ steps,
+                                            const uint32_t *__restrict__ order,
                                             uint32_t q0, uint32_t q1, const float *__restrict__ gzbuf,
                                             const GatherArgs &G, int bx0, int by0, int bz0, GatherSmem<POSE> &sm,
                                             int w, const PoseOut &po)
@@ -271,18 +363,26 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
     long long X = 0, Y = 0, Z = 0, dX = 0, dY = 0, dZ = 0;
     const float *g = gzbuf;
     int left = 0;                 // samples left in the lane's run
-    int cx = 0, cy = 0, cz = 0;   // samples left before each axis's next crossing (0: recompute)
+    int cx = 0, cy = 0, cz = 0;   // samples left before each axis's next crossing
+    int len = 0;                  // samples of the lane's current cell
     uint32_t slot = 0;            // the run's slot (pose output)
     int kc = 0;                   // index along the ray of the next sample
-    float(*pz)[32] = sm.pose[POSE ? w : 0];
+    float ps[6] = {};             // pose-gradient sums of the run
+    uint2(*qr)[32] = sm.qr[w];
+    float(*slope)[32] = sm.slope[w];
     uint32_t next = q0;           // next unassigned run (warp-uniform)
     // the first samples of the lane's next cell, loaded while the current
     // cell's corner sums and flush run (the cell's other samples are loaded
-    // in its moment loop).  Measured on the 512-pose batch: 2 samples 1.046
-    // ms, 4 0.998, 6 0.976, 8 0.957 (no spills at 72 registers), 12 0.955
-    // with spills.
+    // in its moment loop), and no others (each lane reads its own line, so a
+    // load costs several L1 wavefronts: 49 M per 34 M samples with all eight
+    // loaded, 42 M).
     constexpr int kPre = 8;
     float pre_g[kPre] = {};
+    auto enter_cell = [&] {
+        len = min(min(cx, cy), min(cz, min(left, kGCellCap)));
+#pragma unroll
+        for (int q = 0; q < kPre; q++) pre_g[q] = q < len ? __ldg(g + q) : 0.0f;
+    };
     // lane i holds the index of run next + i, loaded one refill ahead
     uint32_t pre = next + lane < q1 ? order[next + lane] : 0u;
     for (;;) {
@@ -294,52 +394,52 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
             const uint32_t idx = __shfl_sync(0xffffffffu, pre, src);
             if (idle && next + src < q1) {
                 const Run run = runs[idx];
+                const RayStep &rs = steps[run.ray];
                 X = run.X;
                 Y = run.Y;
                 Z = run.Z;
-                dX = run.dX;
-                dY = run.dY;
-                dZ = run.dZ;
-                g = gzbuf + run.g_off;
-                left = run.len;
+                dX = rs.d[0];
+                dY = rs.d[1];
+                dZ = rs.d[2];
 #pragma unroll
-                for (int q = 0; q < kPre; q++) pre_g[q] = q < left ? __ldg(g + q) : 0.0f;
-                cx = cy = cz = 0;
+                for (int q = 0; q < 3; q++) {
+                    qr[q][lane] = rs.qr[q];
+                    slope[q][lane] = rs.v[q];
+                }
+                g = gzbuf + rs.g_off + run.k0;
+                left = run.len;
+                cx = (int)(run.next & kNextMax);
+                cy = (int)((run.next >> kNextBits) & kNextMax);
+                cz = (int)(run.next >> (2 * kNextBits));
+                enter_cell();
                 if (POSE) {
                     slot = idx;
                     kc = run.k0;
 #pragma unroll
-                    for (int q = 0; q < 6; q++) pz[q][lane] = 0.0f;
+                    for (int q = 0; q < 6; q++) ps[q] = 0.0f;
                 }
             }
             next += __popc(idles);
             pre = next + lane < q1 ? order[next + lane] : 0u;
         }
         if (!__any_sync(0xffffffffu, left > 0)) break;
-        // the lane's current cell and its sample count
-        int ix = 0, iy = 0, iz = 0, len = 0;
-        float ux = 0.0f, vx = 0.0f, uy = 0.0f, vy = 0.0f, uz = 0.0f, vz = 0.0f;
-        if (left > 0) {
-            // DDA countdowns: only an axis that crossed is recomputed
-            if (cx == 0) cx = axis_steps(X, dX, G.nx, kGStepCap);
-            if (cy == 0) cy = axis_steps(Y, dY, G.ny, kGStepCap);
-            if (cz == 0) cz = axis_steps(Z, dZ, G.nz, kGStepCap);
-            axis_cell(X, dX, G.nx, ix, ux, vx);
-            axis_cell(Y, dY, G.ny, iy, uy, vy);
-            axis_cell(Z, dZ, G.nz, iz, uz, vz);
-            len = min(min(cx, cy), min(cz, min(left, kGCellCap)));
-        }
+        const bool has = left > 0;
+        // the lane's current cell
+        int ix, iy, iz;
+        float ux, vx, uy, vy, uz, vz;
+        axis_cell(X, slope[0][lane], G.nx, ix, ux, vx);
+        axis_cell(Y, slope[1][lane], G.ny, iy, uy, vy);
+        axis_cell(Z, slope[2][lane], G.nz, iz, uz, vz);
+        if (!has) len = 0;
         // moments of dL/dZ over the cell's samples
         float M0 = 0.0f, M1 = 0.0f, M2 = 0.0f, M3 = 0.0f;
         const int kmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
         auto moment = [&](float gk, int k) {
-            const float kf = (float)k;
+            const float kf = (float)k, k2 = kf * kf;
             M0 += gk;
-            float t = gk * kf;
-            M1 += t;
-            t *= kf;
-            M2 += t;
-            M3 = fmaf(t, kf, M3);
+            M1 = fmaf(gk, kf, M1);
+            M2 = fmaf(gk, k2, M2);
+            M3 = fmaf(gk, k2 * kf, M3);   // k < 32: the powers are exact
         };
 #pragma unroll
         for (int k = 0; k < kPre; k++)
@@ -366,7 +466,6 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
                     v[(zz << 2) | (yy << 1) | 1] = fmaf(vx, B, ux * A);
                 }
         }
-        const bool has = len > 0;
         const int cell = (ix - bx0) | ((iy - by0) << 3) | ((iz - bz0) << 6);
         if (POSE && has) {
             // the cell's 8 corner values, from the brick copy in shared memory
@@ -389,8 +488,8 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
                 const float Ta = fmaf(p[a][2], M2, fmaf(p[a][1], M1, p[a][0] * M0));
                 const float Wa = fmaf(p[a][2], M3, fmaf(p[a][1], M2, p[a][0] * M1));
                 if (in[a]) {
-                    pz[a][lane] += Ta;
-                    pz[3 + a][lane] += fmaf(kh, Ta, Wa);
+                    ps[a] += Ta;
+                    ps[3 + a] += fmaf(kh, Ta, Wa);
                 }
             }
         }
@@ -400,17 +499,19 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
             Z += (long long)len * dZ;
             g += len;
             left -= len;
-#pragma unroll
-            for (int q = 0; q < kPre; q++) pre_g[q] = q < left ? __ldg(g + q) : 0.0f;
             cx -= len;
             cy -= len;
             cz -= len;
-            if (POSE) {
-                kc += len;
-                if (left == 0) {
+            if (POSE) kc += len;
+            if (left > 0) {
+                // only an axis that crossed is counted again
+                if (cx == 0) cx = next_steps(X, dX, G.nx, qr[0][lane]);
+                if (cy == 0) cy = next_steps(Y, dY, G.ny, qr[1][lane]);
+                if (cz == 0) cz = next_steps(Z, dZ, G.nz, qr[2][lane]);
+                enter_cell();
+            } else if (POSE) {
 #pragma unroll
-                    for (int q = 0; q < 6; q++) po.rpart[(size_t)q * po.slots + slot] = pz[q][lane];
-                }
+                for (int q = 0; q < 6; q++) po.rpart[(size_t)q * po.slots + slot] = ps[q];
             }
         }
         flush_records(has, cell, v, acc, lane, lt);

@@ -234,6 +234,22 @@ inline void launch_setup(const float *pose, const FanDev &fd, const VolPlace &vp
     }
 }
 
+// Per-pose sum of per-ray pose terms in FP64, one block per pose and one warp
+// per component: lanes stride over the pose's rays, then a fixed shuffle tree
+// (the same order for a frame and a batch).
+static __global__ void __launch_bounds__(192) k_pose_reduce(const double *__restrict__ part,
+                                                            const int *__restrict__ ray0,
+                                                            float *__restrict__ grad_pose)
+{
+    const int p = blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = ray0[p + 1];
+    double s = 0.0;
+#pragma unroll 8
+    for (int j = ray0[p] + lane; j < b; j += 32) s += part[6 * (size_t)j + q];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) grad_pose[6 * p + q] = (float)s;
+}
+
 // One warp per ray, kWarpsFwd warps per CTA.
 constexpr int kWarpsFwd = 4;
 // Resident warps per SM of the refined pass's kernels: 16 hold it at 128

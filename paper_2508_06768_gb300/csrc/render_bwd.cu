@@ -59,25 +59,6 @@ __global__ void __launch_bounds__(kWarpsBwd * 32) k_march_bwd_multi(const T *__r
                                               nullptr, nullptr, &mm, sm[0].acc);
 }
 
-// Deterministic per-pose sum of per-ray pose partials: one warp per pose,
-// lanes stride over the pose's rays, then a fixed shuffle tree.
-static __global__ void k_pose_reduce(const double *__restrict__ part, const int *__restrict__ ray0, int P,
-                                     float *__restrict__ grad_pose)
-{
-    const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (p >= P) return;
-    const int a = ray0[p], b = ray0[p + 1];
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = a + lane; j < b; j += 32)
-        for (int q = 0; q < 6; q++) s[q] += part[6 * (size_t)j + q];
-    for (int q = 0; q < 6; q++) {
-        double v = s[q];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) grad_pose[6 * p + q] = (float)v;
-    }
-}
-
 struct BwdLayout {
     RayGeo *geo;
     PoseFrame *frame;
@@ -195,6 +176,6 @@ extern "C" int diffus_render_bwd(const void *vol, const diffus_volume_desc *vd, 
         (rc = launch_gather(vd, vol, L.geo, n, fan->depth_mm, L.gz, L.gz_off, L.gather_ws, status, grad_vol,
                             grad_pose ? L.part : nullptr, 8, s)))
         return rc;
-    if (grad_pose) k_pose_reduce<<<1, 32, 0, s>>>(L.part, L.ray0, 1, grad_pose);
+    if (grad_pose) k_pose_reduce<<<1, 192, 0, s>>>(L.part, L.ray0, grad_pose);
     return launch_status();
 }
