@@ -182,9 +182,8 @@ __global__ void k_batch_setup(const PoseFrame *__restrict__ frames, BatchDev B, 
     if (r >= B.total_rays) return;
     const int p = B.ray_pose[r];
     const PlanPose pp = B.pose[p];
-    FanDev fd{pp.n_rays, pp.S, pp.fov, pp.depth};
     RayGeo rg;
-    setup_ray(frames[p], p, B.ray_j[r], fd, vp, rg);
+    setup_ray(frames[p], p, B.ray_j[r], pp.fan, vp, rg);
     geo[r] = rg;
 }
 
@@ -419,7 +418,7 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
         double a = attenuation_a(&f);
         float hi, lo;
         gain_l2(a, hi, lo);
-        pp[p] = PlanPose{f.n_rays, f.n_samples, f.fov_rad, f.depth_mm, (float)(a * a), H.blurW, img, a * a, hi, lo, ld, 0,
+        pp[p] = PlanPose{f.n_rays, f.n_samples, make_fan(f.n_rays, f.n_samples, f.fov_rad, f.depth_mm), (float)(a * a), H.blurW, img, a * a, hi, lo, ld, 0,
                          pad};
         depth[p] = f.depth_mm;
         ray0[p] = (int32_t)r;

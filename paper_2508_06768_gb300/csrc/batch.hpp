@@ -9,7 +9,7 @@ namespace dfs {
 
 struct PlanPose {
     int32_t n_rays, S;
-    double fov, depth;
+    FanDev fan;
     float a2;
     int32_t W;
     int64_t img_off;

@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(WARPS * 32, kRefineWarpsPerSM / WARPS) k_batch
             Ap.a2 = pp.a2;
             Ap.a2d = pp.a2d;
         }
-        const FanDev fd{pp.n_rays, pp.S, pp.fov, pp.depth};
+        const FanDev &fd = pp.fan;
         RayOut o{out + (padded ? B.pad_off[r] : B.row_off[r]), valid ? valid + r : nullptr, status,
                  ckpt ? ckpt + B.ck_off[r] : nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, r, padded};
         refine_ray<T, true>(vol, Ap, rg, frames[rg.pose], fd, vp, o, sel.rinfo[r], buf[w], dbuf[w]);

@@ -127,7 +127,7 @@ inline VolGeo make_volgeo(const diffus_volume_desc *vd)
 
 inline VolPlace make_place(const diffus_volume_desc *vd)
 {
-    return {vd->sx, vd->sy, vd->sz, vd->ox, vd->oy, vd->oz};
+    return {1.0 / vd->sx, 1.0 / vd->sy, 1.0 / vd->sz, vd->ox, vd->oy, vd->oz};
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }

@@ -5,13 +5,23 @@
 
 namespace dfs {
 
+// A fan and the volume's placement as the ray setup needs them: the steps of
+// depth and beam angle and the reciprocal spacings come from the host, because
+// an FP64 division is some forty instructions on a pipe that takes 16 clocks
+// for each (147 K rays: 53 us with the divisions, 33 us; a frame's setup 7.0 and
+// 6.2 us).
 struct FanDev {
     int n_rays, S;
-    double fov, depth;
+    double half_fov, dth, ds;
 };
 
+inline FanDev make_fan(int n_rays, int S, double fov, double depth)
+{
+    return {n_rays, S, n_rays > 1 ? 0.5 * fov : 0.0, n_rays > 1 ? fov / (double)(n_rays - 1) : 0.0, depth / (double)S};
+}
+
 struct VolPlace {
-    double sx, sy, sz, ox, oy, oz;
+    double isx, isy, isz, ox, oy, oz;
 };
 
 // Rotation R = Rz Ry Rx of ZYX Euler angles and its three partial
@@ -92,31 +102,27 @@ static __global__ void k_pose_frames(const float *__restrict__ poses, int P, Pos
 
 // FP64 voxel coordinates of sample 0 of ray `ray` and the step between
 // samples (Section 2.4): sample k lies at x0 + k dx = (t + (k + 1/2) ds u -
-// origin) / spacing.  st, ct: sin and cos of the beam angle.
+// origin) / spacing (times the FP64 reciprocal).  st, ct: sin and cos of the beam angle.
 __device__ __forceinline__ void beam_sincos(int ray, const FanDev &fan, double &st, double &ct)
 {
-    const double th = fan.n_rays > 1 ? __fma_rn(-0.5, fan.fov, __ddiv_rn(__dmul_rn(fan.fov, (double)ray),
-                                                                         (double)(fan.n_rays - 1)))
-                                     : 0.0;
-    sincos(th, &st, &ct);
+    sincos(__fma_rn((double)ray, fan.dth, -fan.half_fov), &st, &ct);
 }
 
 // One axis of the line: Rc, t: the pose frame's row of that axis.
-__device__ __forceinline__ void axis_line(const double Rc[2], double t, double ds, double sp, double org, double st,
+__device__ __forceinline__ void axis_line(const double Rc[2], double t, double ds, double isp, double org, double st,
                                           double ct, double &x0, double &dx)
 {
     const double u = __fma_rn(Rc[0], st, __dmul_rn(Rc[1], ct));
-    x0 = __ddiv_rn(__dsub_rn(__fma_rn(__dmul_rn(0.5, ds), u, t), org), sp);
-    dx = __ddiv_rn(__dmul_rn(ds, u), sp);
+    x0 = __dmul_rn(__dsub_rn(__fma_rn(__dmul_rn(0.5, ds), u, t), org), isp);
+    dx = __dmul_rn(__dmul_rn(ds, u), isp);
 }
 
 __device__ __forceinline__ void ray_line(const PoseFrame &f, int ray, const FanDev &fan, const VolPlace &vp,
                                          double x0[3], double dx[3], double &st, double &ct)
 {
     beam_sincos(ray, fan, st, ct);
-    const double ds = __ddiv_rn(fan.depth, (double)fan.S);
-    const double sp[3] = {vp.sx, vp.sy, vp.sz}, org[3] = {vp.ox, vp.oy, vp.oz};
-    for (int i = 0; i < 3; i++) axis_line(f.Rc[i], f.t[i], ds, sp[i], org[i], st, ct, x0[i], dx[i]);
+    const double isp[3] = {vp.isx, vp.isy, vp.isz}, org[3] = {vp.ox, vp.oy, vp.oz};
+    for (int i = 0; i < 3; i++) axis_line(f.Rc[i], f.t[i], fan.ds, isp[i], org[i], st, ct, x0[i], dx[i]);
 }
 
 __device__ __forceinline__ long long step_fixed(double dx) { return __double2ll_rn(__dmul_rn(dx, 4294967296.0)); }
@@ -142,15 +148,14 @@ __device__ __forceinline__ void setup_ray(const PoseFrame &f, int pose_idx, int 
     out.pose = pose_idx;
     out.ray = ray;
     out.S = fan.S;
-    out.ds = (float)__ddiv_rn(fan.depth, (double)fan.S);
+    out.ds = (float)fan.ds;
 }
 
 // Setup of one pose's rays in one launch: the pose frame, the ray table and
 // (rows not null) the offsets that the backward's kernels read.  FP64 runs at
 // two operations per clock and SM, so a warp's FP64 instruction takes 16 clocks
 // whatever its lanes do: a block takes ten rays with one lane per ray and
-// axis (two divisions in series instead of six) while a second warp works out
-// the pose frame.  Frame kernel, ray kernel and offset kernel took 6.5 + 8.5 +
+// axis while a second warp works out the pose frame.  Frame kernel, ray kernel and offset kernel took 6.5 + 8.5 +
 // 2 us for a frame; this one 7.0 us.  Above kSetupFrameRays rays the blocks'
 // repeated pose frames cost more than the separate kernel.
 constexpr int kSetupRays = 10;
@@ -195,9 +200,8 @@ static __global__ void __launch_bounds__(64) k_setup_frame(const float *__restri
     }
     __syncthreads();
     if (w == 1 || !on) return;
-    const double ds = __ddiv_rn(fan.depth, (double)fan.S);
     double x0, dx;
-    axis_line(f.Rc[a], f.t[a], ds, a == 0 ? vp.sx : (a == 1 ? vp.sy : vp.sz), a == 0 ? vp.ox : (a == 1 ? vp.oy : vp.oz),
+    axis_line(f.Rc[a], f.t[a], fan.ds, a == 0 ? vp.isx : (a == 1 ? vp.isy : vp.isz), a == 0 ? vp.ox : (a == 1 ? vp.oy : vp.oz),
               st, ct, x0, dx);
     RayGeo &g = geo[j];
     g.X0[a] = to_fixed(x0);
@@ -207,7 +211,7 @@ static __global__ void __launch_bounds__(64) k_setup_frame(const float *__restri
         g.pose = 0;
         g.ray = j;
         g.S = fan.S;
-        g.ds = (float)ds;
+        g.ds = (float)fan.ds;
         if (off.row) write_offsets(off, j, fan.n_rays, fan.S);
     }
 }

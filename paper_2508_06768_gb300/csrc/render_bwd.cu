@@ -153,7 +153,7 @@ extern "C" int diffus_render_bwd(const void *vol, const diffus_volume_desc *vd, 
     cudaStream_t s = (cudaStream_t)stream;
     if (status && cudaMemsetAsync(status, 0, 4 * sizeof(uint32_t), s) != cudaSuccess) return DIFFUS_E_LAUNCH;
     const int n = fan->n_rays, S = fan->n_samples;
-    FanDev fd{n, S, fan->fov_rad, fan->depth_mm};
+    const FanDev fd = make_fan(n, S, fan->fov_rad, fan->depth_mm);
     launch_setup(pose, fd, make_place(vd), L.frame, L.geo,
                  RowOffsets{L.row_off, L.gz_off, L.ck_off, L.ray0, prm->blur ? row_stride(S) : S}, s);
     const float *gy = grad_image;

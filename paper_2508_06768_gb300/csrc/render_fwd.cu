@@ -75,7 +75,7 @@ int launch_fwd_march(const void *vol, const diffus_volume_desc *vd, const float 
                      const diffus_params *prm, RayGeo *geo, PoseFrame *frame, float *out, int32_t *ray_valid,
                      uint32_t *status, const RefineSel &sel, cudaStream_t s)
 {
-    FanDev fd{fan->n_rays, fan->n_samples, fan->fov_rad, fan->depth_mm};
+    const FanDev fd = make_fan(fan->n_rays, fan->n_samples, fan->fov_rad, fan->depth_mm);
     launch_setup(pose, fd, make_place(vd), frame, geo, RowOffsets{nullptr, nullptr, nullptr, nullptr, 0}, s);
     MarchArgs A = make_march_args(vd, fan, prm);
     const int grid = (fan->n_rays + kWarpsFwd - 1) / kWarpsFwd;
