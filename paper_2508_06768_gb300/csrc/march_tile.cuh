@@ -220,11 +220,12 @@ namespace dfs {
 
 // ------------------------------------------------ speckle field, ahead of the march
 
-// rows of one speckle work item: 32 keep the staging at 4.2 KB per warp, so
-// that 8 CTAs of 4 warps fit an SM (forward phase on the 512-pose batch
-// 1.847 ms with 64-row items, 1.777 with 32)
-constexpr int kSpkRows = 32;
-constexpr int kSpkLd = kSpkRows + 1;
+// Rows of one speckle work item: each item draws two radial groups of four
+// rows beyond its own, so long items waste less of the Philox work (18 calls
+// for 16 groups at 64 rows, 10 for 8 at 32).
+constexpr int kSpkRows = 64;
+constexpr int kSpkStage = 32;               // rows staged before they leave
+constexpr int kSpkLd = kSpkStage + 4;       // padded stage row: conflict-free 16-byte accesses both ways
 
 // A speckle work item: rows k0 .. k0+kSpkRows-1 of the rays of one forward tile.
 struct SpkItem {
@@ -232,9 +233,9 @@ struct SpkItem {
 };
 
 struct SpkSmem {
-    float m[kWarp * kSpkLd];
-    float2 zrg[kSpkRows];      // per row: Ar z^pr, Ag z^pg
-    uint32_t cell[kSpkRows];   // per row: grain cell (band << 24 | index)
+    float4 zr[kSpkRows / 4], zg[kSpkRows / 4];   // per row: Ar z^pr, Ag z^pg
+    uint4 cell[kSpkRows / 4];                    // per row: grain cell (band << 24 | index)
+    float4 m[kWarp][kSpkLd / 4];                 // factors of kSpkStage rows per ray
 };
 
 // Speckle factors (Section 2.4) of rows k0 .. k0+63 of the tile's rays,
@@ -244,22 +245,28 @@ struct SpkSmem {
 // in order: the radial window from byte sums of Philox groups of four rows
 // (exact integer sums, as the march's own speckle), one grain normal per
 // grain cell, and the same factor arithmetic, so the factors equal the
-// march's bit for bit.
+// march's bit for bit.  Bound by the Philox rounds' integer multiplies; the
+// row-only terms are read and the factors staged and stored four rows at a
+// time, a warp's store covering four 128-byte row segments.  512 frames: 481 us
+// with 32-row items, staged and stored a row at a time; 630 us with the
+// factors stored from each lane's registers to its own row (half the
+// instructions gone, but 16-byte pieces of every sector); 423 us this way.
 static __device__ void speckle_item(const Speckle &sp, const TileDesc &tl, int k0, float *__restrict__ mbuf, SpkSmem &sm)
 {
     const int lane = threadIdx.x & 31;
-    const int S = tl.S, cnt = tl.cnt;
+    const int S = tl.S;
     const uint32_t pose = sp.pose_ctr + (uint32_t)tl.pose;
     const uint32_t ray = (uint32_t)(tl.j0 + lane);
-    const int n = min(kSpkRows, S - k0);
+    const int ng = (min(kSpkRows, S - k0) + 3) / 4;      // groups of four rows
     const float invS = 1.0f / (float)S;
     const int kb1 = (S + 3) / 4, kb2 = (2 * S + 3) / 4, kb3 = (3 * S + 3) / 4;
     // what depends on the row only: depth powers and grain cell, once per item
-    for (int e = lane; e < kSpkRows; e += kWarp) {
+    for (int e = lane; e < 4 * ng; e += kWarp) {
         const int i = k0 + e;
         const float lz = __log2f((float)(i + 1) * invS);
-        sm.zrg[e] = make_float2(sp.Ar * exp2f(sp.pr * lz), sp.Ag * exp2f(sp.pg * lz));
-        sm.cell[e] = grain_cell(i, kb1, kb2, kb3, sp.gshift);
+        reinterpret_cast<float *>(sm.zr)[e] = sp.Ar * exp2f(sp.pr * lz);
+        reinterpret_cast<float *>(sm.zg)[e] = sp.Ag * exp2f(sp.pg * lz);
+        reinterpret_cast<uint32_t *>(sm.cell)[e] = grain_cell(i, kb1, kb2, kb3, sp.gshift);
     }
     int sm1[4], s0[4];
     group_sums(radial_group(sp, (k0 >> 2) - 1, (int)ray, pose), sm1);
@@ -267,15 +274,14 @@ static __device__ void speckle_item(const Speckle &sp, const TileDesc &tl, int k
     const int L = sp.Lr, off_nr = (2 * L + 1) * 510;
     uint32_t cur_grp = 0xffffffffu;
     uint4 gw = make_uint4(0, 0, 0, 0);
+    const int ld = row_stride(S);
     __syncwarp();
-    for (int g4 = 0; g4 < kSpkRows / 4; g4++) {
-        const int q = (k0 >> 2) + g4;
-        if (4 * q >= k0 + n) break;
+    for (int g4 = 0; g4 < ng; g4++) {
         int sp1[4];
-        group_sums(radial_group(sp, q + 1, (int)ray, pose), sp1);
-        int Wr[4];   // radial window sums of rows 4q .. 4q+3 (exact integers)
+        group_sums(radial_group(sp, (k0 >> 2) + g4 + 1, (int)ray, pose), sp1);
+        int Wr[4];   // radial window sums of the group's rows (exact integers)
         if (L == 4) {
-            // row 4q's window spans groups q-1 .. q+1 but the last three
+            // the first row's window spans groups q-1 .. q+1 but the last three
             // rows; each later row drops one byte sum and takes the next
             Wr[0] = ((sm1[0] + sm1[1]) + (sm1[2] + sm1[3])) + ((s0[0] + s0[1]) + (s0[2] + s0[3])) + sp1[0];
 #pragma unroll
@@ -292,34 +298,41 @@ static __device__ void speckle_item(const Speckle &sp, const TileDesc &tl, int k
                 Wr[t] = W;
             }
         }
+        const float4 zr4 = sm.zr[g4], zg4 = sm.zg[g4];
+        const uint4 c4 = sm.cell[g4];
+        const float zr[4] = {zr4.x, zr4.y, zr4.z, zr4.w}, zg[4] = {zg4.x, zg4.y, zg4.z, zg4.w};
+        const uint32_t cell[4] = {c4.x, c4.y, c4.z, c4.w};
+        float m[4];
 #pragma unroll
         for (int t = 0; t < 4; t++) {
-            const int i = 4 * q + t;
-            if (i >= k0 + n) break;
             const float nr = (float)(Wr[t] - off_nr) * sp.nr_scale;
-            const int e = i - k0;
-            const uint32_t cell = sm.cell[e];
-            if ((cell >> 2) != cur_grp) {   // the same row for every lane
-                cur_grp = cell >> 2;
+            if ((cell[t] >> 2) != cur_grp) {   // the same row for every lane
+                cur_grp = cell[t] >> 2;
                 gw = philox10_rk(make_uint4(cur_grp, ray, pose, 1u), sp.rk);
             }
-            const float ng = ih_normal(pick4(gw, cell & 3u));
-            const float2 zrg = sm.zrg[e];
-            sm.m[lane * kSpkLd + e] = fmaxf(fmaf(zrg.x, nr, fmaf(zrg.y, ng, 1.0f)), 0.0f);
+            const float ng_ = ih_normal(pick4(gw, cell[t] & 3u));
+            m[t] = fmaxf(fmaf(zr[t], nr, fmaf(zg[t], ng_, 1.0f)), 0.0f);
         }
+        constexpr int kG = kSpkStage / 4;       // groups per stage
+        sm.m[lane][g4 % kG] = make_float4(m[0], m[1], m[2], m[3]);
 #pragma unroll
         for (int u = 0; u < 4; u++) {
             sm1[u] = s0[u];
             s0[u] = sp1[u];
         }
+        if (g4 % kG == kG - 1 || g4 == ng - 1) {
+            __syncwarp();
+            // rows past S in the last group fall into the row's padding
+            const int gs = g4 - g4 % kG, part = lane & (kG - 1), r0 = lane / kG;
+            float *dst = mbuf + tl.pad0 + k0 + 4 * (gs + part);
+            if (gs + part <= g4) {
+#pragma unroll
+                for (int rr = r0; rr < kWarp; rr += kWarp / kG)
+                    if (rr < tl.cnt) __stcs(reinterpret_cast<float4 *>(dst + (int64_t)rr * ld), sm.m[rr][part]);
+            }
+            __syncwarp();
+        }
     }
-    __syncwarp();
-    // one ray's rows of the item per store instruction
-    for (int rr = 0; rr < cnt; rr++) {
-        float *dst = mbuf + tl.pad0 + (int64_t)rr * row_stride(S) + k0;
-        for (int e = lane; e < n; e += kWarp) __stcs(dst + e, sm.m[rr * kSpkLd + e]);
-    }
-    __syncwarp();
 }
 
 }  // namespace dfs
