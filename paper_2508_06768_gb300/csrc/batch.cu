@@ -20,8 +20,8 @@ namespace {
 
 constexpr uint32_t kPlanMagic = 0x44465351u;   // "DFSQ": plans with internal row offsets
 
-struct BlurTile {                 // one 32-row strip of one pose image
-    int32_t pose, n_rays, k0, pad;
+struct BlurTile {                 // a 32-row strip of rays j0 .. j0+nj-1 of one pose image
+    int32_t pose, j0, k0, nj;
 };
 
 struct PlanHeader {
@@ -93,10 +93,29 @@ PlanSizes plan_sizes(int P, int64_t total_rays, int64_t n_tiles, int64_t n_ftile
     return z;
 }
 
+// Rays per blur tile: whole fans where the strips fill the GPU (a range reads
+// 2W halo rays more), else ranges as short as the single-pose blur's, because a
+// few small frames are bound by one warp's sweep over its rays (nine frames of
+// 17-70 rays: 14.2 and 15.5 us for the blur and its
+// transpose with whole fans, 7.2 and 11.7 us with ranges of 8).
+int blur_range(const diffus_fan *fans, int P)
+{
+    int seg = 1 << 20;
+    for (;;) {
+        int64_t t = 0;
+        for (int p = 0; p < P && t < 1216; p++)
+            t += (int64_t)((fans[p].n_samples + kBlurRows - 1) / kBlurRows) * ((fans[p].n_rays + seg - 1) / seg);
+        if (t >= 1216 || seg <= kBlurStep) return seg;
+        seg = seg > kBlurSegRays ? kBlurSegRays : seg / 2;
+    }
+}
+
 int64_t count_tiles(const diffus_fan *fans, int P)
 {
+    const int seg = blur_range(fans, P);
     int64_t t = 0;
-    for (int p = 0; p < P; p++) t += (int64_t)((fans[p].n_samples + kBlurRows - 1) / kBlurRows);
+    for (int p = 0; p < P; p++)
+        t += (int64_t)((fans[p].n_samples + kBlurRows - 1) / kBlurRows) * ((fans[p].n_rays + seg - 1) / seg);
     return t;
 }
 
@@ -262,7 +281,7 @@ __global__ void __launch_bounds__(kBlurWarps * 32) k_batch_blur(const float *__r
         // the march's side of the blur is internal rows, the caller's packed
         const int64_t io = TRANSPOSE ? pp.img_off : pp.pad_off, oo = TRANSPOSE ? pp.pad_off : pp.img_off;
         blur_strip<TRANSPOSE, WT>(in + io, out + oo, pp.n_rays, pp.S, TRANSPOSE ? pp.S : pp.ld,
-                                  TRANSPOSE ? pp.ld : pp.S, b, tl.k0, 0, pp.n_rays, pp.l2_hi, pp.l2_lo);
+                                  TRANSPOSE ? pp.ld : pp.S, b, tl.k0, tl.j0, tl.j0 + tl.nj, pp.l2_hi, pp.l2_lo);
     }
 }
 
@@ -401,6 +420,7 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
     BlurTile *tiles = at_mut<BlurTile>(plan_host, H.off_tiles);
     TileDesc *ftiles = at_mut<TileDesc>(plan_host, H.off_ftiles);
 
+    const int seg = blur_range(fans, P);
     int64_t r = 0, img = 0, pad = 0, g = 0, ck = 0, t = 0, ft = 0, cb = 0;
     for (int p = 0; p < P; p++) {
         const diffus_fan &f = fans[p];
@@ -434,7 +454,8 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
             g += ldz;
             ck += nseg;
         }
-        for (int k0 = 0; k0 < f.n_samples; k0 += kBlurRows) tiles[t++] = BlurTile{p, f.n_rays, k0, 0};
+        for (int k0 = 0; k0 < f.n_samples; k0 += kBlurRows)
+            for (int j0 = 0; j0 < f.n_rays; j0 += seg) tiles[t++] = BlurTile{p, j0, k0, std::min(seg, f.n_rays - j0)};
         img += (int64_t)f.n_rays * f.n_samples;
         pad += (int64_t)f.n_rays * ld;
     }
@@ -462,12 +483,11 @@ extern "C" int diffus_batch_plan(const diffus_volume_desc *vd, const diffus_fan 
         for (int64_t tix = 0; tix < n_ftiles; tix++)
             for (int k0 = 0; k0 < ftiles[tix].S; k0 += kSpkRows) items[q++] = SpkItem{(int32_t)tix, k0};
     }
-    // blur strips of the widest poses first within each chunk (a strip's
-    // work grows with n_rays)
+    // blur tiles of the most rays first within each chunk
     std::stable_sort(tiles, tiles + n_tiles, [&](const BlurTile &x, const BlurTile &y) {
         const int cx = chunk_of[x.pose], cy = chunk_of[y.pose];
         if (cx != cy) return cx < cy;
-        return x.n_rays > y.n_rays;
+        return x.nj > y.nj;
     });
     {
         int64_t tix = 0;
