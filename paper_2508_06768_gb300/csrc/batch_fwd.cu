@@ -72,7 +72,9 @@ __global__ void __launch_bounds__(WARPS * 32, kRefineWarpsPerSM / WARPS) k_batch
                                                                 const PoseFrame *__restrict__ frames, VolPlace vp,
                                                                 float *__restrict__ out, int *__restrict__ valid,
                                                                 uint32_t *__restrict__ status,
-                                                                float4 *__restrict__ ckpt, RefineSel sel, bool padded)
+                                                                float4 *__restrict__ ckpt,
+                                                                const float *__restrict__ spk_in, RefineSel sel,
+                                                                bool padded)
 {
     __shared__ float buf[WARPS][kSegPad];
     __shared__ float2 dbuf[WARPS][kSegPad];
@@ -93,7 +95,8 @@ __global__ void __launch_bounds__(WARPS * 32, kRefineWarpsPerSM / WARPS) k_batch
         }
         const FanDev &fd = pp.fan;
         RayOut o{out + (padded ? B.pad_off[r] : B.row_off[r]), valid ? valid + r : nullptr, status,
-                 ckpt ? ckpt + B.ck_off[r] : nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, r, padded};
+                 ckpt ? ckpt + B.ck_off[r] : nullptr, nullptr, nullptr, spk_in ? spk_in + B.pad_off[r] : nullptr, nullptr,
+                 nullptr, nullptr, r, padded};
         refine_ray<T, true>(vol, Ap, rg, frames[rg.pose], fd, vp, o, sel.rinfo[r], buf[w], dbuf[w]);
         __syncwarp();
     }
@@ -125,7 +128,7 @@ void launch_fwd_t(const void *vol, const MarchArgs &A, const BatchDev &B, const 
     }
     if (sel.rinfo)
         k_batch_refine<T, WARPS><<<kRefineWarpsPerSM / WARPS * sm_count(), WARPS * 32, 0, s>>>(
-            (const T *)vol, A, B, geo, frames, vp, out, valid, status, kp.ckpt, sel, fl.padded);
+            (const T *)vol, A, B, geo, frames, vp, out, valid, status, kp.ckpt, fl.spk_in, sel, fl.padded);
 }
 
 template <typename T>

@@ -732,7 +732,9 @@ __device__ void march_refine_ray(const T *__restrict__ vol, const MarchArgs &A, 
             Ds *= dall;
         }
         float m[kChunk];
-        if (A.sp.on) {
+        if (out.min) {
+            load_chunk(out.min + i0, i0 < S, m);
+        } else if (A.sp.on) {
             chunk_speckle(A.sp, i0, S, rg.ray, pose, m);
         } else {
 #pragma unroll
