@@ -49,12 +49,13 @@ _PLAIN = (torch.Tensor, torch.nn.Parameter)
 
 def _native_call(volume, pose, fan, params, spacing, origin, pose_ctr):
     """The packed descriptors if the native node takes this call as the Python
-    function does: plain CUDA tensors outside of tracing and functorch
-    transforms (which the Python function refuses or traces), values that fit
-    the C descriptors.  None otherwise."""
+    function does: plain CUDA tensors outside of tracing, dispatch modes and
+    functorch transforms (which the Python function refuses or sees through),
+    values that fit the C descriptors.  None otherwise."""
     if (type(volume) not in _PLAIN or type(pose) not in _PLAIN or not volume.is_cuda or pose.device != volume.device
             or volume.dim() != 3 or volume.dtype not in (torch.float32, torch.bfloat16)
-            or torch._C._are_functorch_transforms_active() or torch.compiler.is_compiling()):
+            or torch._C._are_functorch_transforms_active() or torch.compiler.is_compiling() or torch.jit.is_tracing()
+            or torch._C._len_torch_dispatch_stack() != 0):
         return None
     try:
         return B.pack_call(spacing, origin, fan, params, pose_ctr)
