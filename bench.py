@@ -141,10 +141,10 @@ BOUND = {"march_fwd": "alu", "march_bwd": "alu", "gather_units": "alu", "blur": 
 # dram__bytes_write.sum of one launch over the first 192 poses of the
 # workload, the forward phase being the speckle kernel plus the march,
 # divided by its ray-samples); absent where the kernel changed since.
-NCU_DRAM_PER_UNIT = {"blur": 7.44, "blur_T": 7.44, "gather_units": 8.54}
+NCU_DRAM_PER_UNIT = {"blur": 7.98, "blur_T": 7.93, "gather_units": 8.61}
 # the marches' figures depend on the forward form (fwd_form 0: one warp per
 # ray; 1: one lane per ray), set from the capture of that form
-NCU_DRAM_PER_UNIT_FORM = {0: {"march_fwd": 18.86, "march_bwd": 19.69}, 1: {"march_fwd": 25.77, "march_bwd": 21.51}}
+NCU_DRAM_PER_UNIT_FORM = {0: {"march_fwd": 18.87, "march_bwd": 19.75}, 1: {}}
 
 
 def median_pose_order(fans):
@@ -947,16 +947,17 @@ def run_native(args):
     # kernels per step: pose frames, ray setup, [speckle field, with the
     # warp-per-ray form], forward march, [refined pass], [blur, blur
     # transpose] or [two depth-gain row passes], adjoint march, pose
-    # reduction; gather: brick runs, one radix pass per 8 bits of brick id of
-    # (histogram, 3 scan kernels, scatter), brick bounds, unit counts, 3 scan
-    # kernels, unit-brick table, unit work, class cursors, unit order, unit
-    # gather, voxel reduction, per-ray pose terms (memsets are not kernels)
+    # reduction; gather (of a batch too large for the place-and-rank sort):
+    # brick runs, brick plan (with per-block sums above 65536 bricks), one
+    # radix pass per 8 bits of brick id of (histogram, 3 scan kernels,
+    # scatter), unit work, class cursors, unit order, unit gather, voxel
+    # reduction, per-ray pose terms (memsets are not kernels)
     nbricks = int(np.prod([(n - 2) // 8 + 1 for n in vol.data.shape]))
-    passes = (nbricks.bit_length() + 7) // 8
+    passes = (max(1, (nbricks - 1).bit_length()) + 7) // 8
     form = 0 if sched is None else sched.fwd_form
     launches = (5 + (1 if form == 0 and prm.speckle else 0) + (1 if prm.refine else 0) +
                 (2 if prm.blur else (2 if prm.atten else 0)) +
-                (1 + 5 * passes + 1 + 1 + 3 + 1 + 3 + 1 + 1 + 1))
+                (1 + (2 if nbricks > 65536 else 1) + 5 * passes + 3 + 1 + 1 + 1))
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
