@@ -8,7 +8,11 @@ namespace {
 
 // Persistent forward: each warp takes rays from the queue (longest first).
 // TRACK (refinement on, sel.rinfo set): it is the FP32 pass, which lists the
-// rays that need the refined pass.
+// rays that need the refined pass.  Bound by L1 wavefronts (88 % of peak, two
+// thirds of them the eight corner loads, 4.4 lines each) with the issue slots
+// at 74 %.  512 uneven frames with everything kept for the adjoint: 1433 us
+// with packed rows, per-row tests and per-sample neighbour exchange, 1097 us
+// as it stands (225 and 181 warp instructions per 32 samples).
 template <typename T, int WARPS, int MODE, bool TRACK>
 __global__ void __launch_bounds__(WARPS * 32, kFwdThreadsPerSM / (WARPS * 32))
     k_batch_fwd(const T *__restrict__ vol, MarchArgs A, BatchDev B, const RayGeo *__restrict__ geo,
@@ -39,7 +43,7 @@ __global__ void __launch_bounds__(WARPS * 32, kFwdThreadsPerSM / (WARPS * 32))
 
 // Persistent forward with one lane per ray: each warp takes tiles of 32
 // consecutive rays of a pose from the queue (longest first).
-template <typename T>
+template <typename T, bool KEEP>
 __global__ void __launch_bounds__(kTileWarps * 32, kFwdThreadsPerSM / (kTileWarps * 32)) k_batch_fwd_tiles(const T *__restrict__ vol, MarchArgs A, BatchDev B,
                                                           const RayGeo *__restrict__ geo,
                                                           const TileDesc *__restrict__ tiles, int64_t n_tiles,
@@ -56,10 +60,10 @@ __global__ void __launch_bounds__(kTileWarps * 32, kFwdThreadsPerSM / (kTileWarp
         if (lane == 0) q = atomicAdd(counter, 1u);
         q = __shfl_sync(0xffffffffu, q, 0);
         if ((int64_t)q >= n_tiles) break;
-        const TileDesc tl = tiles[q];
+        const TileDesc *tl = tiles + q;
         MarchArgs Ap = A;
-        if (!A.atten) Ap.a2 = B.pose[tl.pose].a2;   // the depth-gain reading keeps a2 = 1
-        march_fwd_tile<T>(vol, Ap, tl, geo, out, valid, status, ckpt, mbuf, kbuf, bcar, sel, padded, sm[w]);
+        if (!A.atten) Ap.a2 = B.pose[tl->pose].a2;   // the depth-gain reading keeps a2 = 1
+        march_fwd_tile<T, KEEP>(vol, Ap, tl, geo, out, valid, status, ckpt, mbuf, kbuf, bcar, sel, padded, sm[w]);
         __syncwarp();
     }
 }
@@ -108,9 +112,10 @@ void launch_fwd_t(const void *vol, const MarchArgs &A, const BatchDev &B, const 
                   const PoseFrame *frames, const VolPlace &vp, int64_t q0, int64_t qn, cudaStream_t s)
 {
     if (fl.form == 1) {
-        k_batch_fwd_tiles<T><<<fl.grid, kTileWarps * 32, 0, s>>>((const T *)vol, A, B, geo, fl.tiles, fl.n_tiles,
-                                                                 out, valid, status, counter, kp.ckpt, kp.mbuf,
-                                                                 kp.kbuf, kp.bcar, sel, fl.padded);
+        const bool keep = kp.ckpt || kp.mbuf || kp.kbuf || kp.bcar;
+        auto kernel = keep ? k_batch_fwd_tiles<T, true> : k_batch_fwd_tiles<T, false>;
+        kernel<<<fl.grid, kTileWarps * 32, 0, s>>>((const T *)vol, A, B, geo, fl.tiles, fl.n_tiles, out, valid, status,
+                                                   counter, kp.ckpt, kp.mbuf, kp.kbuf, kp.bcar, sel, fl.padded);
     } else {
 #define DFS_BF(MODE, TRACK)                                                                                         \
     k_batch_fwd<T, WARPS, MODE, TRACK><<<fl.grid, WARPS * 32, 0, s>>>((const T *)vol, A, B, geo, out, valid, status, \

@@ -82,3 +82,26 @@ def test_frame_without_blur_and_with_nonfinite_volume():
             assert torch.equal(valid, r.ray_valid[:19])
             n = int(np.count_nonzero(~np.isfinite(a)))
             assert n > 0 and int(status[1]) == n
+
+
+@pytest.mark.parametrize("mode,bf16,refine", [(0, False, 0), (1, True, 0), (0, False, 1)])
+@pytest.mark.parametrize("fans", [[(1, 1), (33, 17)], [(64, 300), (31, 255), (70, 1030)]])
+def test_lane_form_forward_alone(fans, mode, bf16, refine):
+    # the forward-only kernel of the one-lane-per-ray form keeps nothing, and
+    # renders the bits of the call with a backward
+    import torch
+    from paper_2508_06768_gb300 import binding as B
+    from paper_2508_06768_gb300.render import BatchRenderer
+    rng = np.random.default_rng(len(fans))
+    data = (1.5 + 0.02 * rng.standard_normal((37, 41, 44))).astype(np.float32)
+    vol = torch.from_numpy(data).cuda().to(torch.bfloat16 if bf16 else torch.float32)
+    fans = [I.Fan(n, s, math.radians(64), 0.1 * s ** 0.8, 5.0, 0.5) for n, s in fans]
+    prm = I.Params(seed=11, mode=mode, refine=refine)
+    poses = torch.tensor([[21.3, 18.4, 1.2, 0.11, -0.07, 0.4]] * len(fans), device="cuda")
+    poses[:, 0] += torch.arange(len(fans), device="cuda")
+    a, b = [BatchRenderer(vol, (1.0, 0.9, 1.1), (0.0, 0.0, 0.0), fans, prm, schedule=B.ScheduleDesc(0, 0, 0, 1),
+                          with_bwd=w) for w in (False, True)]
+    a.run(poses)
+    b.run(poses, torch.ones_like(b.images))
+    assert torch.equal(a.images, b.images) and torch.equal(a.ray_valid, b.ray_valid)
+    assert torch.equal(a.status, b.status)
