@@ -19,14 +19,14 @@ constexpr int kSeg = kWarp * kChunk;         // interfaces per warp segment
 constexpr int kSegPad = kSeg + kSeg / kChunk;  // padded smem row (conflict-free chunk reads)
 // Resident-thread targets of the batched march kernels per SM (launch-bound
 // hints): the adjoint that samples dZ/dp for the pose terms at <= 128
-// registers, the adjoint that samples values only and the unrefined forward
-// at <= 85.
+// registers, the adjoint that reads the kept rows at <= 85 (512-pose batch:
+// 1097 us at 640 threads, 942 at 768, 971 at 896, 947 at 1024).
 constexpr int kBwdThreadsPerSM = 512;
 constexpr int kBwdValThreadsPerSM = 768;
-// resident threads per SM the forward marches are compiled for: 896 holds
-// the 4-warp forward at 72 registers with 7 CTAs per SM (measured on the
-// 512-pose batch: forward phase 1.780 ms at 768 threads, 1.711 at 896, 1.789
-// at 1024 and 64 registers)
+// Resident threads per SM the forward marches are compiled for: 896 holds
+// the 4-warp forward at 72 registers with 7 CTAs per SM (march on the 512-pose
+// batch and on 100 frames of 192 x 1000: 1097 and 125 us at 896 threads, 1083
+// and 130 at 1024, 1170 and 129 at 768).
 constexpr int kFwdThreadsPerSM = 896;
 // Internal rows (pre-blur echoes, speckle factors, blurred gradients) of S
 // values are kept at a stride of whole 32-byte sectors, so that a lane's

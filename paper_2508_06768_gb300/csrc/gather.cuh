@@ -7,9 +7,11 @@
 //             3D DDA on the exact fixed-point line; clamping is monotone
 //             along a ray, so each brick is one run [k0, k1] of samples.
 //  2. sort:   the runs, written at fixed slots (run i of ray r at slot
-//             i * n_rays + r), are sorted by brick with a stable radix sort,
-//             so every brick's runs appear in slot order whatever the launch
-//             schedule.
+//             i * n_rays + r), are put in order of brick, then slot: by a
+//             stable radix sort, or, for a frame or a few, by placing each
+//             in its brick's range and counting the smaller slots there.
+//             Either way every brick's runs appear in slot order whatever
+//             the launch schedule.
 //  3. units:  each brick's runs are cut into units of at most unit_runs() runs
 //             (hot bricks crossed by many poses spread over many CTAs).
 //  4. gather: one warp per unit accumulates its samples into the 9^3 voxels
