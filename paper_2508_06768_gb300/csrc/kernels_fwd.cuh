@@ -431,13 +431,16 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
             // a block whose rays all have the full window inside the fan (the
             // same for every lane): no edge guards and the interior norm;
             // the other lanes' rows of this block are read at row 0 (valid
-            // memory) and not written
+            // memory) and not written; running pointers, because input and
+            // output have their own strides (512 poses: blur 297 -> 295 us,
+            // transpose 285 -> 267 us against an offset per row)
             if (jb >= WW && jb + B + 2 * WW <= n && jb + B <= j1) {
                 const float *p = src + (size_t)(jb + WW) * si;
                 float *q = dst + (size_t)jb * so;
 #pragma unroll
                 for (int t = 0; t < B; t++) {
-                    const float x = __ldg(p + (size_t)t * si);
+                    const float x = __ldg(p);
+                    p += si;
                     win[2 * WW + t] = TRANSPOSE ? x * rfull : x;
                 }
 #pragma unroll
@@ -446,7 +449,8 @@ __device__ void blur_strip(const float *__restrict__ in, float *__restrict__ out
 #pragma unroll
                     for (int m = 1; m <= WW; m++) acc = fmaf(w[m], win[i + WW - m] + win[i + WW + m], acc);
                     if (!TRANSPOSE) acc *= rfull;
-                    if (kin) q[(size_t)i * so] = acc * gk;
+                    if (kin) *q = acc * gk;
+                    q += so;
                 }
 #pragma unroll
                 for (int t = 0; t < 2 * WW; t++) win[t] = win[t + B];
