@@ -80,14 +80,24 @@ __device__ __forceinline__ float ldv(const unsigned short *__restrict__ p, unsig
     return __uint_as_float(((unsigned)__ldg(p + i)) << 16);   // bfloat16 -> float, exact
 }
 
+// The fraction of a fixed-point coordinate, to 23 bits: 1.f with those bits is
+// (0x7F : low word) >> 9, one funnel shift.
+__host__ __device__ __forceinline__ float frac23(unsigned lo)
+{
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(__funnelshift_r(lo, 0x7Fu, 9)) - 1.0f;
+#else
+    return (float)(lo >> 9) * 0x1p-23f;
+#endif
+}
+
 // Split a fixed-point coordinate into the cell index i0 in [0, n-2] and the
 // weight f in [0, 1] after clamping the coordinate to [0, n-1] (edge
 // replicate outside the volume).  inside = coordinate strictly in (0, n-1).
 __device__ __forceinline__ void axis_split(long long X, int n, int &i0, float &f, bool &inside)
 {
     int hi = (int)(X >> 32);
-    // 1.f with the 23-bit fraction: (0x7F : low word) >> 9 is one funnel shift
-    float fr = __uint_as_float(__funnelshift_r((unsigned)X, 0x7Fu, 9)) - 1.0f;
+    float fr = frac23((unsigned)X);
     bool below = X < 0;
     bool above = hi >= n - 1;
     i0 = below ? 0 : (above ? n - 2 : hi);

@@ -594,9 +594,9 @@ __global__ void __launch_bounds__(kGatherWarps * 32, kGatherCtas)
         const uint32_t r0 = bstart[b] + part * (uint32_t)unit;
         uint32_t r1 = r0 + (uint32_t)unit;
         r1 = r1 < bend[b] ? r1 : bend[b];
-        const int bx0 = (b % G.nbx) * kBrick, by0 = ((b / G.nbx) % G.nby) * kBrick, bz0 = (b / (G.nbx * G.nby)) * kBrick;
         for (int i = lane; i < kBrickVox; i += 32) acc[i] = 0.0f;
         if (POSE) {
+            const int bx0 = (b % G.nbx) * kBrick, by0 = ((b / G.nbx) % G.nby) * kBrick, bz0 = (b / (G.nbx * G.nby)) * kBrick;
             // the 9^3 voxels the brick's cells touch (clamped at the far faces,
             // where no cell of the brick reaches)
             const unsigned sy = (unsigned)G.nx, sz = (unsigned)G.nx * (unsigned)G.ny;
@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32, kGatherCtas)
             }
         }
         __syncwarp();
-        gather_runs<POSE>(runs, steps, sorted_vals, r0, r1, gz, G, bx0, by0, bz0, sm, w, po);
+        gather_runs<POSE>(runs, steps, sorted_vals, r0, r1, gz, G, sm, w, po);
         __syncwarp();
         float *out = upart + (size_t)u * kBrickVox;
         for (int i = lane; i < kBrickVox; i += 32) out[i] = acc[i];

@@ -85,7 +85,7 @@ struct alignas(16) RayStep {
 };
 static_assert(sizeof(RayStep) == 80, "RayStep layout");
 
-__device__ __forceinline__ uint2 cell_steps(long long d)
+__host__ __device__ __forceinline__ uint2 cell_steps(long long d)
 {
     const unsigned long long e = (unsigned long long)(d < 0 ? -d : d);
     if (e <= 1) return make_uint2(0xffffffffu, 0u);      // (never within a run)
@@ -99,19 +99,29 @@ __device__ __forceinline__ uint2 cell_steps(long long d)
 // integer conversion runs on the FP64 pipe, which is narrow on this part;
 // every use here is an estimate that exact integer tests correct, or the
 // weight slope of a cell record.
-__device__ __forceinline__ float ll_to_float(long long x)
+__host__ __device__ __forceinline__ float ll_to_float(long long x)
 {
     return fmaf((float)(int)(x >> 32), 4294967296.0f, (float)(unsigned)(x & 0xffffffffll));
+}
+
+// An estimate of a / b (every use is corrected with exact integer tests).
+__host__ __device__ __forceinline__ float quotient_estimate(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fdividef(a, b);
+#else
+    return a / b;
+#endif
 }
 
 // First k in [0, kmax+1] with X0 + k DX >= L for DX > 0, or kmax+1 if no
 // k <= kmax qualifies.  Exact in fixed point: the float estimate is off by
 // at most a step or two and is corrected with integer tests.
-__device__ __forceinline__ long long first_at_or_above(long long X0, long long DX, long long L, long long kmax)
+__host__ __device__ __forceinline__ long long first_at_or_above(long long X0, long long DX, long long L, long long kmax)
 {
     if (X0 >= L) return 0;
     if (X0 + (kmax + 1) * DX < L) return kmax + 1;
-    float est = ceilf(__fdividef(ll_to_float(L - X0), ll_to_float(DX)));
+    float est = ceilf(quotient_estimate(ll_to_float(L - X0), ll_to_float(DX)));
     est = fminf(fmaxf(est, 0.0f), (float)(int)(kmax + 1));   // kmax < 2^31: 32-bit conversions
     long long k = (long long)(int)est;
     while (k > 0 && X0 + (k - 1) * DX >= L) k--;
@@ -121,7 +131,7 @@ __device__ __forceinline__ long long first_at_or_above(long long X0, long long D
 
 // k at which the brick index of one axis changes next, for a ray whose
 // brick index on that axis is b (kmax + 1 when it never does).
-__device__ __forceinline__ long long next_change(long long X0, long long DX, int b, int n, long long kmax)
+__host__ __device__ __forceinline__ long long next_change(long long X0, long long DX, int b, int n, long long kmax)
 {
     if (DX > 0) {
         int c = (b + 1) * kBrick;               // first cell of the next brick
@@ -137,7 +147,7 @@ __device__ __forceinline__ long long next_change(long long X0, long long DX, int
     return kmax + 1;
 }
 
-__device__ __forceinline__ int cell_of(long long X, int n)
+__host__ __device__ __forceinline__ int cell_of(long long X, int n)
 {
     int hi = (int)(X >> 32);
     return X < 0 ? 0 : (hi > n - 2 ? n - 2 : hi);
@@ -196,10 +206,10 @@ constexpr int kGCellCap = 32;  // samples of one cell record at most (bounds the
 // of samples before the cell or the clamping changes (at most cap).
 // Boundaries are found exactly on the fixed-point line: the float estimate
 // of ceil(num / den) is corrected with integer tests.
-__device__ __forceinline__ int ceil_div_fixed(long long num, long long den, int cap)
+__host__ __device__ __forceinline__ int ceil_div_fixed(long long num, long long den, int cap)
 {
     // smallest k >= 1 with k den >= num (num >= 1, den >= 1), at most cap
-    float est = ceilf(__fdividef(ll_to_float(num), ll_to_float(den)));
+    float est = ceilf(quotient_estimate(ll_to_float(num), ll_to_float(den)));
     long long k = est < 1.0f ? 1 : (est > (float)cap ? cap : (long long)(int)est);
     while (k > 1 && (k - 1) * den >= num) k--;
     while (k < cap && k * den < num) k++;
@@ -208,11 +218,11 @@ __device__ __forceinline__ int ceil_div_fixed(long long num, long long den, int 
 
 // Cell index i and upper-corner weight u + v k of one axis at position X
 // (exact in the clamped regions, where v = 0); vd = d / 2^32.
-__device__ __forceinline__ void axis_cell(long long X, float vd, int n, int &i, float &u, float &v)
+__host__ __device__ __forceinline__ void axis_cell(long long X, float vd, int n, int &i, float &u, float &v)
 {
     const int hi = (int)(X >> 32);
     i = hi;
-    u = __uint_as_float(__funnelshift_r((unsigned)X, 0x7Fu, 9)) - 1.0f;   // 23-bit fraction
+    u = frac23((unsigned)X);
     v = vd;
     if (hi < 0) {
         i = 0;
@@ -226,7 +236,7 @@ __device__ __forceinline__ void axis_cell(long long X, float vd, int n, int &i, 
 }
 
 // dX / 2^32 as a float.
-__device__ __forceinline__ float slope_of(long long dX)
+__host__ __device__ __forceinline__ float slope_of(long long dX)
 {
     return fmaf((float)(unsigned)(dX & 0xffffffffll), 2.3283064365386963e-10f, (float)(int)(dX >> 32));
 }
@@ -237,7 +247,7 @@ __device__ __forceinline__ float slope_of(long long dX)
 // own: there the sampler's gradient along the axis is zero (the coordinate
 // is not strictly inside the volume), so every record is either wholly
 // strictly inside or wholly not, along each axis.
-__device__ __forceinline__ int axis_steps(long long X, long long dX, int n, int cap)
+__host__ __device__ __forceinline__ int axis_steps(long long X, long long dX, int n, int cap)
 {
     const long long top = (long long)(n - 1) << 32;
     if (X < 0) return dX > 0 ? ceil_div_fixed(-X, dX, cap) : cap;
@@ -272,7 +282,7 @@ constexpr int kGStepCap = 1 << 24;   // "no crossing within the run"
 // clamped regions and for steps so small that a run's first count was cut at
 // kNextMax, from axis_steps (512 frames: 173 M warp instructions per 34 M
 // samples with that division at every crossing, 142 M).
-__device__ __forceinline__ int next_steps(long long X, long long dX, int n, uint2 qr)
+__host__ __device__ __forceinline__ int next_steps(long long X, long long dX, int n, uint2 qr)
 {
     const int hi = (int)(X >> 32);
     if ((unsigned)(hi - 1) < (unsigned)(n - 2) && qr.x < (unsigned)(kNextMax - 1)) {
@@ -286,7 +296,7 @@ __device__ __forceinline__ int next_steps(long long X, long long dX, int n, uint
 // cell in the direction of travel (a 32-bit number), the next crossing comes
 // after floor(t / e) + 1 samples; inv = 1 / e estimates the quotient (below
 // kNextMax, so off by one at most) and an exact product corrects it.
-__device__ __forceinline__ int first_steps1(long long X, long long dX, uint32_t q, float inv, int n)
+__host__ __device__ __forceinline__ int first_steps1(long long X, long long dX, uint32_t q, float inv, int n)
 {
     const int hi = (int)(X >> 32);
     if ((unsigned)(hi - 1) < (unsigned)(n - 2) && q < (unsigned)(kNextMax - 1)) {
@@ -311,7 +321,7 @@ struct FirstSteps {
     float inv[3];
 };
 
-__device__ __forceinline__ FirstSteps first_steps_of(const long long d[3])
+__host__ __device__ __forceinline__ FirstSteps first_steps_of(const long long d[3])
 {
     FirstSteps f;
 #pragma unroll
@@ -323,7 +333,7 @@ __device__ __forceinline__ FirstSteps first_steps_of(const long long d[3])
 }
 
 // The three first counts of a run, packed.
-__device__ __forceinline__ uint32_t first_steps(long long X, long long Y, long long Z, const long long d[3],
+__host__ __device__ __forceinline__ uint32_t first_steps(long long X, long long Y, long long Z, const long long d[3],
                                                 const FirstSteps &f, int nx, int ny, int nz)
 {
     return (uint32_t)first_steps1(X, d[0], f.q[0], f.inv[0], nx) |
@@ -340,8 +350,7 @@ struct PoseOut {
     size_t slots;
 };
 
-// Gather the runs [q0, q1) of one brick (first cell (bx0, by0, bz0)) into
-// this warp's 9^3 accumulator.  Each lane walks one run, one cell at a
+// Gather the runs [q0, q1) of one brick into this warp's 9^3 accumulator.  Each lane walks one run, one cell at a
 // time.  Inside a cell the upper-corner weights along each axis are linear
 // in the sample index k (u + v k), so each of the cell's 8 trilinear corner
 // sums sum_k g_k w_x(k) w_y(k) w_z(k) is a fixed combination of the four
@@ -355,8 +364,7 @@ template <bool POSE>
 __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const RayStep *__restrict__ steps,
                                             const uint32_t *__restrict__ order,
                                             uint32_t q0, uint32_t q1, const float *__restrict__ gzbuf,
-                                            const GatherArgs &G, int bx0, int by0, int bz0, GatherSmem<POSE> &sm,
-                                            int w, const PoseOut &po)
+                                            const GatherArgs &G, GatherSmem<POSE> &sm, int w, const PoseOut &po)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -468,10 +476,13 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
                     v[(zz << 2) | (yy << 1) | 1] = fmaf(vx, B, ux * A);
                 }
         }
-        const int cell = (ix - bx0) | ((iy - by0) << 3) | ((iz - bz0) << 6);
+        // the cell within its brick: the low bits, so that no cell index
+        // reaches past the brick's arrays
+        const int lx = ix & (kBrick - 1), ly = iy & (kBrick - 1), lz = iz & (kBrick - 1);
+        const int cell = lx | (ly << 3) | (lz << 6);
         if (POSE && has) {
             // the cell's 8 corner values, from the brick copy in shared memory
-            const int base = ((iz - bz0) * kBrickV + (iy - by0)) * kBrickV + (ix - bx0);
+            const int base = (lz * kBrickV + ly) * kBrickV + lx;
             float c[8];
 #pragma unroll
             for (int q = 0; q < 8; q++) c[q] = vox[base + ((q >> 2) * kBrickV + ((q >> 1) & 1)) * kBrickV + (q & 1)];

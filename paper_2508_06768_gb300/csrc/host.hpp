@@ -125,9 +125,12 @@ inline VolGeo make_volgeo(const diffus_volume_desc *vd)
     return {vd->nx, vd->ny, vd->nz, (float)(1.0 / vd->sx), (float)(1.0 / vd->sy), (float)(1.0 / vd->sz)};
 }
 
+// The reciprocals stay finite for subnormal spacings too: a step of 0 x inf or
+// inf voxels has no fixed-point form.
 inline VolPlace make_place(const diffus_volume_desc *vd)
 {
-    return {1.0 / vd->sx, 1.0 / vd->sy, 1.0 / vd->sz, vd->ox, vd->oy, vd->oz};
+    auto inv = [](double s) { return fmin(1.0 / s, 1.7976931348623157e308); };
+    return {inv(vd->sx), inv(vd->sy), inv(vd->sz), vd->ox, vd->oy, vd->oz};
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }

@@ -56,12 +56,29 @@ __device__ __forceinline__ void rotation_zyx(const double sn[3], const double cs
     dR[2][2][0] = 0;        dR[2][2][1] = 0;        dR[2][2][2] = 0;
 }
 
-__device__ __forceinline__ long long to_fixed(double x)
+// Fixed-point (2^-32 voxel) position and step.  No sample X0 + k DX, k = 0..S,
+// may leave 64 bits, because everything after the setup counts on a line that
+// is monotone along each axis: positions are clamped to 2^30 voxels, a fan is
+// at most 2^29 voxels long, and the step of a pose that is not finite (NaN
+// reaches here from the device, for example from a diverged optimiser) is 0,
+// where the conversion would give the lowest integer, whose multiples wrap.
+// Such a pose still shows in rg.v, and so in its gradient.
+__host__ __device__ __forceinline__ long long round_fixed(double x)
+{
+#ifdef __CUDA_ARCH__
+    return __double2ll_rn(__dmul_rn(x, 4294967296.0));
+#else
+    return llrint(x * 4294967296.0);
+#endif
+}
+
+__host__ __device__ __forceinline__ long long to_fixed(double x)
 {
     const double lim = 1073741824.0;   // 2^30 voxels: far outside any volume
-    x = fmin(fmax(x, -lim), lim);
-    return __double2ll_rn(x * 4294967296.0);
+    return round_fixed(fmin(fmax(x, -lim), lim));   // NaN: -lim
 }
+
+__host__ __device__ __forceinline__ long long step_fixed(double dx) { return dx == dx ? round_fixed(dx) : 0; }
 
 // What the rays of one pose need from it (Section 2.4): columns 0 and 2 of
 // R and of each dR/dr_q (a fan direction d = (sin th, 0, cos th) has no
@@ -124,8 +141,6 @@ __device__ __forceinline__ void ray_line(const PoseFrame &f, int ray, const FanD
     const double isp[3] = {vp.isx, vp.isy, vp.isz}, org[3] = {vp.ox, vp.oy, vp.oz};
     for (int i = 0; i < 3; i++) axis_line(f.Rc[i], f.t[i], fan.ds, isp[i], org[i], st, ct, x0[i], dx[i]);
 }
-
-__device__ __forceinline__ long long step_fixed(double dx) { return __double2ll_rn(__dmul_rn(dx, 4294967296.0)); }
 
 __device__ __forceinline__ float dir_derivative(const double dRc[2], double st, double ct)
 {
