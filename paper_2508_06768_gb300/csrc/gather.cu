@@ -123,24 +123,7 @@ __global__ void __launch_bounds__(128, 6) k_ray_runs(const RayGeo *__restrict__ 
 // number in its brick (any order; ranked by slot afterwards), else brick_work
 // receives the samples of each brick for the unit order.
 constexpr int kRunWarps = 8;
-constexpr int kRunMax = 255;
 constexpr int kRunWarpRays = 50000;
-
-__device__ __forceinline__ int count_below(const int *k, int n, int v, bool or_equal)
-{
-    int lo = 0;
-    while (n > 0) {
-        const int h = n >> 1;
-        const int m = k[lo + h];
-        if (m < v || (or_equal && m == v)) {
-            lo += h + 1;
-            n -= h + 1;
-        } else {
-            n = h;
-        }
-    }
-    return lo;
-}
 
 template <bool ARRIVE>
 __global__ void __launch_bounds__(kRunWarps * 32)
@@ -156,43 +139,16 @@ __global__ void __launch_bounds__(kRunWarps * 32)
     const RayGeo rg = geo[r];
     const int S = rg.S;
     const int n[3] = {G.nx, G.ny, G.nz};
-    int b0[3], off[4];
-    off[0] = 0;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        b0[a] = cell_of(rg.X0[a], n[a]) / kBrick;
-        const int b1 = cell_of(rg.X0[a] + (long long)S * rg.DX[a], n[a]) / kBrick;
-        off[a + 1] = off[a] + abs(b1 - b0[a]);
-    }
-    const int m = min(off[3], kRunMax);        // off[3] <= cap - 1 <= kRunMax
+    const Cuts c = ray_cuts(rg.X0, rg.DX, S, n);
+    const int m = c.off[3];                     // <= kRunMax
     int *k = sk[w], *start = sm[w];
-    for (int e = lane; e < m; e += 32) {
-        const int a = e < off[1] ? 0 : (e < off[2] ? 1 : 2);
-        const int j = e - (a == 0 ? 0 : (a == 1 ? off[1] : off[2]));
-        const long long X0 = a == 0 ? rg.X0[0] : (a == 1 ? rg.X0[1] : rg.X0[2]);
-        const long long DX = a == 0 ? rg.DX[0] : (a == 1 ? rg.DX[1] : rg.DX[2]);
-        const int b = a == 0 ? b0[0] : (a == 1 ? b0[1] : b0[2]);
-        long long kk;
-        if (DX > 0)
-            kk = first_at_or_above(X0, DX, (long long)((b + j + 1) * kBrick) << 32, S);
-        else   // cell < 8c  <=>  -X >= -(8c << 32) + 1
-            kk = first_at_or_above(-X0, -DX, -((long long)((b - j) * kBrick) << 32) + 1, S);
-        k[e] = (int)kk;
-    }
+    for (int e = lane; e < m; e += 32) k[e] = cut_sample(c, e, rg.X0, rg.DX, S);
     __syncwarp();
     int *order = start;                         // merged, with repeats
-    for (int e = lane; e < m; e += 32) {
-        const int a = e < off[1] ? 0 : (e < off[2] ? 1 : 2);
-        const int v = k[e];
-        int pos = e - (a == 0 ? 0 : (a == 1 ? off[1] : off[2]));
-        if (a != 0) pos += count_below(k, off[1], v, true);
-        if (a != 1) pos += count_below(k + off[1], off[2] - off[1], v, a == 2);
-        if (a != 2) pos += count_below(k + off[2], m - off[2], v, false);
-        order[pos] = v;
-    }
+    for (int e = lane; e < m; e += 32) order[cut_rank(c, k, m, e)] = k[e];
     __syncwarp();
     // distinct crossings: the first sample of every run after the first
-    int cnt = 1;
+    int cnt = c.fits ? 1 : 0;
     for (int e0 = 0; e0 < m; e0 += 32) {
         const int e = e0 + lane;
         const int v = e < m ? order[e] : 0;
@@ -202,13 +158,13 @@ __global__ void __launch_bounds__(kRunWarps * 32)
         cnt += __popc(bal);
     }
     __syncwarp();
-    if (cnt > cap) {
-        if (status && lane == 0) atomicOr(status + 2, (uint32_t)DIFFUS_STATUS_QUEUE);
-        cnt = cap;
-    }
+    // as in k_ray_runs, samples beyond the last slot are dropped and reported
+    const int kept = min(cnt, cap);
+    if ((kept < cnt || !c.fits) && status && lane == 0) atomicOr(status + 2, (uint32_t)DIFFUS_STATUS_QUEUE);
     const FirstSteps fs = first_steps_of(rg.DX);
-    for (int i = lane; i < cnt; i += 32) {
-        const int ka = i ? k[i - 1] : 0, kb = i + 1 < cnt ? k[i] : S + 1;
+    for (int i = lane; i < kept; i += 32) {
+        int ka, kb;
+        run_span(k, i, cnt, S, ka, kb);
         Run run;
         run.X = rg.X0[0] + (long long)ka * rg.DX[0];
         run.Y = rg.X0[1] + (long long)ka * rg.DX[1];
@@ -230,7 +186,7 @@ __global__ void __launch_bounds__(kRunWarps * 32)
         }
     }
     if (lane == 0) {
-        nrun[r] = cnt;
+        nrun[r] = kept;
         store_steps(steps + r, rg.DX, gz_off[r]);
     }
 }

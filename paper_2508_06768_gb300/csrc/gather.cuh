@@ -153,6 +153,87 @@ __host__ __device__ __forceinline__ int cell_of(long long X, int n)
     return X < 0 ? 0 : (hi > n - 2 ? n - 2 : hi);
 }
 
+// A ray's brick crossings, for the run pass that solves them independently: the
+// brick index of an axis is monotone along the ray, so axis a is crossed
+// off[a+1] - off[a] times, as entries off[a] .. off[a+1]-1 of the ray's list.
+// A ray crosses at most cap - 1 <= kRunMax times (runs_per_ray); one that did
+// not keep to that has no entries (fits = false), because a list cut short
+// would put the missing bricks' samples into other bricks' runs.
+constexpr int kRunMax = 255;
+
+struct Cuts {
+    int b0[3], off[4];
+    bool fits;
+};
+
+__host__ __device__ __forceinline__ Cuts ray_cuts(const long long X0[3], const long long DX[3], int S, const int n[3])
+{
+    Cuts c;
+    c.off[0] = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        c.b0[a] = cell_of(X0[a], n[a]) / kBrick;
+        const int b1 = cell_of(X0[a] + (long long)S * DX[a], n[a]) / kBrick;
+        c.off[a + 1] = c.off[a] + abs(b1 - c.b0[a]);
+    }
+    c.fits = c.off[3] <= kRunMax;
+    if (!c.fits) c.off[1] = c.off[2] = c.off[3] = 0;
+    return c;
+}
+
+__host__ __device__ __forceinline__ int cut_axis(const Cuts &c, int e) { return e < c.off[1] ? 0 : (e < c.off[2] ? 1 : 2); }
+
+// The sample that crosses at entry e.
+__host__ __device__ __forceinline__ int cut_sample(const Cuts &c, int e, const long long X0[3], const long long DX[3],
+                                                   int S)
+{
+    const int a = cut_axis(c, e);
+    const int j = e - (a == 0 ? 0 : (a == 1 ? c.off[1] : c.off[2]));
+    const long long x = a == 0 ? X0[0] : (a == 1 ? X0[1] : X0[2]);
+    const long long d = a == 0 ? DX[0] : (a == 1 ? DX[1] : DX[2]);
+    const int b = a == 0 ? c.b0[0] : (a == 1 ? c.b0[1] : c.b0[2]);
+    if (d > 0) return (int)first_at_or_above(x, d, (long long)((b + j + 1) * kBrick) << 32, S);
+    // cell < 8c  <=>  -X >= -(8c << 32) + 1
+    return (int)first_at_or_above(-x, -d, -((long long)((b - j) * kBrick) << 32) + 1, S);
+}
+
+__host__ __device__ __forceinline__ int count_below(const int *k, int n, int v, bool or_equal)
+{
+    int lo = 0;
+    while (n > 0) {
+        const int h = n >> 1;
+        const int m = k[lo + h];
+        if (m < v || (or_equal && m == v)) {
+            lo += h + 1;
+            n -= h + 1;
+        } else {
+            n = h;
+        }
+    }
+    return lo;
+}
+
+// Entry e's place in the merged order of all m entries (equal samples: lower
+// axis first).
+__host__ __device__ __forceinline__ int cut_rank(const Cuts &c, const int *k, int m, int e)
+{
+    const int a = cut_axis(c, e), v = k[e];
+    int pos = e - (a == 0 ? 0 : (a == 1 ? c.off[1] : c.off[2]));
+    if (a != 0) pos += count_below(k, c.off[1], v, true);
+    if (a != 1) pos += count_below(k + c.off[1], c.off[2] - c.off[1], v, a == 2);
+    if (a != 2) pos += count_below(k + c.off[2], m - c.off[2], v, false);
+    return pos;
+}
+
+// Samples [k0, k1) of run i of the ray's cnt runs (start: the first sample of
+// runs 1 .. cnt-1).  A run ends where the next one starts, whether or not that
+// one has a slot.
+__host__ __device__ __forceinline__ void run_span(const int *start, int i, int cnt, int S, int &k0, int &k1)
+{
+    k0 = i ? start[i - 1] : 0;
+    k1 = i + 1 < cnt ? start[i] : S + 1;
+}
+
 template <bool POSE>
 struct GatherSmem {
     float acc[kGatherWarps][kBrickVox];

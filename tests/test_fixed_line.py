@@ -115,3 +115,86 @@ def host_program(tmp_path_factory):
 def test_cells_and_bricks_of_a_line(host_program):
     r = subprocess.run([host_program(SOURCE)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+RUNS = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <cmath>
+#include <vector>
+#include "host.hpp"
+#include "gather.cuh"
+using namespace dfs;
+
+static int fails = 0;
+#define CHECK(c, ...) do { if (!(c)) { if (fails++ < 5) { printf(__VA_ARGS__); printf("\n"); } } } while (0)
+
+static int brick_at(const long long X0[3], const long long DX[3], const int n[3], int k)
+{
+    int b = 0;
+    for (int a = 2; a >= 0; a--) b = b * 8192 + cell_of(X0[a] + k * DX[a], n[a]) / kBrick;
+    return b;
+}
+
+// The runs of one ray as the warp-per-ray pass forms them, with room for cap.
+static void runs_of(const long long X0[3], const long long DX[3], const int n[3], int S, int cap)
+{
+    std::vector<int> want{0};             // first sample of every run
+    for (int k = 1; k <= S; k++)
+        if (brick_at(X0, DX, n, k) != brick_at(X0, DX, n, k - 1)) want.push_back(k);
+    const Cuts c = ray_cuts(X0, DX, S, n);
+    const int m = c.off[3];
+    CHECK(c.off[1] >= 0 && c.off[2] >= c.off[1] && m >= c.off[2] && m <= kRunMax, "entries %d %d %d", c.off[1], c.off[2], m);
+    if (m > kRunMax || c.off[2] > kRunMax || c.off[1] > kRunMax) return;   // what follows would leave the lists
+    if (!c.fits) {                        // no entry, no run: the pass reports the ray
+        CHECK(m == 0 && (int)want.size() > 1, "%d entries of a ray that does not fit", m);
+        return;
+    }
+    std::vector<int> k(m), start(m, -1);
+    for (int e = 0; e < m; e++) k[e] = cut_sample(c, e, X0, DX, S);
+    for (int e = 0; e < m; e++) {
+        const int p = cut_rank(c, k.data(), m, e);
+        CHECK(p >= 0 && p < m && start[p] == -1, "entry %d at place %d of %d", e, p, m);
+        if (p >= 0 && p < m) start[p] = k[e];
+    }
+    int cnt = 1;
+    for (int e = 0; e < m; e++)
+        if (e == 0 || start[e] != start[e - 1]) k[cnt++ - 1] = start[e];
+    CHECK(cnt == (int)want.size(), "%d runs, %d expected", cnt, (int)want.size());
+    const int kept = std::min(cnt, cap);
+    for (int i = 0; i < kept && !fails; i++) {
+        int a, b;
+        run_span(k.data(), i, cnt, S, a, b);
+        CHECK(a == want[i] && b == (i + 1 < cnt ? want[i + 1] : S + 1), "run %d of %d (room for %d): %d..%d", i, cnt, cap,
+              a, b);
+    }
+}
+
+int main()
+{
+    srand(2);
+    auto uni = [] { return rand() / (double)RAND_MAX; };
+    const int shapes[][3] = {{44, 41, 37}, {2, 2, 2}, {9, 17, 64}, {700, 700, 600}, {2000, 2000, 16}, {16, 2000, 2000},
+                             {65535, 16, 16}, {16, 16, 65535}};
+    for (auto &n : shapes)
+        for (int q = 0; q < 200; q++) {
+            const int S = q % 5 == 0 ? 1 + (int)(uni() * 8) : 1 + (int)(uni() * 3000);
+            long long X0[3], DX[3];
+            for (int a = 0; a < 3; a++) {
+                const double p = (uni() * 1.2 - 0.1) * n[a], e = (uni() * 1.2 - 0.1) * n[a];
+                X0[a] = to_fixed(q % 3 ? p : std::floor(p));
+                DX[a] = step_fixed(q % 7 == 0 && a ? 1.0 * (a == 1 ? 1 : -1) : (e - p) / S);
+            }
+            for (int cap : {256, 256, 40, 7, 2, 1}) runs_of(X0, DX, n, S, cap);
+        }
+    printf("%d faults\n", fails);
+    return fails ? 1 : 0;
+}
+"""
+
+
+def test_runs_of_a_ray_with_more_crossings_than_room(host_program):
+    # a ray of more runs than slots, or of more crossings than the pass has
+    # entries, loses the samples beyond; none lands in another brick's run
+    r = subprocess.run([host_program(RUNS)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
