@@ -244,13 +244,14 @@ struct GatherSmem {
 
 // Adds one closed cell record per flagged lane into the warp's accumulator.
 // Records on the same cell are grouped with a warp match and added into the
-// group's lowest lane in lane order; the group leaders, all on distinct
+// group's lowest lane in lane order (base: the cell's first voxel in the
+// accumulator); the group leaders, all on distinct
 // cells, then write one corner at a time: for a fixed corner offset
 // distinct cells hit distinct voxels.
-__device__ __forceinline__ void flush_records(bool fl, int fcell, float (&fv)[8], float *acc, int lane,
+__device__ __forceinline__ void flush_records(bool fl, int base, float (&fv)[8], float *acc, int lane,
                                               unsigned lt)
 {
-    const int key = fl ? fcell : 1024 + lane;
+    const int key = fl ? base : 1024 + lane;
     const unsigned grp = __match_any_sync(0xffffffffu, key);
     const bool leader = (grp & lt) == 0;
     unsigned rest = (fl && leader) ? (grp & (grp - 1u)) : 0u;   // other members, lane order
@@ -267,8 +268,6 @@ __device__ __forceinline__ void flush_records(bool fl, int fcell, float (&fv)[8]
         }
     }
     const bool writes = fl && leader;
-    const int cx = fcell & 7, cy = (fcell >> 3) & 7, cz = (fcell >> 6) & 7;
-    const int base = (cz * kBrickV + cy) * kBrickV + cx;
 #pragma unroll
     for (int q = 0; q < 8; q++) {
         if (writes) {
@@ -557,13 +556,11 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
                     v[(zz << 2) | (yy << 1) | 1] = fmaf(vx, B, ux * A);
                 }
         }
-        // the cell within its brick: the low bits, so that no cell index
-        // reaches past the brick's arrays
-        const int lx = ix & (kBrick - 1), ly = iy & (kBrick - 1), lz = iz & (kBrick - 1);
-        const int cell = lx | (ly << 3) | (lz << 6);
+        // the cell's first voxel in the brick's arrays, from the low bits of
+        // the cell, so that no cell index reaches past them
+        const int base = ((iz & (kBrick - 1)) * kBrickV + (iy & (kBrick - 1))) * kBrickV + (ix & (kBrick - 1));
         if (POSE && has) {
             // the cell's 8 corner values, from the brick copy in shared memory
-            const int base = (lz * kBrickV + ly) * kBrickV + lx;
             float c[8];
 #pragma unroll
             for (int q = 0; q < 8; q++) c[q] = vox[base + ((q >> 2) * kBrickV + ((q >> 1) & 1)) * kBrickV + (q & 1)];
@@ -608,7 +605,7 @@ __device__ __forceinline__ void gather_runs(const Run *__restrict__ runs, const 
                 for (int q = 0; q < 6; q++) po.rpart[(size_t)q * po.slots + slot] = ps[q];
             }
         }
-        flush_records(has, cell, v, acc, lane, lt);
+        flush_records(has, base, v, acc, lane, lt);
     }
 }
 
