@@ -170,9 +170,10 @@ _CALL = struct.Struct("@6d ii4d Qii4diiiiddIi")
 
 def pack_call(spacing, origin, f, p, pose_ctr: int = 0):
     """The descriptors of one single-pose call as bytes, with the conversions
-    of fan_desc and params_desc; struct.error if a value does not fit as it is."""
-    return _CALL.pack(*spacing, *origin, f.n_rays, f.n_samples, f.fov, f.depth, f.f_mhz, f.alpha,
-                      int(p.seed) & (2**64 - 1), int(p.mode), int(p.speckle), p.Ar, p.pr, p.Ag, p.pg, int(p.Lr),
+    of volume_desc, fan_desc and params_desc; struct.error if a value does not
+    fit as it is."""
+    return _CALL.pack(spacing[0], spacing[1], spacing[2], origin[0], origin[1], origin[2],
+                      f.n_rays, f.n_samples, f.fov, f.depth, f.f_mhz, f.alpha, int(p.seed) & (2**64 - 1), int(p.mode), int(p.speckle), p.Ar, p.pr, p.Ag, p.pg, int(p.Lr),
                       int(p.gshift), int(p.blur), int(getattr(p, "refine", 0)), p.sigma0, p.sigma1,
                       int(pose_ctr) & 0xFFFFFFFF, int(getattr(p, "atten", 0)))
 
