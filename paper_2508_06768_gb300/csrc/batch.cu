@@ -528,6 +528,8 @@ extern "C" int diffus_render_batch(const void *vol, const diffus_volume_desc *vd
     const PlanHeader &H = *(const PlanHeader *)plan_host;
     if (H.magic != kPlanMagic || H.params_fp != params_fingerprint(prm) || H.blurW != blur_halfwidth(prm))
         return DIFFUS_E_PLAN;
+    // the plan checked its fans against its own spacing, which need not be this one
+    if (!path_fits(H.max_depth, vd)) return DIFFUS_E_PARAM;
     size_t el = vd->dtype == DIFFUS_F32 ? 4 : 2;
     if (((uintptr_t)vol) % el || ((uintptr_t)poses) % 4 || ((uintptr_t)images) % 4 ||
         ((uintptr_t)workspace) % 256 || ((uintptr_t)plan_dev) % 256)

@@ -30,6 +30,12 @@ inline int check_vol(const diffus_volume_desc *vd)
     return DIFFUS_OK;
 }
 
+// Fixed-point positions: a ray must stay within 2^29 voxels.
+inline bool path_fits(double depth_mm, const diffus_volume_desc *vd)
+{
+    return depth_mm / fmin(vd->sx, fmin(vd->sy, vd->sz)) <= 536870912.0;
+}
+
 inline int check_fan(const diffus_fan *f, const diffus_volume_desc *vd)
 {
     if (!f) return DIFFUS_E_NULL;
@@ -39,9 +45,7 @@ inline int check_fan(const diffus_fan *f, const diffus_volume_desc *vd)
     if (!(f->depth_mm > 0.0) || !finite_d(f->depth_mm)) return DIFFUS_E_PARAM;
     if (!(f->f_mhz >= 0.0) || !finite_d(f->f_mhz)) return DIFFUS_E_PARAM;
     if (!(f->alpha_db_cm_mhz >= 0.0) || !finite_d(f->alpha_db_cm_mhz)) return DIFFUS_E_PARAM;
-    // fixed-point positions: the ray must stay within 2^29 voxels
-    double smin = fmin(vd->sx, fmin(vd->sy, vd->sz));
-    if (f->depth_mm / smin > 536870912.0) return DIFFUS_E_PARAM;
+    if (!path_fits(f->depth_mm, vd)) return DIFFUS_E_PARAM;
     return DIFFUS_OK;
 }
 
