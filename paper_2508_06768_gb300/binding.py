@@ -14,6 +14,7 @@ import importlib.util
 import os
 import struct
 import threading
+import warnings
 
 import numpy as np
 import torch
@@ -113,23 +114,28 @@ def load(build_if_missing: bool = True):
 
 def load_node():
     """Load the native autograd node of render() (a torch extension module
-    linked against libdiffus.so)."""
+    linked against libdiffus.so), building it when it is missing or was built
+    for another torch.  None, with one warning, where that is not possible:
+    render() then takes the Python function of the same calls."""
     global _node
     if _node is not None:
-        return _node
+        return _node or None
     load()
     with _lock:
         if _node is None:
-            if not os.path.exists(_build.NODE):
-                _build.build()
-            spec = importlib.util.spec_from_file_location(
-                _build.NODE_NAME, _build.NODE, loader=importlib.machinery.ExtensionFileLoader(_build.NODE_NAME,
-                                                                                             _build.NODE))
-            mod = importlib.util.module_from_spec(spec)
-            spec.loader.exec_module(mod)
-            mod.set_error(DiffusError)
-            _node = mod
-    return _node
+            try:
+                _build.build_node()
+                spec = importlib.util.spec_from_file_location(
+                    _build.NODE_NAME, _build.NODE,
+                    loader=importlib.machinery.ExtensionFileLoader(_build.NODE_NAME, _build.NODE))
+                mod = importlib.util.module_from_spec(spec)
+                spec.loader.exec_module(mod)
+                mod.set_error(DiffusError)
+                _node = mod
+            except (ImportError, OSError, RuntimeError) as e:
+                warnings.warn("render() runs without its native autograd node: %s" % e, RuntimeWarning, stacklevel=3)
+                _node = False
+    return _node or None
 
 
 def _check(rc: int, what: str):
@@ -173,7 +179,8 @@ def pack_call(spacing, origin, f, p, pose_ctr: int = 0):
     of volume_desc, fan_desc and params_desc; struct.error if a value does not
     fit as it is."""
     return _CALL.pack(spacing[0], spacing[1], spacing[2], origin[0], origin[1], origin[2],
-                      f.n_rays, f.n_samples, f.fov, f.depth, f.f_mhz, f.alpha, int(p.seed) & (2**64 - 1), int(p.mode), int(p.speckle), p.Ar, p.pr, p.Ag, p.pg, int(p.Lr),
+                      f.n_rays, f.n_samples, f.fov, f.depth, f.f_mhz, f.alpha,
+                      int(p.seed) & (2**64 - 1), int(p.mode), int(p.speckle), p.Ar, p.pr, p.Ag, p.pg, int(p.Lr),
                       int(p.gshift), int(p.blur), int(getattr(p, "refine", 0)), p.sigma0, p.sigma1,
                       int(pose_ctr) & 0xFFFFFFFF, int(getattr(p, "atten", 0)))
 
