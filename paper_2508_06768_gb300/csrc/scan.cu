@@ -115,58 +115,70 @@ ScanHeader scan_layout(const ScanGeom &g, int64_t n_ent)
 // own x axis, so a warp takes a compact 2D patch rather than 32 neighbours of
 // one line: the patch's taps then share lines on the other side.  What bounds
 // them is the number of lines per load (L1 wavefronts), then the streams to
-// HBM.  Measured on 64 images of 256 x 1024 and a 1024 x 1024 display: forward
-// 143 us with 32 x 1 pixels per warp, 120 us with 8 x 4 (2.8 TB/s); adjoint
-// 531 us with 1 ray x 32 rows and 4 images per pass over the lists, 335 us with
-// 4 x 8 and 8 images, 215 us with the image groups side by side instead of in
-// turn, 198 us with 8 rays x 4 rows (fewer display lines per load; L1
-// wavefronts near their peak).
-constexpr int kScanTileX = 32, kScanTileY = 8;   // a block's pixels (8 x 4 per warp), or rows x rays (4 x 8)
+// HBM; a few images of a small display are bound by one thread's chain.
+// 64 images of 256 x 1024 and a 1024 x 1024 display: forward 143 us with
+// 32 x 1 pixels per warp, 105 us (3.2 TB/s) with 8 x 4; adjoint 531 us with 1 ray
+// x 32 rows and 4 images per pass over the lists, 335 us with 4 x 8 and 8 images,
+// 215 us with the image groups side by side instead of in turn, 198 us with 8
+// rays x 4 rows.
+constexpr int kScanTile = 256;                   // threads per block: 8 warps of 8 x 4 pixels, or of 4 rows x 8 rays
 constexpr int kScanImgs = 8;                     // images per pass over the lists (adjoint)
-constexpr int kScanUnroll = 4;                   // images with their taps in flight together (forward)
 
-// One thread per display pixel: the tap is read once and applied to all
-// `count` images.
-__global__ void __launch_bounds__(kScanTileX *kScanTileY)
+// One thread per display pixel: the tap is read once and applied to the
+// images of the block's group (blockIdx.z, GROUPED; else all), U images' taps in
+// flight together.  A block is 2^cols warps wide and 8 / 2^cols high; tile0: the
+// grid's first tile along its y axis.  U and the resident blocks MINB trade loads
+// in flight against warps: one image of 256 x 1024 to 1024 x 1024 takes 5.1 us
+// with 4 and 5, 4.65 with 2 and 8; 64 images 105 us with 4 and 5.
+template <int U, int MINB, bool GROUPED>
+__global__ void __launch_bounds__(kScanTile, MINB)
     k_scan_fwd(const float *__restrict__ img, const ScanTap *__restrict__ map, int S, int64_t img_stride, int W, int H,
-               int tiles_x, int count, float *__restrict__ out)
+               int64_t npix, int cols, int tile0, int count, int group, float *__restrict__ out)
 {
+    constexpr bool kDown = U == 2;               // grid x runs down the display
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int ix = (blockIdx.x % tiles_x) * kScanTileX + (w & 3) * 8 + (lane & 7);
-    const int iz = (blockIdx.x / tiles_x) * kScanTileY + (w >> 2) * 4 + (lane >> 3);
+    const int wx = w & ((1 << cols) - 1), wy = w >> cols;
+    const int gx = blockIdx.x, gy = blockIdx.y + tile0;
+    const int ix = (((kDown ? gy : gx) << cols) + wx) * 8 + (lane & 7);
+    const int iz = ((kDown ? gx : gy) * (8 >> cols) + wy) * 4 + (lane >> 3);
     if (ix >= W || iz >= H) return;
-    const int64_t npix = (int64_t)W * H, p = (int64_t)iz * W + ix;
+    const int64_t p = (int64_t)iz * W + ix;
     const ScanTap t = map[p];
-    float *o = out + p;
+    if (GROUPED) {
+        const int c0 = blockIdx.z * group;
+        img += (int64_t)c0 * img_stride;
+        out += (int64_t)c0 * npix;
+        count = min(count - c0, group);
+    }
+    out += p;
     if (t.j0 < 0) {
-        for (int c = 0; c < count; c++, o += npix) *o = 0.0f;
+#pragma unroll 1
+        for (; count > 0; count--, out += npix) *out = 0.0f;
         return;
     }
     const float a = (1.0f - t.fv) * (1.0f - t.fu), b = t.fv * (1.0f - t.fu);
     const float cc = (1.0f - t.fv) * t.fu, d = t.fv * t.fu;
-    const float *r0 = img + (int64_t)t.j0 * S + t.k0, *r1 = r0 + S;
-    int c = 0;
-    for (; c + kScanUnroll <= count; c += kScanUnroll) {
-        float v[kScanUnroll][4];
+    img += (int64_t)t.j0 * S + t.k0;
+    for (; count >= U; count -= U) {
+        float v[U][4];
 #pragma unroll
-        for (int u = 0; u < kScanUnroll; u++) {
-            v[u][0] = __ldg(r0);
-            v[u][1] = __ldg(r1);
-            v[u][2] = __ldg(r0 + 1);
-            v[u][3] = __ldg(r1 + 1);
-            r0 += img_stride;
-            r1 += img_stride;
+        for (int u = 0; u < U; u++, img += img_stride) {
+            v[u][0] = __ldg(img);
+            v[u][1] = __ldg(img + S);
+            v[u][2] = __ldg(img + 1);
+            v[u][3] = __ldg(img + S + 1);
         }
 #pragma unroll
-        for (int u = 0; u < kScanUnroll; u++, o += npix)
-            *o = fmaf(d, v[u][3], fmaf(cc, v[u][2], fmaf(b, v[u][1], a * v[u][0])));
+        for (int u = 0; u < U; u++, out += npix)
+            *out = fmaf(d, v[u][3], fmaf(cc, v[u][2], fmaf(b, v[u][1], a * v[u][0])));
     }
-    for (; c < count; c++, r0 += img_stride, r1 += img_stride, o += npix)
-        *o = fmaf(d, __ldg(r1 + 1), fmaf(cc, __ldg(r0 + 1), fmaf(b, __ldg(r1), a * __ldg(r0))));
+#pragma unroll 1
+    for (; count > 0; count--, img += img_stride, out += npix)
+        *out = fmaf(d, __ldg(img + S + 1), fmaf(cc, __ldg(img + 1), fmaf(b, __ldg(img + S), a * __ldg(img))));
 }
 
-// One thread per polar pixel: its list is read once for kScanImgs gradients
-// at a time, each summed in the list's fixed order.
+// One thread per polar pixel: its list is read once for N gradients at a time,
+// each summed in the list's fixed order.
 template <int N>
 __device__ __forceinline__ void scan_bwd_pass(const float *__restrict__ g, const ScanEnt *__restrict__ ent, uint32_t e0,
                                               uint32_t e1, int64_t npix, int64_t nq, float *__restrict__ out)
@@ -195,17 +207,17 @@ __device__ __forceinline__ void scan_bwd_pass(const float *__restrict__ g, const
     for (int u = 0; u < N; u++) out[(int64_t)u * nq] = s[u];
 }
 
-__global__ void __launch_bounds__(kScanTileX *kScanTileY)
+__global__ void __launch_bounds__(kScanTile)
     k_scan_bwd(const float *__restrict__ gout, const uint32_t *__restrict__ rowptr, const ScanEnt *__restrict__ ent, int n,
                int S, int tiles_x, int64_t npix, int count, float *__restrict__ gimg)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int k = (blockIdx.x % tiles_x) * kScanTileX + w * 4 + (lane & 3);
-    const int j = (blockIdx.x / tiles_x) * kScanTileY + (lane >> 2);
+    const int k = (blockIdx.x % tiles_x) * 32 + w * 4 + (lane & 3);
+    const int j = (blockIdx.x / tiles_x) * 8 + (lane >> 2);
     if (k >= S || j >= n) return;
     const int64_t nq = (int64_t)n * S, q = (int64_t)j * S + k;
     const uint32_t e0 = rowptr[q], e1 = rowptr[q + 1];
-    // one group of kScanImgs images per block row
+    // one group of kScanImgs images per block row, what is left over in pairs
     int c = blockIdx.y * kScanImgs;
     const float *g = gout + (int64_t)c * npix;
     float *o = gimg + (int64_t)c * nq + q;
@@ -217,6 +229,68 @@ __global__ void __launch_bounds__(kScanTileX *kScanTileY)
     c = 0;
     for (; c + 2 <= m; c += 2) scan_bwd_pass<2>(g + (int64_t)c * npix, ent, e0, e1, npix, nq, o + (int64_t)c * nq);
     if (c < m) scan_bwd_pass<1>(g + (int64_t)c * npix, ent, e0, e1, npix, nq, o + (int64_t)c * nq);
+}
+
+// The same pass with no more than two entries' loads in flight, which lets every
+// group size keep a pass of its own in one kernel's registers.
+template <int N>
+__device__ __forceinline__ void scan_bwd_rolled(const float *__restrict__ g, const ScanEnt *__restrict__ ent, uint32_t e0,
+                                                uint32_t e1, int64_t npix, int64_t nq, float *__restrict__ out)
+{
+    float s[N];
+#pragma unroll
+    for (int u = 0; u < N; u++) s[u] = 0.0f;
+#pragma unroll 1
+    for (uint32_t e = e0; e + 2 <= e1; e += 2) {
+        const ScanEnt x = ent[e], y = ent[e + 1];
+        float gx[N], gy[N];
+#pragma unroll
+        for (int u = 0; u < N; u++) {
+            gx[u] = __ldg(g + (int64_t)u * npix + x.pixel);
+            gy[u] = __ldg(g + (int64_t)u * npix + y.pixel);
+        }
+#pragma unroll
+        for (int u = 0; u < N; u++) s[u] = fmaf(y.w, gy[u], fmaf(x.w, gx[u], s[u]));
+    }
+    if ((e1 - e0) & 1) {
+        const ScanEnt x = ent[e1 - 1];
+#pragma unroll
+        for (int u = 0; u < N; u++) s[u] = fmaf(x.w, __ldg(g + (int64_t)u * npix + x.pixel), s[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < N; u++) out[(int64_t)u * nq] = s[u];
+}
+
+// Calls of fewer than two full groups: one pass over the list whatever the
+// group's size, where the pairs above read it up to four times.  64 rays x 256
+// rows and a 1024 x 1024 display: three images 88.8 us in pairs, 67.6; seven 184
+// and 131 us; three of 256 x 1024 22.6 and 17.8 us.  With two full groups and
+// more the pairs are a small part, and the kernel above, whose loop over a full
+// group the compiler schedules with fewer loads in flight, keeps more of a small
+// display in L1 (30 images of 64 x 256: 387 us, 475 with one pass per group).
+__global__ void __launch_bounds__(kScanTile, 6)
+    k_scan_bwd_few(const float *__restrict__ gout, const uint32_t *__restrict__ rowptr, const ScanEnt *__restrict__ ent,
+                   int n, int S, int tiles_x, int64_t npix, int count, float *__restrict__ gimg)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int k = (blockIdx.x % tiles_x) * 32 + w * 4 + (lane & 3);
+    const int j = (blockIdx.x / tiles_x) * 8 + (lane >> 2);
+    if (k >= S || j >= n) return;
+    const int64_t nq = (int64_t)n * S, q = (int64_t)j * S + k;
+    const uint32_t e0 = rowptr[q], e1 = rowptr[q + 1];
+    const int c = blockIdx.y * kScanImgs;
+    const float *g = gout + (int64_t)c * npix;
+    float *o = gimg + (int64_t)c * nq + q;
+    switch (min(kScanImgs, count - c)) {
+    case 1: scan_bwd_pass<1>(g, ent, e0, e1, npix, nq, o); break;
+    case 2: scan_bwd_pass<2>(g, ent, e0, e1, npix, nq, o); break;
+    case 3: scan_bwd_rolled<3>(g, ent, e0, e1, npix, nq, o); break;
+    case 4: scan_bwd_rolled<4>(g, ent, e0, e1, npix, nq, o); break;
+    case 5: scan_bwd_rolled<5>(g, ent, e0, e1, npix, nq, o); break;
+    case 6: scan_bwd_rolled<6>(g, ent, e0, e1, npix, nq, o); break;
+    case 7: scan_bwd_rolled<7>(g, ent, e0, e1, npix, nq, o); break;
+    default: scan_bwd_rolled<kScanImgs>(g, ent, e0, e1, npix, nq, o); break;
+    }
 }
 
 int check_scan_plan(const void *plan_host, const void *plan_dev)
@@ -302,9 +376,24 @@ extern "C" int diffus_scan_convert(const float *images, int32_t count, const voi
     if (count < 1 || count > 65535) return DIFFUS_E_PARAM;
     if (((uintptr_t)images) % 4 || ((uintptr_t)out) % 4) return DIFFUS_E_ALIGN;
     const ScanHeader &h = *(const ScanHeader *)plan_host;
-    const int tx = (h.W + kScanTileX - 1) / kScanTileX, ty = (h.H + kScanTileY - 1) / kScanTileY;
-    k_scan_fwd<<<(unsigned)((int64_t)tx * ty), kScanTileX * kScanTileY, 0, (cudaStream_t)stream>>>(
-        images, at<ScanTap>(plan_dev, h.off_map), h.S, (int64_t)h.n * h.S, h.W, h.H, tx, count, out);
+    int cols = 2;                          // fewer warp columns for a display narrower than four
+    while (cols > 0 && (4 << cols) >= h.W) cols--;
+    const int tx = (h.W + (8 << cols) - 1) / (8 << cols), ty = (h.H + (32 >> cols) - 1) / (32 >> cols);
+    // a display of fewer than four tiles per SM takes its images in groups side
+    // by side (64 images of 64 x 256 to 256 x 256: 16.7 us in turn, 10.2; at 512 x
+    // 512, seven tiles per SM, eight images take 5.5 us in turn, 6.1 in two groups)
+    int group = count;
+    while (group >= 8 && (int64_t)tx * ty * ((count + group - 1) / group) < 608) group = (group + 1) / 2;
+    // up to three images never fill a step of four
+    const bool few = count <= 3;
+    auto kernel = few ? k_scan_fwd<2, 8, false> : group < count ? k_scan_fwd<4, 5, true> : k_scan_fwd<4, 5, false>;
+    const int gx = few ? ty : tx, gy = few ? tx : ty;
+    for (int t0 = 0; t0 < gy; t0 += 65535) {   // the grid's y axis has 65535 places
+        const dim3 grid((unsigned)gx, (unsigned)(gy - t0 < 65535 ? gy - t0 : 65535), (unsigned)((count + group - 1) / group));
+        kernel<<<grid, kScanTile, 0, (cudaStream_t)stream>>>(images, at<ScanTap>(plan_dev, h.off_map), h.S,
+                                                             (int64_t)h.n * h.S, h.W, h.H, (int64_t)h.W * h.H, cols, t0,
+                                                             count, group, out);
+    }
     return launch_status();
 }
 
@@ -318,10 +407,12 @@ extern "C" int diffus_scan_convert_bwd(const float *grad_out, int32_t count, con
     if (count < 1 || count > 65535) return DIFFUS_E_PARAM;
     if (((uintptr_t)grad_out) % 4 || ((uintptr_t)grad_images) % 4) return DIFFUS_E_ALIGN;
     const ScanHeader &h = *(const ScanHeader *)plan_host;
-    const int tx = (h.S + kScanTileX - 1) / kScanTileX, ty = (h.n + kScanTileY - 1) / kScanTileY;
+    const int tx = (h.S + 31) / 32, ty = (h.n + 7) / 8;
     const dim3 bgrid((unsigned)((int64_t)tx * ty), (unsigned)((count + kScanImgs - 1) / kScanImgs));
-    k_scan_bwd<<<bgrid, kScanTileX * kScanTileY, 0, (cudaStream_t)stream>>>(
-        grad_out, at<uint32_t>(plan_dev, h.off_rowptr), at<ScanEnt>(plan_dev, h.off_ent), h.n, h.S, tx,
-        (int64_t)h.W * h.H, count, grad_images);
+    const bool few = count < 2 * kScanImgs && count != kScanImgs;   // see k_scan_bwd_few
+    auto kernel = few ? k_scan_bwd_few : k_scan_bwd;
+    kernel<<<bgrid, kScanTile, 0, (cudaStream_t)stream>>>(grad_out, at<uint32_t>(plan_dev, h.off_rowptr),
+                                                          at<ScanEnt>(plan_dev, h.off_ent), h.n, h.S, tx,
+                                                          (int64_t)h.W * h.H, count, grad_images);
     return launch_status();
 }
