@@ -12,6 +12,7 @@
 
 #include <cstring>
 #include <string>
+#include <vector>
 
 #include "diffus.h"
 
@@ -27,7 +28,7 @@ struct Call {
     diffus_fan fan;
     diffus_params prm;
 };
-static_assert(sizeof(Call) == 176, "render.py packs this layout");
+static_assert(sizeof(Call) == 176 && sizeof(Call) % sizeof(int64_t) == 0, "binding.py packs this layout");
 
 PyObject *g_error = nullptr;   // binding.DiffusError
 
@@ -79,10 +80,13 @@ struct RenderNode : public torch::autograd::Function<RenderNode> {
                                 valid.data_ptr<int>(), nullptr, ws.data_ptr(), (size_t)ws.numel(), stream()),
               "diffus_render_fwd");
         ctx->save_for_backward({vol, p});
-        ctx->saved_data["call"] = blob;
+        // as integers: compiled autograd reads what a node keeps and takes a
+        // string only as UTF-8
+        std::vector<int64_t> words(sizeof c / sizeof(int64_t));
+        std::memcpy(words.data(), &c, sizeof c);
+        ctx->saved_data["call"] = words;
         ctx->saved_data["want"] = (int64_t)volume.requires_grad() + 2 * (int64_t)pose.requires_grad();
-        ctx->mark_non_differentiable({valid});
-        return {img, valid};
+        return {img, valid};   // an integer output is not differentiable, and compiled autograd takes no such marks
     }
 
     static variable_list backward(AutogradContext *ctx, variable_list grads)
@@ -92,7 +96,8 @@ struct RenderNode : public torch::autograd::Function<RenderNode> {
         const auto saved = ctx->get_saved_variables();
         const Tensor &vol = saved[0], &p = saved[1];
         Call c;
-        std::memcpy(&c, ctx->saved_data["call"].toStringRef().data(), sizeof c);
+        const std::vector<int64_t> words = ctx->saved_data["call"].toIntVector();
+        std::memcpy(&c, words.data(), sizeof c);
         const diffus_volume_desc vd = desc(vol, c);
         const Tensor g = grads[0].detach().contiguous().to(at::kFloat);
         Tensor gv, gp;
