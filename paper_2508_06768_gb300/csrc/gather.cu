@@ -517,8 +517,9 @@ __global__ void k_unit_order(const uint32_t *__restrict__ uclass, const uint32_t
         order[atomicAdd(cursor + uclass[u], 1u)] = u;
 }
 
-// Resident blocks per SM of the unit kernel: 6 at 80 registers.  Measured on
-// the 512-pose batch: 5 (96 registers) 1056 us, 6 986, 7 (72, spilling) 1270.
+// Resident blocks per SM of the unit kernel: 6 at 80 registers, where the form
+// with pose terms keeps 12 bytes on the stack.  Measured on the 512-pose batch:
+// 5 (96 registers) 1056 us, 6 986, 7 (72 registers, spills in the cell loop) 1270.
 constexpr int kGatherCtas = 6;
 
 // One warp per unit, units handed out by a ticket queue: the warp gathers

@@ -45,13 +45,14 @@ constexpr int kGatherWarps = 4;
 // Runs per unit.  A warp walks a unit's runs 32 at a time, so a unit of n
 // runs is n/32 run walks in series (about 20 us each); more units cost more
 // partials (729 floats each).  Large problems fill the GPU with units of 256;
-// below, units shrink to one run per lane, for as long as the slots (about
-// four per run) make no more units than twice the resident warps (152 x 28).
-// Measured with 256 and with 32: a 251-ray frame's unit kernel 182 and 43 us,
-// nine small frames' 132 and 45 us; 512 frames stay at 256.
+// below, units shrink to one run per lane.  The cut-offs are plain ones: with
+// about four slots per run each allows some 8000 units, a little more than two
+// per resident warp (152 SMs x 24).  Measured with 256 and with 32: a 251-ray
+// frame's unit kernel 182 and 43 us, nine small frames' 132 and 45 us; 512 frames
+// stay at 256.
 __host__ __device__ inline int unit_runs(size_t slots)
 {
-        return slots <= (1u << 20) ? 32 : slots <= (1u << 21) ? 64 : slots <= (1u << 22) ? 128 : 256;
+    return slots <= (1u << 20) ? 32 : slots <= (1u << 21) ? 64 : slots <= (1u << 22) ? 128 : 256;
 }
 
 struct GatherArgs {

@@ -450,48 +450,48 @@ __device__ __forceinline__ void chunk_rows(const MarchArgs &A, const RayGeo &rg,
 {
     const int S = rg.S;
     const float a2 = A.a2;
-        float m[kChunk];
-        if (out.min) {
-            load_chunk(out.min + i0, i0 < S, m);
-        } else if (SPK_INLINE && A.sp.on) {
-            chunk_speckle(A.sp, i0, S, rg.ray, A.sp.pose_ctr + (uint32_t)rg.pose, m);
-        } else {
+    float m[kChunk];
+    if (out.min) {
+        load_chunk(out.min + i0, i0 < S, m);
+    } else if (SPK_INLINE && A.sp.on) {
+        chunk_speckle(A.sp, i0, S, rg.ray, A.sp.pose_ctr + (uint32_t)rg.pose, m);
+    } else {
 #pragma unroll
-            for (int t = 0; t < kChunk; t++) m[t] = 1.0f;
-        }
-        float y[kChunk];
-        const float cb0 = b0, cb1 = b1;          // state at the chunk start
-        float minq = 3.402823466e38f, fin = 0.0f;
+        for (int t = 0; t < kChunk; t++) m[t] = 1.0f;
+    }
+    float y[kChunk];
+    const float cb0 = b0, cb1 = b1;          // state at the chunk start
+    float minq = 3.402823466e38f, fin = 0.0f;
+#pragma unroll
+    for (int t = 0; t < kChunk; t++) {
+        const Xfer x = xfer_t<MODE>(rr[t], a2);
+        const float q = fmaf(b0, x.m01, b1);          // det(A_{i+1})
+        const float e = x.m01 * D * frcp(b1 * q);
+        if (TRACK && i0 + t < S && fminf(b1, q) < need_md) f.last_need = i0 + t;
+        minq = fminf(minq, q);
+        const float nb0 = fmaf(b0, x.m00, b1 * x.m10);
+        b1 = q;
+        b0 = nb0;
+        D *= x.delta;
+        y[t] = m[t] * e;
+        fin = fmaf(y[t], 0.0f, fin);
+    }
+    const bool odd = !(fin == 0.0f);          // a row that is not finite (NaN states among them)
+    if (odd || (!pole_seen && minq < kPoleEps)) {
+        float c0 = cb0, c1 = cb1;
 #pragma unroll
         for (int t = 0; t < kChunk; t++) {
             const Xfer x = xfer_t<MODE>(rr[t], a2);
-            const float q = fmaf(b0, x.m01, b1);          // det(A_{i+1})
-            const float e = x.m01 * D * frcp(b1 * q);
-            if (TRACK && i0 + t < S && fminf(b1, q) < need_md) f.last_need = i0 + t;
-            minq = fminf(minq, q);
-            const float nb0 = fmaf(b0, x.m00, b1 * x.m10);
-            b1 = q;
-            b0 = nb0;
-            D *= x.delta;
-            y[t] = m[t] * e;
-            fin = fmaf(y[t], 0.0f, fin);
-        }
-        const bool odd = !(fin == 0.0f);          // a row that is not finite (NaN states among them)
-        if (odd || (!pole_seen && minq < kPoleEps)) {
-            float c0 = cb0, c1 = cb1;
-#pragma unroll
-            for (int t = 0; t < kChunk; t++) {
-                const Xfer x = xfer_t<MODE>(rr[t], a2);
-                const float q = fmaf(c0, x.m01, c1);
-                if (i0 + t < S) {
-                    if (!(q >= kPoleEps)) f.first_bad = min(f.first_bad, i0 + t + 1);
-                    f.nonfinite += !isfinite(y[t]);
-                }
-                c0 = fmaf(c0, x.m00, c1 * x.m10);
-                c1 = q;
+            const float q = fmaf(c0, x.m01, c1);
+            if (i0 + t < S) {
+                if (!(q >= kPoleEps)) f.first_bad = min(f.first_bad, i0 + t + 1);
+                f.nonfinite += !isfinite(y[t]);
             }
+            c0 = fmaf(c0, x.m00, c1 * x.m10);
+            c1 = q;
         }
-        if (i0 < S) store_rows<STREAM>(out, i0, S, y);
+    }
+    if (i0 < S) store_rows<STREAM>(out, i0, S, y);
 }
 
 // The ray's counts after its last segment (called by one warp; f holds each

@@ -303,146 +303,146 @@ __device__ void march_bwd_ray(const T *__restrict__ vol, const MarchArgs &A, con
             }
         }
         for (int turn = 0; turn < nw; turn++) {
-        if (MULTI) {
-            __syncthreads();
-            if (turn != w || !on) continue;
-            lam0 = mm->lam0;
-            lam1 = mm->lam1;
-            mus = mm->mu;
-            carry_gz1 = mm->carry;
-        }
-        // adjoint at this lane's chunk end = G_{lane+1}(lambda_seg)
-        float le0, le1, lmu;
-        {
-            Mat2 Po = {__shfl_down_sync(0xffffffffu, Pm.a, 1), __shfl_down_sync(0xffffffffu, Pm.b, 1),
-                       __shfl_down_sync(0xffffffffu, Pm.c, 1), __shfl_down_sync(0xffffffffu, Pm.d, 1)};
-            float o0 = __shfl_down_sync(0xffffffffu, pc0, 1);
-            float o1 = __shfl_down_sync(0xffffffffu, pc1, 1);
-            float oal = __shfl_down_sync(0xffffffffu, pal, 1);
-            float od = __shfl_down_sync(0xffffffffu, pd, 1);
-            if (lane == kWarp - 1) {
-                le0 = lam0; le1 = lam1; lmu = mus;
-            } else {
-                le0 = o0 + fmaf(lam0, Po.a, lam1 * Po.b);
-                le1 = o1 + fmaf(lam0, Po.c, lam1 * Po.d);
-                lmu = fmaf(mus, oal, od);
+            if (MULTI) {
+                __syncthreads();
+                if (turn != w || !on) continue;
+                lam0 = mm->lam0;
+                lam1 = mm->lam1;
+                mus = mm->mu;
+                carry_gz1 = mm->carry;
             }
-        }
-
-        // E': true reverse pass: parameter adjoints -> dL/dr -> dL/dZ.
-        // dL/dZ of sample i0+t+1 (t < 7) is complete once interfaces t and
-        // t+1 are done, so it is finalised inside the loop; sample i0+8 also
-        // needs the next lane's interface and is finalised after it.
-        float a[6] = {0, 0, 0, 0, 0, 0};
-        float c_next = 0.0f;     // Z1-role contribution of interface t+1 to sample i0+t+1
-        float n_last = 0.0f;     // Z2-role contribution of interface i0+7 to sample i0+8
-        float c_first = 0.0f;    // Z1-role contribution of interface i0 to sample i0
-        float G[kChunk];         // dL/dZ of samples i0+1 .. i0+8
-        auto add_pose = [&](int k, int o, float g) {
-            if (!POSE) return;
-            const float gx = sm.gx[o], gyv = sm.gy[o], gzv = sm.gz[o];
-            const float sk = ((float)k + 0.5f) * ds;
-            a[0] = fmaf(g, gx, a[0]);
-            a[1] = fmaf(g, gyv, a[1]);
-            a[2] = fmaf(g, gzv, a[2]);
-            a[3] = fmaf(g * sk, gx, a[3]);
-            a[4] = fmaf(g * sk, gyv, a[4]);
-            a[5] = fmaf(g * sk, gzv, a[5]);
-        };
-        if (STORED) {
-            const float zl = __shfl_up_sync(0xffffffffu, zz[kChunk - 1], 1);
-            if (lane) z_first = zl;
-        }
-#pragma unroll
-        for (int t = kChunk - 1; t >= 0; t--) {
-            const float r = rr[t];
-            const Xfer x = xfer_t<MODE>(r, a2);
-            float gm00 = b0s[t] * le0, gm10 = b1s[t] * le0, gm01 = b0s[t] * le1;
-            float gdel = lmu * Dsv[t];
-            const float4 gv = sm.eg[t * kWarp + lane];   // written by this lane in C'
-            const EchoGrad g{gv.x, gv.y, gv.z, gv.w};
-            float gr;
-            if (MODE == DIFFUS_MODE_LITERAL) {
-                float R = fabsf(r);
-                float gR = gm00 * (-4.0f * a2 * R) + (gm01 + g.gx) * a2 - gm10 + gdel * (-2.0f * a2 * R);
-                gr = r > 0.0f ? gR : (r < 0.0f ? -gR : 0.0f);
-            } else {
-                gr = (gm01 + g.gx) * a2 + gm10 + gdel * (-2.0f * a2 * r);
-            }
-            float n0 = g.gb0 + fmaf(le0, x.m00, le1 * x.m01);
-            float n1 = g.gb1 + fmaf(le0, x.m10, le1);
-            lmu = fmaf(lmu, x.delta, g.gD);
-            le0 = n0;
-            le1 = n1;
-            float z1, z2;
-            if (STORED) {
-                z1 = t == 0 ? z_first : zz[t == 0 ? 0 : t - 1];
-                z2 = zz[t];
-            } else {
-                const int o1 = smem_idx(lane * kChunk + t), o2 = smem_idx(lane * kChunk + t + 1);
-                z1 = sm.zr[o1] + sm.dz[o1];
-                z2 = sm.zr[o2] + sm.dz[o2];
-            }
-            const float sz = z1 + z2;
-            const float is2 = frcp(sz * sz);
-            const float gzc = i0 + t < S ? gr * (-2.0f * z2) * is2 : 0.0f;
-            const float gzn = gr * (2.0f * z1) * is2;
-            if (t == kChunk - 1) {
-                n_last = gzn;
-            } else {
-                const int k = i0 + t + 1;
-                G[t] = c_next + gzn;
-                if (k <= S) add_pose(k, smem_idx(lane * kChunk + t + 1), G[t]);
-            }
-            c_next = gzc;
-            if (t == 0) c_first = gzc;
-        }
-        // adjoint at the segment start for the earlier segment
-        lam0 = __shfl_sync(0xffffffffu, le0, 0);
-        lam1 = __shfl_sync(0xffffffffu, le1, 0);
-        mus = __shfl_sync(0xffffffffu, lmu, 0);
-
-        // F': sample i0+8 (the next lane's first sample) and sample 0
-        {
-            float nextc = __shfl_down_sync(0xffffffffu, c_first, 1);
-            if (lane == kWarp - 1) nextc = carry_gz1;
-            const int k = i0 + kChunk;
-            G[kChunk - 1] = n_last + nextc;
-            if (k <= S) add_pose(k, smem_idx(lane * kChunk + kChunk), G[kChunk - 1]);
-            if (!POSE && i0 < S) {
-                // samples i0+1 .. i0+8 lie on one aligned sector (samples past
-                // S fall into the block's padding)
-                float4 *dst = reinterpret_cast<float4 *>(gz_row + i0 + 1);
-                const float4 lo = make_float4(G[0], G[1], G[2], G[3]), hi = make_float4(G[4], G[5], G[6], G[7]);
-                if (STORED) {
-                    __stcs(dst, lo);
-                    __stcs(dst + 1, hi);
+            // adjoint at this lane's chunk end = G_{lane+1}(lambda_seg)
+            float le0, le1, lmu;
+            {
+                Mat2 Po = {__shfl_down_sync(0xffffffffu, Pm.a, 1), __shfl_down_sync(0xffffffffu, Pm.b, 1),
+                           __shfl_down_sync(0xffffffffu, Pm.c, 1), __shfl_down_sync(0xffffffffu, Pm.d, 1)};
+                float o0 = __shfl_down_sync(0xffffffffu, pc0, 1);
+                float o1 = __shfl_down_sync(0xffffffffu, pc1, 1);
+                float oal = __shfl_down_sync(0xffffffffu, pal, 1);
+                float od = __shfl_down_sync(0xffffffffu, pd, 1);
+                if (lane == kWarp - 1) {
+                    le0 = lam0; le1 = lam1; lmu = mus;
                 } else {
-                    dst[0] = lo;
-                    dst[1] = hi;
+                    le0 = o0 + fmaf(lam0, Po.a, lam1 * Po.b);
+                    le1 = o1 + fmaf(lam0, Po.c, lam1 * Po.d);
+                    lmu = fmaf(mus, oal, od);
                 }
             }
-        }
-        if (s == 0 && lane == 0) {
-            if (!POSE) gz_row[0] = c_first;
-            add_pose(0, smem_idx(0), c_first);
-        }
-        carry_gz1 = __shfl_sync(0xffffffffu, c_first, 0);
-        if (POSE) {
-#pragma unroll
-            for (int q = 0; q < 6; q++) {
-                float v = a[q];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                if (lane == 0) acc[q] += (double)v;
+
+            // E': true reverse pass: parameter adjoints -> dL/dr -> dL/dZ.
+            // dL/dZ of sample i0+t+1 (t < 7) is complete once interfaces t and
+            // t+1 are done, so it is finalised inside the loop; sample i0+8 also
+            // needs the next lane's interface and is finalised after it.
+            float a[6] = {0, 0, 0, 0, 0, 0};
+            float c_next = 0.0f;     // Z1-role contribution of interface t+1 to sample i0+t+1
+            float n_last = 0.0f;     // Z2-role contribution of interface i0+7 to sample i0+8
+            float c_first = 0.0f;    // Z1-role contribution of interface i0 to sample i0
+            float G[kChunk];         // dL/dZ of samples i0+1 .. i0+8
+            auto add_pose = [&](int k, int o, float g) {
+                if (!POSE) return;
+                const float gx = sm.gx[o], gyv = sm.gy[o], gzv = sm.gz[o];
+                const float sk = ((float)k + 0.5f) * ds;
+                a[0] = fmaf(g, gx, a[0]);
+                a[1] = fmaf(g, gyv, a[1]);
+                a[2] = fmaf(g, gzv, a[2]);
+                a[3] = fmaf(g * sk, gx, a[3]);
+                a[4] = fmaf(g * sk, gyv, a[4]);
+                a[5] = fmaf(g * sk, gzv, a[5]);
+            };
+            if (STORED) {
+                const float zl = __shfl_up_sync(0xffffffffu, zz[kChunk - 1], 1);
+                if (lane) z_first = zl;
             }
-        }
-        if (MULTI && lane == 0) {
-            mm->lam0 = lam0;
-            mm->lam1 = lam1;
-            mm->mu = mus;
-            mm->carry = carry_gz1;
-        }
+#pragma unroll
+            for (int t = kChunk - 1; t >= 0; t--) {
+                const float r = rr[t];
+                const Xfer x = xfer_t<MODE>(r, a2);
+                float gm00 = b0s[t] * le0, gm10 = b1s[t] * le0, gm01 = b0s[t] * le1;
+                float gdel = lmu * Dsv[t];
+                const float4 gv = sm.eg[t * kWarp + lane];   // written by this lane in C'
+                const EchoGrad g{gv.x, gv.y, gv.z, gv.w};
+                float gr;
+                if (MODE == DIFFUS_MODE_LITERAL) {
+                    float R = fabsf(r);
+                    float gR = gm00 * (-4.0f * a2 * R) + (gm01 + g.gx) * a2 - gm10 + gdel * (-2.0f * a2 * R);
+                    gr = r > 0.0f ? gR : (r < 0.0f ? -gR : 0.0f);
+                } else {
+                    gr = (gm01 + g.gx) * a2 + gm10 + gdel * (-2.0f * a2 * r);
+                }
+                float n0 = g.gb0 + fmaf(le0, x.m00, le1 * x.m01);
+                float n1 = g.gb1 + fmaf(le0, x.m10, le1);
+                lmu = fmaf(lmu, x.delta, g.gD);
+                le0 = n0;
+                le1 = n1;
+                float z1, z2;
+                if (STORED) {
+                    z1 = t == 0 ? z_first : zz[t == 0 ? 0 : t - 1];
+                    z2 = zz[t];
+                } else {
+                    const int o1 = smem_idx(lane * kChunk + t), o2 = smem_idx(lane * kChunk + t + 1);
+                    z1 = sm.zr[o1] + sm.dz[o1];
+                    z2 = sm.zr[o2] + sm.dz[o2];
+                }
+                const float sz = z1 + z2;
+                const float is2 = frcp(sz * sz);
+                const float gzc = i0 + t < S ? gr * (-2.0f * z2) * is2 : 0.0f;
+                const float gzn = gr * (2.0f * z1) * is2;
+                if (t == kChunk - 1) {
+                    n_last = gzn;
+                } else {
+                    const int k = i0 + t + 1;
+                    G[t] = c_next + gzn;
+                    if (k <= S) add_pose(k, smem_idx(lane * kChunk + t + 1), G[t]);
+                }
+                c_next = gzc;
+                if (t == 0) c_first = gzc;
+            }
+            // adjoint at the segment start for the earlier segment
+            lam0 = __shfl_sync(0xffffffffu, le0, 0);
+            lam1 = __shfl_sync(0xffffffffu, le1, 0);
+            mus = __shfl_sync(0xffffffffu, lmu, 0);
+
+            // F': sample i0+8 (the next lane's first sample) and sample 0
+            {
+                float nextc = __shfl_down_sync(0xffffffffu, c_first, 1);
+                if (lane == kWarp - 1) nextc = carry_gz1;
+                const int k = i0 + kChunk;
+                G[kChunk - 1] = n_last + nextc;
+                if (k <= S) add_pose(k, smem_idx(lane * kChunk + kChunk), G[kChunk - 1]);
+                if (!POSE && i0 < S) {
+                    // samples i0+1 .. i0+8 lie on one aligned sector (samples past
+                    // S fall into the block's padding)
+                    float4 *dst = reinterpret_cast<float4 *>(gz_row + i0 + 1);
+                    const float4 lo = make_float4(G[0], G[1], G[2], G[3]), hi = make_float4(G[4], G[5], G[6], G[7]);
+                    if (STORED) {
+                        __stcs(dst, lo);
+                        __stcs(dst + 1, hi);
+                    } else {
+                        dst[0] = lo;
+                        dst[1] = hi;
+                    }
+                }
+            }
+            if (s == 0 && lane == 0) {
+                if (!POSE) gz_row[0] = c_first;
+                add_pose(0, smem_idx(0), c_first);
+            }
+            carry_gz1 = __shfl_sync(0xffffffffu, c_first, 0);
+            if (POSE) {
+#pragma unroll
+                for (int q = 0; q < 6; q++) {
+                    float v = a[q];
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                    if (lane == 0) acc[q] += (double)v;
+                }
+            }
+            if (MULTI && lane == 0) {
+                mm->lam0 = lam0;
+                mm->lam1 = lam1;
+                mm->mu = mus;
+                mm->carry = carry_gz1;
+            }
         }
         __syncwarp();
     }

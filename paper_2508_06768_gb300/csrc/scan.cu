@@ -117,7 +117,7 @@ ScanHeader scan_layout(const ScanGeom &g, int64_t n_ent)
 // them is the number of lines per load (L1 wavefronts), then the streams to
 // HBM; a few images of a small display are bound by one thread's chain.
 // 64 images of 256 x 1024 and a 1024 x 1024 display: forward 143 us with
-// 32 x 1 pixels per warp, 105 us (3.2 TB/s) with 8 x 4; adjoint 531 us with 1 ray
+// 32 x 1 pixels per warp, 105 us (3.4 TB/s) with 8 x 4; adjoint 531 us with 1 ray
 // x 32 rows and 4 images per pass over the lists, 335 us with 4 x 8 and 8 images,
 // 215 us with the image groups side by side instead of in turn, 198 us with 8
 // rays x 4 rows.
@@ -128,8 +128,8 @@ constexpr int kScanImgs = 8;                     // images per pass over the lis
 // images of the block's group (blockIdx.z, GROUPED; else all), U images' taps in
 // flight together.  A block is 2^cols warps wide and 8 / 2^cols high; tile0: the
 // grid's first tile along its y axis.  U and the resident blocks MINB trade loads
-// in flight against warps: one image of 256 x 1024 to 1024 x 1024 takes 5.1 us
-// with 4 and 5, 4.65 with 2 and 8; 64 images 105 us with 4 and 5.
+// in flight against warps: one image of 256 x 1024 to 1024 x 1024 takes 5.0 us
+// with 4 and 6, 4.65 with 2 and 8; 64 images 105 us with 4 and 5, 108 with 2 and 8.
 template <int U, int MINB, bool GROUPED>
 __global__ void __launch_bounds__(kScanTile, MINB)
     k_scan_fwd(const float *__restrict__ img, const ScanTap *__restrict__ map, int S, int64_t img_stride, int W, int H,
