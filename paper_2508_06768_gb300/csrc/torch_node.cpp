@@ -79,27 +79,30 @@ struct RenderNode : public torch::autograd::Function<RenderNode> {
         check(diffus_render_fwd(vol.data_ptr(), &vd, p.data_ptr<float>(), &c.fan, &c.prm, img.data_ptr<float>(),
                                 valid.data_ptr<int>(), nullptr, ws.data_ptr(), (size_t)ws.numel(), stream()),
               "diffus_render_fwd");
+        const int64_t want = (int64_t)volume.requires_grad() + 2 * (int64_t)pose.requires_grad();
+        if (want == 0) return {img, valid};
+        ctx->set_materialize_grads(false);   // valid has none: no zeros are made for it
         ctx->save_for_backward({vol, p});
         // as integers: compiled autograd reads what a node keeps and takes a
         // string only as UTF-8
         std::vector<int64_t> words(sizeof c / sizeof(int64_t));
         std::memcpy(words.data(), &c, sizeof c);
-        ctx->saved_data["call"] = words;
-        ctx->saved_data["want"] = (int64_t)volume.requires_grad() + 2 * (int64_t)pose.requires_grad();
+        ctx->saved_data["call"] = std::move(words);
+        ctx->saved_data["want"] = want;
         return {img, valid};   // an integer output is not differentiable, and compiled autograd takes no such marks
     }
 
     static variable_list backward(AutogradContext *ctx, variable_list grads)
     {
         const int64_t want = ctx->saved_data["want"].toInt();
-        if (!grads[0].defined() || want == 0) return {Tensor(), Tensor(), Tensor()};
         const auto saved = ctx->get_saved_variables();
         const Tensor &vol = saved[0], &p = saved[1];
         Call c;
         const std::vector<int64_t> words = ctx->saved_data["call"].toIntVector();
         std::memcpy(&c, words.data(), sizeof c);
         const diffus_volume_desc vd = desc(vol, c);
-        const Tensor g = grads[0].detach().contiguous().to(at::kFloat);
+        const Tensor g = grads[0].defined() ? grads[0].detach().contiguous().to(at::kFloat)
+                                            : at::zeros({c.fan.n_rays, c.fan.n_samples}, vol.options().dtype(at::kFloat));
         Tensor gv, gp;
         if (want & 1) gv = at::empty(vol.sizes(), vol.options().dtype(at::kFloat));
         if (want & 2) gp = at::empty({6}, vol.options().dtype(at::kFloat));

@@ -67,9 +67,10 @@ def render(volume: torch.Tensor, pose: torch.Tensor, fan, params, spacing=(1.0, 
            origin=(0.0, 0.0, 0.0), pose_ctr: int = 0):
     """Render one pose: returns (image [n_rays][S] float32, ray_valid int32)."""
     call = _native_call(volume, pose, fan, params, spacing, origin, pose_ctr)
-    node = B.load_node() if call is not None else None
-    if node is not None:
-        return node.render(volume, pose, call)
+    if call is not None:
+        node = B.load_node()
+        if node is not None:
+            return node.render(volume, pose, call)
     return _Render.apply(volume, pose, tuple(spacing), tuple(origin), fan, params, int(pose_ctr))
 
 
