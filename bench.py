@@ -141,7 +141,7 @@ BOUND = {"march_fwd": "alu", "march_bwd": "alu", "gather_units": "alu", "blur": 
 # dram__bytes_write.sum of one launch over the first 192 poses of the
 # workload, the forward phase being the speckle kernel plus the march,
 # divided by its ray-samples); absent where the kernel changed since.
-NCU_DRAM_PER_UNIT = {"blur": 7.98, "blur_T": 7.93, "gather_units": 8.61}
+NCU_DRAM_PER_UNIT = {"blur": 7.36, "blur_T": 7.42, "gather_units": 8.56}
 # the marches' figures depend on the forward form (fwd_form 0: one warp per
 # ray; 1: one lane per ray), set from the capture of that form
 NCU_DRAM_PER_UNIT_FORM = {0: {"march_fwd": 18.87, "march_bwd": 19.75}, 1: {}}

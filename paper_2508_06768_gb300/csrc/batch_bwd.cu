@@ -10,8 +10,8 @@ namespace {
 
 // POSE: the pose-only call, which samples Z and dZ/dp itself; otherwise the
 // march reads the rows that the forward of the same call kept (STORED) and
-// never touches the volume, whatever its type.  STORED is bound by issue (74 %)
-// and L1 wavefronts (66 %): 512 uneven frames 1535 us with the kept pairs
+// never touches the volume, whatever its type.  STORED is bound by issue (77 %)
+// and L1 wavefronts (64 to 68 %): 512 uneven frames 1535 us with the kept pairs
 // transposed through shared memory and scalar rows, 942 us with each lane
 // loading its chunks of the kept rows (249 and 155 warp instructions per 32
 // samples).

@@ -8,9 +8,9 @@ namespace {
 
 // Persistent forward: each warp takes rays from the queue (longest first).
 // TRACK (refinement on, sel.rinfo set): it is the FP32 pass, which lists the
-// rays that need the refined pass.  Bound by L1 wavefronts (88 % of peak, two
-// thirds of them the eight corner loads, 4.4 lines each) with the issue slots
-// at 74 %.  512 uneven frames with everything kept for the adjoint: 1433 us
+// rays that need the refined pass.  Bound by L1 wavefronts (90 to 92 % of peak,
+// two thirds of them the eight corner loads, 4.4 lines each) with the issue slots
+// at 76 to 78 %.  512 uneven frames with everything kept for the adjoint: 1433 us
 // with packed rows, per-row tests and per-sample neighbour exchange, 1097 us
 // as it stands (225 and 181 warp instructions per 32 samples).
 template <typename T, int WARPS, int MODE, bool TRACK>

@@ -36,3 +36,27 @@ def test_backward_under_compiled_autograd():
                 I.Fan(20, 99, math.radians(55), 33.0, 5.0, 0.5)):
         for a, b in zip(grads(fan, False), grads(fan, True)):
             assert torch.equal(a, b)
+
+
+def test_image_without_a_gradient():
+    # a function downstream that passes no gradient on: zeros, as from the Python function
+    import torch
+    from paper_2508_06768_gb300 import render as R
+
+    class Stop(torch.autograd.Function):
+        @staticmethod
+        def forward(ctx, x):
+            return x.sum()
+
+        @staticmethod
+        def backward(ctx, g):
+            return None
+
+    vol, prm = I.small_phantom(n=40, seed=9), I.Params(seed=3, mode=1)
+    fan = I.Fan(33, 150, math.radians(55), 33.0, 5.0, 0.5)
+    for f in (lambda v, p: R.render(v, p, fan, prm),
+              lambda v, p: R._Render.apply(v, p, (1.0,) * 3, (0.0,) * 3, fan, prm, 0)):
+        v = torch.from_numpy(vol.data).cuda().requires_grad_()
+        p = torch.from_numpy(I.top_face_pose(vol)).cuda().requires_grad_()
+        gv, gp = torch.autograd.grad(Stop.apply(f(v, p)[0]), (v, p))
+        assert not gv.any() and not gp.any() and gv.shape == v.shape and gp.shape == (6,)
