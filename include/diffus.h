@@ -314,7 +314,11 @@ int diffus_batch_plan_chunks(const void *plan_host, int32_t *first_pose, int32_t
  * nullable); grad_poses (device float [P][6], overwritten, nullable);
  * ray_valid (device int32, one per ray in pose order, nullable).  The plan
  * must come from diffus_batch_plan with the same blur parameters
- * (DIFFUS_E_PLAN otherwise).  With a backward, the forward keeps in the
+ * (DIFFUS_E_PLAN otherwise), and its longest fan must span at most 2^29
+ * voxels at vd's spacing (DIFFUS_E_PARAM).  A pose that is not finite is
+ * rendered as a probe far outside the volume and has a NaN rotation
+ * gradient when an angle is not finite; the other poses are unaffected.
+ * With a backward, the forward keeps in the
  * workspace what the adjoint of the same call needs (scan carries, speckle
  * factors and, unless only grad_poses is asked, every sample's impedance
  * and coefficient), so the adjoint does not resample the volume.  Only
